@@ -1070,7 +1070,9 @@ int enumerate_run(Ctx *c, Run *R, uint64_t limit, int32_t *h_out, uint64_t *n_ou
   }
   const int D = std::max(1, joins_below[N - 1]);
   const int RW = 3 + D + nF;
-  // pre-order of the nice decomposition from the root
+  // pre-order of the nice decomposition from the root, and the steps that multiply states
+  // (forgets and joins), each with the introduces and leaves since the step before it; those
+  // after the last one no longer change a row
   std::vector<int> pre, stack{N - 1};
   while (!stack.empty()) {
     int x = stack.back();
@@ -1078,6 +1080,19 @@ int enumerate_run(Ctx *c, Run *R, uint64_t limit, int32_t *h_out, uint64_t *n_ou
     pre.push_back(x);
     if (P.nodes[x].child1 >= 0) stack.push_back(P.nodes[x].child1);
     if (P.nodes[x].child0 >= 0) stack.push_back(P.nodes[x].child0);
+  }
+  struct Step {
+    int x, u0, u1;
+  };
+  std::vector<Step> steps;
+  for (int i = 0, u0 = 0; i < N; ++i)
+    if (P.nodes[pre[i]].type >= 2) {
+      steps.push_back({pre[i], u0, i});
+      u0 = i + 1;
+    }
+  if (R->sizes[N - 1] == 0) {  // empty root table: no embedding in any trial
+    *n_out = *n_total = 0;
+    return CC_OK;
   }
   std::vector<void *> owned;
   auto cleanup = [&]() {
@@ -1097,81 +1112,188 @@ int enumerate_run(Ctx *c, Run *R, uint64_t limit, int32_t *h_out, uint64_t *n_ou
       }
     c->arena.release(p);
   };
+  struct Cleanup {
+    decltype(cleanup) &f;
+    ~Cleanup() { f(); }
+  } cleanup_guard{cleanup};
   cc::EnumNode *d_nodes = (cc::EnumNode *)take(sizeof(cc::EnumNode) * N);
-  u64 *scratch = (u64 *)take(sizeof(u64) * (cc::scan_scratch_words(c->dev) + 8));
-  if (!d_nodes || !scratch) {
-    cleanup();
-    return CC_ENOMEM;
-  }
-  if (cudaMemcpyAsync(d_nodes, en.data(), sizeof(cc::EnumNode) * N, cudaMemcpyHostToDevice,
-                      c->stream) != cudaSuccess) {
-    cleanup();
-    return CC_ECUDA;
-  }
+  int *d_pre = (int *)take(sizeof(int) * N);
+  // per step the states it made (word 0: the root states), the distinct rows, an error word
+  const size_t S = steps.size();
+  u64 *d_made = (u64 *)take(sizeof(u64) * (S + 3));
+  if (!d_nodes || !d_pre || !d_made) return CC_ENOMEM;
+  u64 *d_distinct = d_made + S + 1;
+  int *d_err = (int *)(d_made + S + 2);
+  CUDA_OK(cudaMemcpyAsync(d_nodes, en.data(), sizeof(cc::EnumNode) * N, cudaMemcpyHostToDevice,
+                          c->stream));
+  CUDA_OK(cudaMemcpyAsync(d_pre, pre.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->stream));
+  std::vector<u64> per_trial(R->trials), made(S + 3);
+  CUDA_OK(cudaMemcpyAsync(per_trial.data(), R->d_count, R->trials * sizeof(u64),
+                          cudaMemcpyDeviceToHost, c->stream));
+  CUDA_OK(cudaMemsetAsync(d_made, 0, sizeof(u64) * (S + 3), c->stream));
+  CUDA_OK(cudaStreamSynchronize(c->stream));
   cc::EnumArgs a{};
   a.G = cc::GraphDev{c->d_row_ptr, c->d_col, col.d_colors, c->n, c->d_deg8,
                      c->patterns.at(R->pattern).d_allow};
   a.L = R->L;
   a.nodes = d_nodes;
+  a.pre = d_pre;
   a.nF = nF;
   a.R = RW;
   a.D = D;
-  // root states
-  u64 n_cur = R->sizes[N - 1];
-  int *cur = (int *)take(std::max<u64>(1, n_cur) * RW * sizeof(int));
-  if (!cur) {
-    cleanup();
-    return CC_ENOMEM;
-  }
-  a.out = cur;
-  a.n_in = n_cur;
-  u64 *d_n = scratch + cc::scan_scratch_words(c->dev);
-  int rc = CC_OK;
-  if (cudaMemsetAsync(d_n, 0, sizeof(u64), c->stream) != cudaSuccess) rc = CC_ECUDA;
+  a.chunks = 1;
   const cc::NodeTable &rt = R->tables[N - 1];
   const u64 rbound = rt.hashed ? rt.cap : R->sizes[N - 1];
-  if (!rc && cc::launch_enum_init(c->stream, c->dev, R->kw, a, rt.slots, rbound, d_n)) rc = CC_ECUDA;
-  c->launches++;
-  for (size_t i = 0; i < pre.size() && !rc; ++i) {
-    a.x = pre[i];
-    a.in = cur;
-    a.n_in = n_cur;
-    unsigned *cnt = (unsigned *)take(std::max<u64>(1, n_cur) * sizeof(unsigned));
-    u64 *off = (u64 *)take((n_cur + 1) * sizeof(u64));
-    if (!cnt || !off) {
-      rc = CC_ENOMEM;
-      break;
+  const u64 lim_rows = limit;
+  auto read_made = [&]() -> int {
+    CUDA_OK(cudaMemcpyAsync(made.data(), d_made, sizeof(u64) * (S + 3), cudaMemcpyDeviceToHost,
+                            c->stream));
+    CUDA_OK(cudaStreamSynchronize(c->stream));
+    return (int)made[S + 2] & cc::kErrTimeout ? CC_ETIMEOUT : CC_OK;
+  };
+  // The union over trials of n final states (*d_n of them) in lexicographic order without
+  // repeats, as sortable records when a row fits one: its first `limit` rows into *out_buf and
+  // the number of distinct ones into *d_distinct, nothing read back.  `states` is given back.
+  // CC_ENOMEM (and `states` kept) when the rows are too wide or the room is short.
+  auto sort_as_records = [&](int *states, u64 n, const u64 *d_n, int **out_buf) -> int {
+    const int bits = nF * R->L.nb;
+    if (nF > cc::kMaxBag || bits > 127) return CC_ENOMEM;
+    const int kw = bits < 64 ? 1 : 2;
+    const size_t rb = cc::slot_bytes(kw);
+    const cc::SortSpec sp = cc::rows_spec(nF, R->L.nb);
+    cc::SweepScratch sw{};
+    sw.max_tiles = n / cc::sweep_tile(kw) + 2;
+    const u64 lim = std::min<u64>(lim_rows, n);
+    std::vector<void *> got;
+    auto want = [&](size_t bytes) {
+      got.push_back(take(bytes));
+      return got.back();
+    };
+    char *recs = (char *)want(n * rb), *ba = (char *)want(n * rb), *bb = (char *)want(n * rb);
+    sw.ghist = (u64 *)want(256 * 16 * sizeof(u64));
+    sw.tile_ctr = (unsigned *)want(16 * sizeof(unsigned));
+    sw.status = (u64 *)want(256 * sw.max_tiles * sizeof(u64));
+    u64 *blk = (u64 *)want((2 * (size_t)cc::sort_grid(c->dev) + 8) * sizeof(u64));
+    int *out = (int *)want(std::max<u64>(1, lim) * nF * sizeof(int));
+    sw.err = d_err;
+    for (void *p : got)
+      if (!p) {
+        for (void *q : got)
+          if (q) drop(q);
+        return CC_ENOMEM;
+      }
+    int which = 0;
+    if (cc::launch_rows_pack(c->stream, c->dev, kw, states, n, d_n, RW, D, nF, R->L.nb, sets,
+                             recs) ||
+        cc::launch_sort_records(c->stream, c->dev, kw, sp, recs, d_n, n, d_n, n, ba, bb, nullptr,
+                                &which, &sw) ||
+        cc::launch_reduce(c->stream, c->dev, kw, which ? bb : ba, d_n, n, blk, recs, d_distinct,
+                          nullptr) ||
+        cc::launch_rows_unpack(c->stream, c->dev, kw, recs, d_distinct, lim, nF, R->L.nb, out))
+      return CC_ECUDA;
+    c->launches += 7 + cc::sort_passes(sp);
+    drop(states);
+    *out_buf = out;
+    return CC_OK;
+  };
+  int *cur = nullptr, *out = nullptr;
+  u64 n_cur = 0;
+  // The states of a step never outnumber the embeddings, and those are counted: with two state
+  // arrays of that many the steps append one after the other without a read-back between them.
+  // (A count that wrapped past 2^64 shows as more states than room; so does nothing else.)
+  u64 E = 0;
+  for (u64 v : per_trial) E += v;
+  const size_t state_bytes = (size_t)RW * sizeof(int);
+  bool have = false;
+  if (E > 0 && E < (1ull << 40)) {
+    int *buf[2] = {(int *)take(E * state_bytes), (int *)take(E * state_bytes)};
+    if (buf[0] && buf[1]) {
+      a.n_in = E;
+      a.cap = E;
+      a.out = buf[0];
+      if (cc::launch_enum_init(c->stream, c->dev, R->kw, a, rt.slots, rbound, d_made))
+        return CC_ECUDA;
+      c->launches++;
+      for (size_t i = 0; i < S; ++i) {
+        a.x = steps[i].x;
+        a.u0 = steps[i].u0;
+        a.u1 = steps[i].u1;
+        a.in = buf[i & 1];
+        a.out = buf[(i & 1) ^ 1];
+        a.n_dev = d_made + i;
+        a.cursor = d_made + i + 1;
+        // a forget without a neighbour left tries every host vertex: up to 256 warps a state
+        a.chunks = en[a.x].type == 2 && en[a.x].nnb == 0 ? std::min(256, (c->n + 31) / 32) : 1;
+        if (cc::launch_enum_step(c->stream, c->dev, R->kw, 2, a)) return CC_ECUDA;
+        c->launches++;
+      }
+      cur = buf[S & 1];
+      n_cur = E;
+      drop(buf[(S & 1) ^ 1]);
+      int rc = sort_as_records(cur, n_cur, d_made + S, &out);
+      if (rc && rc != CC_ENOMEM) return rc;
+      rc = read_made();
+      if (rc) return rc;
+      have = made[S] == E;
+      for (size_t i = 0; i <= S; ++i) have = have && made[i] <= E;
+      if (!have) {
+        if (out) drop(out);
+        else drop(cur);
+        cur = out = nullptr;
+      }
+    } else {
+      for (int *p : buf)
+        if (p) drop(p);
     }
-    a.cnt = cnt;
-    if (cc::launch_enum_step(c->stream, c->dev, R->kw, 0, a) ||
-        cc::launch_scan_u32(c->stream, c->dev, cnt, n_cur, off, scratch)) {
-      rc = CC_ECUDA;
-      break;
-    }
-    c->launches += 4;
-    u64 n_next = 0;
-    rc = read_u64(c, off + n_cur, &n_next);
-    if (rc) break;
-    int *next = (int *)take(std::max<u64>(1, n_next) * RW * sizeof(int));
-    if (!next) {
-      rc = CC_ENOMEM;
-      break;
-    }
-    a.out = next;
-    a.off = off;
-    if (cc::launch_enum_step(c->stream, c->dev, R->kw, 1, a)) {
-      rc = CC_ECUDA;
-      break;
-    }
-    c->launches++;
-    drop(cnt);
-    drop(off);
-    drop(cur);
-    cur = next;
-    n_cur = n_next;
   }
-  // the union over trials in lexicographic order without repeats
-  if (!rc) {
+  u64 *scratch = nullptr;
+  if (!out) {
+    scratch = (u64 *)take(sizeof(u64) * (cc::scan_scratch_words(c->dev) + 8));
+    if (!scratch) return CC_ENOMEM;
+  }
+  if (!have) {  // each step counted first, with exact room for what it makes
+    a.n_dev = nullptr;
+    a.chunks = 1;
+    n_cur = R->sizes[N - 1];
+    cur = (int *)take(std::max<u64>(1, n_cur) * state_bytes);
+    if (!cur) return CC_ENOMEM;
+    a.out = cur;
+    a.n_in = n_cur;
+    CUDA_OK(cudaMemsetAsync(d_made, 0, sizeof(u64) * (S + 3), c->stream));
+    if (cc::launch_enum_init(c->stream, c->dev, R->kw, a, rt.slots, rbound, d_made))
+      return CC_ECUDA;
+    c->launches++;
+    for (const Step &st : steps) {
+      a.x = st.x;
+      a.u0 = st.u0;
+      a.u1 = st.u1;
+      a.in = cur;
+      a.n_in = n_cur;
+      unsigned *cnt = (unsigned *)take(std::max<u64>(1, n_cur) * sizeof(unsigned));
+      u64 *off = (u64 *)take((n_cur + 1) * sizeof(u64));
+      if (!cnt || !off) return CC_ENOMEM;
+      a.cnt = cnt;
+      if (cc::launch_enum_step(c->stream, c->dev, R->kw, 0, a) ||
+          cc::launch_scan_u32(c->stream, c->dev, cnt, n_cur, off, scratch))
+        return CC_ECUDA;
+      c->launches += 4;
+      u64 n_next = 0;
+      int rc = read_u64(c, off + n_cur, &n_next);
+      if (rc) return rc;
+      int *next = (int *)take(std::max<u64>(1, n_next) * state_bytes);
+      if (!next) return CC_ENOMEM;
+      a.out = next;
+      a.off = off;
+      if (cc::launch_enum_step(c->stream, c->dev, R->kw, 1, a)) return CC_ECUDA;
+      c->launches++;
+      drop(cnt);
+      drop(off);
+      drop(cur);
+      cur = next;
+      n_cur = n_next;
+    }
+  }
+  if (!out) {  // rows too wide for a record, or too little room: an index sort of the rows
     int *rows = (int *)take(std::max<u64>(1, n_cur) * nF * sizeof(int));
     unsigned *perm = (unsigned *)take(std::max<u64>(1, n_cur) * sizeof(unsigned));
     unsigned *tmp = (unsigned *)take(std::max<u64>(1, n_cur) * sizeof(unsigned));
@@ -1179,35 +1301,29 @@ int enumerate_run(Ctx *c, Run *R, uint64_t limit, int32_t *h_out, uint64_t *n_ou
     unsigned *flag = (unsigned *)take(std::max<u64>(1, n_cur) * sizeof(unsigned));
     u64 *off = (u64 *)take((n_cur + 1) * sizeof(u64));
     const u64 lim = std::min<u64>(limit, n_cur);
-    int *out = (int *)take(std::max<u64>(1, lim) * nF * sizeof(int));
-    if (!rows || !perm || !tmp || !hist || !flag || !off || !out) {
-      rc = CC_ENOMEM;
-    } else {
-      unsigned *sorted = nullptr;
-      if (cc::launch_rows_extract(c->stream, c->dev, cur, n_cur, RW, D, nF, rows, perm) ||
-          (sets && cc::launch_rows_canon(c->stream, c->dev, rows, nF, n_cur)) ||
-          cc::launch_rows_sort(c->stream, c->dev, rows, nF, R->L.nb, n_cur, perm, tmp, hist,
-                               &sorted) ||
-          cc::launch_rows_heads(c->stream, c->dev, rows, nF, sorted, n_cur, flag) ||
-          cc::launch_scan_u32(c->stream, c->dev, flag, n_cur, off, scratch) ||
-          cc::launch_rows_gather(c->stream, c->dev, rows, nF, sorted, n_cur, flag, off, lim, out))
-        rc = CC_ECUDA;
-      c->launches += 10;
-      u64 distinct = 0;
-      if (!rc) rc = read_u64(c, off + n_cur, &distinct);
-      if (!rc) {
-        const u64 m = std::min<u64>(limit, distinct);
-        if (m && cudaMemcpyAsync(h_out, out, m * nF * sizeof(int), cudaMemcpyDeviceToHost,
-                                 c->stream) != cudaSuccess)
-          rc = CC_ECUDA;
-        if (!rc && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = CC_ECUDA;
-        *n_out = m;
-        *n_total = distinct;
-      }
-    }
+    out = (int *)take(std::max<u64>(1, lim) * nF * sizeof(int));
+    if (!rows || !perm || !tmp || !hist || !flag || !off || !out) return CC_ENOMEM;
+    unsigned *sorted = nullptr;
+    if (cc::launch_rows_extract(c->stream, c->dev, cur, n_cur, RW, D, nF, rows, perm) ||
+        (sets && cc::launch_rows_canon(c->stream, c->dev, rows, nF, n_cur)) ||
+        cc::launch_rows_sort(c->stream, c->dev, rows, nF, R->L.nb, n_cur, perm, tmp, hist,
+                             &sorted) ||
+        cc::launch_rows_heads(c->stream, c->dev, rows, nF, sorted, n_cur, flag) ||
+        cc::launch_scan_u32(c->stream, c->dev, flag, n_cur, off, scratch) ||
+        cc::launch_rows_gather(c->stream, c->dev, rows, nF, sorted, n_cur, flag, off, lim, out))
+      return CC_ECUDA;
+    c->launches += 10;
+    const int rc = read_u64(c, off + n_cur, &made[S + 1]);
+    if (rc) return rc;
   }
-  cleanup();
-  return rc;
+  const u64 m = std::min<u64>(limit, made[S + 1]);
+  if (m) {
+    CUDA_OK(cudaMemcpyAsync(h_out, out, m * nF * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_OK(cudaStreamSynchronize(c->stream));
+  }
+  *n_out = m;
+  *n_total = made[S + 1];
+  return CC_OK;
 }
 
 // 64-bit fingerprint of a CSR graph (splitmix64 finaliser over its words); never 0.

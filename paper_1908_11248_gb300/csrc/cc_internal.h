@@ -277,18 +277,38 @@ struct EnumArgs {
   GraphDev G;
   KeyLayout L;
   const EnumNode *nodes;  // device array
-  int x;                  // node processed by this step
+  int x;                  // node expanded by this step (a forget or a join)
+  // nodes pre[u0, u1) come between the previous expansion and x in pre-order: introduces and
+  // leaves, which change a state but do not multiply it; a step applies them as it reads a state
+  const int *pre;
+  int u0, u1;
   int nF, R, D;           // state = R ints: trial, colour set, depth, stack[D], Phi[nF]
   const int *in;
-  unsigned long long n_in;
+  unsigned long long n_in;             // states in `in` (the most there can be when n_dev is set)
+  const unsigned long long *n_dev;     // their number, on the device (null: n_in)
   int *out;
   const unsigned long long *off;  // write pass: first output state of each input state
   unsigned *cnt;                  // count pass: output states per input state
+  // append pass: output states taken from *cursor, those beyond `cap` dropped; a state's
+  // candidates are shared by `chunks` warps
+  unsigned long long *cursor, cap;
+  int chunks;
 };
 
 int launch_enum_init(cudaStream_t s, const DevInfo &d, int kw, const EnumArgs &a,
                      const void *root, unsigned long long bound, unsigned long long *n);
+// mode 0 counts, 1 writes at the offsets of the counts, 2 appends
 int launch_enum_step(cudaStream_t s, const DevInfo &d, int kw, int mode, const EnumArgs &a);
+// Rows of at most kMaxBag vertices whose ids take at most 127 bits together, as table records
+// (slot f = Phi(f) without a colour set, a marker bit above them, count 1), and the order that
+// sorts them lexicographically; rows of a table of such records.
+SortSpec rows_spec(int nF, int nb);
+int launch_rows_pack(cudaStream_t s, const DevInfo &d, int kw, const int *states,
+                     unsigned long long n, const unsigned long long *n_dev, int R, int D,
+                     int nF, int nb, int canon, void *recs);
+int launch_rows_unpack(cudaStream_t s, const DevInfo &d, int kw, const void *recs,
+                       const unsigned long long *n, unsigned long long limit, int nF, int nb,
+                       int *out);
 size_t scan_scratch_words(const DevInfo &d);
 // exclusive scan of n u32 values into off[0..n) and the total into off[n]
 int launch_scan_u32(cudaStream_t s, const DevInfo &d, const unsigned *v, unsigned long long n,
