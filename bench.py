@@ -219,7 +219,8 @@ KERNEL_GROUPS = {
     "reduce_write_kernel": "forget", "forget_kernel": "forget", "part_hist_kernel": "forget",
     "part_cursor_kernel": "forget", "part_split_kernel": "forget",
     "part_local_kernel": "forget",
-    "join_build_kernel": "join", "join_probe_kernel": "join", "root_kernel": "root",
+    "join_build_kernel": "join", "join_probe_kernel": "join",
+    "join_group_kernel": "join", "root_kernel": "root",
 }
 
 

@@ -102,8 +102,10 @@ static __device__ __forceinline__ void store_slot(Slot<u128> *s, u64 i, u128 key
 template <typename K>
 __device__ __forceinline__ u64 table_bound(const TableDesc &t) {
   if (t.hashed) return t.cap;
-  u64 c = *t.count;
-  return c < t.cap ? c : t.cap;
+  // more entries than room: some slots below cap may never have been written (the run is
+  // repeated with more room), so none is read
+  const u64 c = *t.count;
+  return c <= t.cap ? c : 0;
 }
 
 // ---- hash table (open addressing, linear probing, key claimed by compare-and-swap) -------
@@ -339,10 +341,8 @@ __device__ __forceinline__ SK sort_key(K key, const SortSpec &sp) {
 #pragma unroll
   for (int j = 0; j < kMaxBag; ++j)
     if (j < ns) s = (s << sp.L.nb) | (SK)(unsigned)key_slot(key, sp.L, sp.order[j]);
-  if (sp.full) {
-    if (sp.L.tb) s = (s << sp.L.tb) | (SK)(unsigned)key_trial(key, sp.L);
-    s = (s << sp.L.k) | (SK)key_mask(key, sp.L);
-  }
+  if ((sp.full || sp.trial) && sp.L.tb) s = (s << sp.L.tb) | (SK)(unsigned)key_trial(key, sp.L);
+  if (sp.full) s = (s << sp.L.k) | (SK)key_mask(key, sp.L);
   if (sp.hbits) s |= (SK)sort_bucket(key, sp) << sp.bits;
   return s;
 }

@@ -273,7 +273,8 @@ __global__ void enum_init_kernel(EnumArgs a, const void *root, u64 bound, unsign
 }
 
 // exclusive scan of n u32 values into u64 offsets; total at off[n]
-__global__ void block_sums_kernel(const unsigned *v, u64 n, u64 per, u64 *sums) {
+__global__ void block_sums_kernel(const unsigned *v, u64 cap, const u64 *n_dev, u64 *sums) {
+  const u64 n = n_dev ? min(*n_dev, cap) : cap, per = (n + gridDim.x - 1) / gridDim.x;
   const u64 lo = blockIdx.x * per, hi = min(n, lo + per);
   u64 s = 0;
   for (u64 i = lo + threadIdx.x; i < hi; i += blockDim.x) s += v[i];
@@ -292,25 +293,36 @@ __global__ void __launch_bounds__(1024) scan_small_kernel(u64 *v, int m, u64 *to
   block_scan_array(v, v, (u64)m, total);
 }
 
-// each block scans its range sequentially in chunks of blockDim (one block per range)
-__global__ void block_scan_kernel(const unsigned *v, u64 n, u64 per, const u64 *sums, u64 *off) {
-  __shared__ u64 s[1024];
+// each block scans its range in chunks of blockDim (one block per range): warp shuffles and one
+// pass over the 32 warp totals a chunk
+__global__ void __launch_bounds__(1024) block_scan_kernel(const unsigned *v, u64 cap,
+                                                          const u64 *n_dev, const u64 *sums,
+                                                          u64 *off) {
+  __shared__ u64 s_w[2][32];  // alternating, so that one barrier a chunk is enough
+  const u64 n = n_dev ? min(*n_dev, cap) : cap, per = (n + gridDim.x - 1) / gridDim.x;
   const u64 lo = blockIdx.x * per, hi = min(n, lo + per);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   u64 run = sums[blockIdx.x];
-  for (u64 b = lo; b < hi; b += blockDim.x) {
+  int flip = 0;
+  for (u64 b = lo; b < hi; b += 1024, flip ^= 1) {
     const u64 i = b + threadIdx.x;
-    const u64 x = i < hi ? v[i] : 0;
-    s[threadIdx.x] = x;
-    __syncthreads();
-    for (unsigned o = 1; o < blockDim.x; o <<= 1) {
-      u64 y = threadIdx.x >= o ? s[threadIdx.x - o] : 0;
-      __syncthreads();
-      s[threadIdx.x] += y;
-      __syncthreads();
+    const u64 own = i < hi ? v[i] : 0;
+    u64 x = own;
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
-    if (i < hi) off[i] = run + s[threadIdx.x] - x;
-    run += s[blockDim.x - 1];
+    if (lane == 31) s_w[flip][w] = x;
     __syncthreads();
+    u64 t = s_w[flip][lane];  // every warp scans the warp totals for itself
+    const u64 mine = t;
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
+    }
+    const u64 before = __shfl_sync(0xffffffffu, t - mine, w);
+    if (i < hi) off[i] = run + before + x - own;
+    run += __shfl_sync(0xffffffffu, t, 31);
   }
 }
 
@@ -573,16 +585,14 @@ int launch_rows_unpack(cudaStream_t s, const DevInfo &d, int kw, const void *rec
 size_t scan_scratch_words(const DevInfo &d) { return (size_t)d.sms * 2 + 2; }
 
 int launch_scan_u32(cudaStream_t s, const DevInfo &d, const unsigned *v, unsigned long long n,
-                    unsigned long long *off, unsigned long long *scratch) {
-  // scratch: block sums (sms * 2 words) then the total
-  const int nb = d.sms * 2;
-  const u64 per = (n + nb - 1) / nb;
-  u64 *sums = scratch, *total = scratch + nb;
-  if (n == 0) return (int)cudaMemsetAsync(off, 0, sizeof(u64), s);
-  block_sums_kernel<<<nb, 256, 0, s>>>(v, n, per, sums);
-  scan_small_kernel<<<1, 1024, 0, s>>>(sums, nb, total);
-  block_scan_kernel<<<nb, 1024, 0, s>>>(v, n, per, sums, off);
-  cudaMemcpyAsync(off + n, total, sizeof(u64), cudaMemcpyDeviceToDevice, s);
+                    unsigned long long *off, unsigned long long *scratch,
+                    const unsigned long long *n_dev, unsigned long long *total) {
+  const int nb = d.sms * 2;  // scratch: block sums
+  if (!total) total = off + n;
+  if (n == 0) return (int)cudaMemsetAsync(total, 0, sizeof(u64), s);
+  block_sums_kernel<<<nb, 256, 0, s>>>(v, n, n_dev, scratch);
+  scan_small_kernel<<<1, 1024, 0, s>>>(scratch, nb, total);
+  block_scan_kernel<<<nb, 1024, 0, s>>>(v, n, n_dev, scratch, off);
   return (int)cudaGetLastError();
 }
 

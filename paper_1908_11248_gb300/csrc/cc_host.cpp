@@ -922,7 +922,99 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                  [&] { return cc::launch_forget(c->stream, c->dev, R->kw, block, a); });
       if (rc) return rc;
       release_child(y);
-    } else {  // join
+    } else if (R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
+               entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries) {
+      // join, group by group (cc_join.cu)
+      const int b = (int)nd.bag.size();
+      int y = nd.child0, z = nd.child1;
+      if (entries(y) > entries(z)) std::swap(y, z);  // y's groups look theirs up in z
+      // the order both must have: that of a child sorted by all its slots (the larger one's if
+      // both are), else the one the parent likes best
+      auto sorted_full = [&](int v) {
+        const cc::NodeTable &t = R->tables[v];
+        return !t.hashed && t.sort_n == b && t.sort_hbits == 0;
+      };
+      cc::SortSpec sp = forget_order(x);
+      const int lead = sorted_full(z) ? z : sorted_full(y) ? y : -1;
+      if (lead >= 0)
+        for (int j = 0; j < b; ++j) sp.order[j] = R->tables[lead].sort_slots[j];
+      sp.nsl = b;
+      sp.full = 0;
+      sp.trial = 1;
+      sp.bits = b * R->L.nb + R->L.tb;
+      struct Held {  // what this node holds until it is done
+        Arena &a;
+        std::vector<void *> p;
+        ~Held() {
+          for (void *q : p) a.release(q);
+        }
+      } held{A, {}};
+      auto in_order = [&](int v, TableDesc *t) -> int {
+        const cc::NodeTable &ty = R->tables[v];
+        bool as_is = sorted_full(v);
+        for (int j = 0; j < b && as_is; ++j) as_is = ty.sort_slots[j] == sp.order[j];
+        *t = desc(v);
+        if (as_is) return CC_OK;
+        const u64 m = entries(v);
+        void *s = nullptr;
+        check(R->d_counters + v, m);
+        const int r = sort_records(x, sp, ty.slots, ty.hashed ? c->d_ones : t->count, ty.cap,
+                                   R->d_counters + v, m, &s);
+        held.p.push_back(s);
+        if (r) return r;
+        *t = TableDesc{s, std::max<u64>(1, m), R->d_counters + v, 0};
+        release_child(v);
+        return CC_OK;
+      };
+      cc::JoinGroupArgs a{};
+      a.G = G;
+      a.L = R->L;
+      a.sp = sp;
+      a.bag = b;
+      a.err = R->d_err;
+      rc = in_order(y, &a.a);
+      if (!rc) rc = in_order(z, &a.b);
+      if (rc) return rc;
+      auto hold = [&](size_t bytes) {
+        held.p.push_back(A.alloc(bytes));
+        return held.p.back();
+      };
+      a.groups = (u64 *)hold(sizeof(u64));
+      a.first = (u64 *)hold(a.a.cap * sizeof(u64));
+      a.blo = (u64 *)hold(a.a.cap * sizeof(u64));
+      a.blen = (unsigned *)hold(a.a.cap * sizeof(unsigned));
+      a.cnt = (unsigned *)hold(a.a.cap * sizeof(unsigned));
+      u64 *off = (u64 *)hold(a.a.cap * sizeof(u64));
+      u64 *scan = (u64 *)hold(cc::scan_scratch_words(c->dev) * sizeof(u64));
+      for (void *q : held.p)
+        if (!q) return CC_ENOMEM;
+      a.off = off;
+      rc = timed(x, CC_K_JOIN_BUILD, 4,
+                 [&] { return cc::launch_join_match(c->stream, c->dev, R->kw, a, blk); });
+      if (rc) return rc;
+      rc = timed(x, CC_K_JOIN_COUNT, 4, [&] {
+        const int r = cc::launch_join_groups(c->stream, c->dev, R->kw, 0, a);
+        return r ? r : cc::launch_scan_u32(c->stream, c->dev, a.cnt, a.a.cap, off, scan, a.groups,
+                                           R->d_counters + x);
+      });
+      if (rc) return rc;
+      u64 total = planned ? room(plan->entries[x]) : 0;
+      if (!planned) rc = read_u64(c, R->d_counters + x, &total);
+      if (rc) return rc;
+      const u64 cap = std::max<u64>(1, total);
+      void *p = A.alloc(cap * rb);
+      if (!p) return CC_ENOMEM;
+      R->tables[x] = {p, cap, 0, true};
+      R->tables[x].sort_n = b;
+      for (int j = 0; j < b; ++j) R->tables[x].sort_slots[j] = sp.order[j];
+      check(R->d_counters + x, cap);
+      a.out = desc(x);
+      rc = timed(x, CC_K_JOIN_WRITE, 1,
+                 [&] { return cc::launch_join_groups(c->stream, c->dev, R->kw, 1, a); });
+      if (rc) return rc;
+      release_child(y);
+      release_child(z);
+    } else {  // join through hash tables
       int y = nd.child0, z = nd.child1;
       if (entries(y) > entries(z)) std::swap(y, z);  // chain the smaller child
       u64 icap = hash_cap(entries(y), lf);
@@ -2067,7 +2159,8 @@ int cc_create(cc_ctx **out, int device, void *stream, void *d_arena, size_t aren
     return CC_ECUDA;
   }
   c->dev.blocks_per_sm = 8;
-  if (cc::prepare_sort_kernels() != 0 || cc::prepare_part_kernels() != 0) {
+  if (cc::prepare_sort_kernels() != 0 || cc::prepare_part_kernels() != 0 ||
+      cc::prepare_join_kernels() != 0) {
     delete c;
     return CC_ECUDA;
   }

@@ -69,3 +69,75 @@ def test_enumeration_first_forget_over_all_vertices(ctx, n):
         run = cc.cc_run_dp(ctx.h, pid, cid, cc.cc_default_opts(retain=1))
         rows, got = cc.cc_enumerate(ctx.h, run, 10 ** 6, nF)
         assert got == total and np.array_equal(rows, want)
+
+
+def rows_of(trial, phi, mask, cnt):
+    """A table as sorted rows (trial, phi, colour set, count)."""
+    cols = [np.asarray(trial, np.uint64)] + [np.asarray(p, np.uint64) for p in np.asarray(phi).T]
+    cols += [np.asarray(mask, np.uint64), np.asarray(cnt, np.uint64)]
+    return np.stack(cols)[:, np.lexsort(cols[::-1])]
+
+
+def check_tables(ctx, g, pat, z, k, reps=2, **opt):
+    """Counts, sizes and every stored table, of an exact and a planned run, against the oracle."""
+    T = z.shape[0]
+    ref = oracle.run_dp(g, pat, z, k)
+    cc.cc_load_graph(ctx.h, *g)
+    pid = cc.cc_load_pattern(ctx.h, *pat)
+    N, _ = cc.cc_pattern_info(ctx.h, pid)
+    nodes = cc.cc_pattern_nodes(ctx.h, pid, pat[0])
+    cid = cc.cc_set_colors(ctx.h, z, k)
+    for rep in range(reps):
+        run = cc.cc_run_dp(ctx.h, pid, cid, cc.cc_default_opts(retain=1, **opt))
+        assert cc.cc_run_mode(ctx.h, run) == ("planned" if rep else "exact")
+        assert np.array_equal(cc.cc_count(ctx.h, run, T), ref.count)
+        assert np.array_equal(cc.cc_decide(ctx.h, run, T), ref.exists)
+        sizes = cc.cc_table_stats(ctx.h, run, N)[0]
+        assert np.array_equal(sizes, ref.node_sizes.sum(axis=0))
+        for x, nd in enumerate(nodes):
+            b = len(nd[4])
+            try:
+                tr, phi, mask, cnt = cc.cc_table_dump(ctx.h, run, x, int(sizes[x]) + 1, b)
+            except cc.CCError as ex:
+                assert ex.code == cc.CC_EINVAL and nd[0] == cc.INTRODUCE
+                continue
+            got = rows_of(tr, phi, mask, cnt)
+            want = [ref.table(t, x, b) for t in range(T)]
+            want = rows_of(np.repeat(np.arange(T), [len(m) for _, m, _ in want]),
+                           np.concatenate([np.reshape(p, (len(m), b)) for p, m, _ in want]),
+                           np.concatenate([m for _, m, _ in want]),
+                           np.concatenate([c for _, _, c in want]))
+            assert np.array_equal(got, want), (rep, x)
+        cc.cc_release(ctx.h, run)
+    cc.cc_release_colors(ctx.h, cid)
+
+
+# a bag of one vertex: k - 1 private colours.  One word of sums, the edge of a word, several
+# words, the most a warp keeps (11 private colours), one more (hash tables); few entries (hash
+# tables) and more than the 2^21 at which children are sorted and joined group by group
+@pytest.mark.parametrize("k", [4, 6, 7, 12, 13])
+@pytest.mark.parametrize("many", [0, 1])
+def test_join_routes(ctx, k, many):
+    n, trials = (8000, 3 + 36 // (k - 1)) if many else (70, 3)
+    g = synth.erdos_renyi(n, 8 / n, 6)
+    check_tables(ctx, g, star_of_joins(4), oracle.colors(n, trials, k, seed=k), k)
+
+
+# the 4-cycle as the join of its two paths between opposite corners, bag {0, 2}: 64-bit keys, and
+# 128-bit keys (20 bits a vertex)
+@pytest.mark.parametrize("n,deg", [(1100, 37.0), (530_000, 2.0)])
+def test_join_of_paths(ctx, n, deg):
+    pat = (4, np.array([(0, 1), (1, 2), (2, 3), (0, 3)], np.int32),
+           ([[0, 2], [0, 1, 2], [0, 2, 3]], [-1, 0, 0]))
+    g = synth.erdos_renyi(n, deg / n, 8)
+    check_tables(ctx, g, pat, oracle.colors(n, 2, 5, seed=8), 5)
+
+
+def test_join_routes_hubs_and_empty(ctx):
+    """Bags of up to three vertices over hubs, and a graph without an edge."""
+    n = 150
+    g = synth.power_law_config(n, 4.0, 2.5, 3)
+    for pat in (synth.pattern_A(), synth.random_partial_ktree(8, 3, 7)):
+        check_tables(ctx, g, pat, oracle.colors(n, 2, pat[0], seed=8), pat[0])
+    e = synth.csr_from_edges(n, np.zeros((0, 2), np.int64))
+    check_tables(ctx, e, synth.pattern_A(), oracle.colors(n, 2, 9, seed=1), 9)
