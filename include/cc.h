@@ -148,8 +148,9 @@ typedef struct {
   int32_t fuse;          /* introduce followed by forget: 0 each node stores its own table;   */
                          /* 1 the introduce adds its entries, projected, into the forget's     */
                          /*   hash table; 2 (default) it writes them projected and densely,    */
-                         /*   they are sorted and equal keys reduced.  With 1 and 2 the        */
-                         /*   introduce's table is never stored (its size is still counted)    */
+                         /*   they are sorted and equal keys reduced (few entries: as 1, when  */
+                         /*   sort_sweep is 1).  With 1 and 2 the introduce's table is never   */
+                         /*   stored (its size is still counted)                               */
   int32_t use_graph;     /* 1: replay the node kernels from a captured CUDA graph when the     */
                          /*    plan's capacities are known (falls back to planning otherwise)  */
   float load_factor;     /* hash-table fill target in (0, 0.9]; 0 = library default           */

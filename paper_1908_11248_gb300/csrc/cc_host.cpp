@@ -399,6 +399,9 @@ int pos_in(const std::vector<int32_t> &bag, int u) {
   return (int)(std::lower_bound(bag.begin(), bag.end(), u) - bag.begin());
 }
 
+// most entries an introduce adds into its forget's hash table instead of having them sorted
+constexpr u64 kHashEntries = 1ull << 18;
+
 // ---- the planner: node by node in post-order, exact capacities ----------------------------
 int finish_run(Ctx *c, Run *R);
 int near_slot(const Pattern &P, int u, const std::vector<int32_t> &child_bag, int *dist);
@@ -529,6 +532,24 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     return x2;
   };
   std::vector<int> chain_from(N, -1);  // x2 -> the x1 it runs together with
+  // Few entries (default sort schedule): an introduce adds them into its forget's hash table and
+  // a grouped introduce takes its child unsorted, because the dozen launches of a sort and its
+  // reduce cost more than the atomics and the shared lists save.  Measured in planned runs,
+  // introduce and forget together: 0.087 ms with a sort, 0.014 with the hash table at 10 000
+  // entries; 0.12 and 0.08 at 60 000; 0.15 and 0.14 at 155 000; a million about the same
+  // (0.21 and 0.2), but then without the order that a grouped introduce above could use.
+  // Small windows (IntroArgs::win) go with it: 29 000 entries whose lists are built one by one
+  // take 0.36 ms in 900 warps of 32 entries, 0.09 ms in 7000 warps of 4.
+  const bool hash_few = R->opts.sort_sweep == 1;
+  auto few = [&](u64 e) { return hash_few && e <= kHashEntries; };
+  // true if an introduce above forget f hands f's order on to a grouped introduce above it
+  auto order_handed_on = [&](int f) {
+    const int g = P.nodes[f].parent, h = g >= 0 ? P.nodes[g].parent : -1;
+    if (h < 0 || P.nodes[g].type != 1 || P.nodes[h].type != 1 || !R->opts.group) return false;
+    int nnb = 0;
+    for (int w : P.nodes[g].bag) nnb += P.adj[P.nodes[h].vertex] >> w & 1u;
+    return nnb >= 2;
+  };
   // full sort order for the table of forget node f: when the next node introduces a vertex
   // with bag neighbours, their slots come first so that its runs are contiguous (when that
   // introduce runs chained with its parent, the parent's bag neighbours come first)
@@ -676,7 +697,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       // that a run shares one candidate list; sort it unless its order already starts with them
       const int grouped = R->opts.group && a.nnb >= 2 && a.nnb * R->L.nb <= 64;
       void *sorted = nullptr;
-      if (grouped && !grouped_by(R->tables[y], a.nnb, a.nb_slot)) {
+      if (grouped && !grouped_by(R->tables[y], a.nnb, a.nb_slot) &&
+          !few(planned ? plan->entries[y] : R->sizes[y])) {
         cc::SortSpec sp{};
         sp.L = R->L;
         sp.b = a.b_in;
@@ -704,7 +726,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         });
         if (rc) return rc;
         rc = read_u64(c, blk + 2 * grid, &total);
-        if (!rc) rc = read_u64(c, a.cand, &cand);
+        if (!rc && R->opts.profile) rc = read_u64(c, a.cand, &cand);
         if (rc) return rc;
         if (R->opts.profile) R->timings.back().candidates = cand;
         R->sizes[x] = total;
@@ -714,11 +736,16 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       // chunk shrinks for small tables so that those holes stay under a quarter of the entries
       const bool warp_path = planned && (a.nnb <= 1 || grouped);
       a.chunk = 256;
+      a.win = 32;
       u64 slack = chunk_slack;
       if (warp_path) {
         const u64 warps = (u64)c->dev.sms * c->dev.blocks_per_sm * 8;
         while (a.chunk > 32 && warps * a.chunk * 4 > plan->entries[x]) a.chunk >>= 1;
         slack = warps * a.chunk;
+        // fewer entries a window while that puts more of the GPU's warps to work
+        const cc::NodeTable &ty = R->tables[y];
+        const u64 scan = ty.hashed ? ty.cap : plan->entries[y];
+        while (a.win > 4 && warps * a.win > scan) a.win >>= 1;
       }
       const u64 raw = planned ? room(plan->entries[x]) + slack : std::max<u64>(1, total);
       if (planned) check(R->d_counters + x, room(plan->entries[x]));
@@ -756,7 +783,9 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         return r;
       };
       const int f = nd.parent;
-      const int fuse = (f >= 0 && P.nodes[f].type == 2) ? R->opts.fuse : 0;
+      int fuse = (f >= 0 && P.nodes[f].type == 2) ? R->opts.fuse : 0;
+      if (fuse == 2 && x1 < 0 && few(planned ? plan->entries[x] : total) && !order_handed_on(f))
+        fuse = 1;
       if (fuse == 1) {  // add projected entries into the forget's hash table
         rc = new_hash(f, planned ? room(plan->entries[f]) : total);
         if (rc) return rc;

@@ -75,6 +75,7 @@ struct IntroArgs {
   int *err;
   uint32_t ubit;             // 1 << u, tested against G.allow
   unsigned chunk;            // warp kernels, mode 1: slots a warp reserves at a time (32..256)
+  unsigned win;              // warp kernels: child entries a warp takes at a time (4..32)
   // chained introduce (launch_intro_chain): the input is the child y of a lower introduce x1
   // whose table is not stored; the fields above describe the upper introduce x2 (its bag
   // neighbours' slots counted in y's bag), these the lower one

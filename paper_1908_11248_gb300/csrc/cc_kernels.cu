@@ -499,12 +499,14 @@ __global__ void __launch_bounds__(256, 4) intro_warp_kernel(IntroArgs a) {
   // the next window's records are loaded while the current one is expanded
   K nkey = 0;
   u64 nc_ = 0;
-  if (wid * 32 + lane < bound) load_slot(in, wid * 32 + lane, nkey, nc_);
-  for (u64 base = wid * 32; base < bound; base += warps * 32) {
+  const u64 win = a.win;
+  const u64 mylane = lane < (int)win ? (u64)lane : bound;  // lanes beyond the window hold nothing
+  if (wid * win + mylane < bound) load_slot(in, wid * win + mylane, nkey, nc_);
+  for (u64 base = wid * win; base < bound; base += warps * win) {
     const K key = nkey;
     const u64 c = nc_;
     {
-      const u64 i2 = base + warps * 32 + lane;
+      const u64 i2 = base + warps * win + mylane;
       nkey = 0;
       nc_ = 0;
       if (i2 < bound) load_slot(in, i2, nkey, nc_);
@@ -683,7 +685,8 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   const u64 warps = (u64)gridDim.x * (blockDim.x / 32);
   const u64 wid = (u64)blockIdx.x * (blockDim.x / 32) + wib;
   const u64 bound = warp_run_failed(a.err) ? 0 : table_bound<K>(a.in);
-  const u64 nwin = (bound + 31) / 32, per = (nwin + warps - 1) / warps;
+  const u64 width = a.win, mylane = lane < (int)width ? (u64)lane : bound;
+  const u64 nwin = (bound + width - 1) / width, per = (nwin + warps - 1) / warps;
   const u64 w0 = min(nwin, wid * per), w1 = min(nwin, w0 + per);
   const int q = MODE == 2 ? a.q : a.proj_q;
   const int vsh = intro_vshift(a.L, a.p, q);
@@ -699,12 +702,12 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   // the next window's records are loaded while the current one is processed
   K nkey = 0;
   u64 nc_ = 0;
-  if (w0 < w1 && w0 * 32 + lane < bound) load_slot(in, w0 * 32 + lane, nkey, nc_);
+  if (w0 < w1 && w0 * width + mylane < bound) load_slot(in, w0 * width + mylane, nkey, nc_);
   for (u64 win = w0; win < w1; ++win) {
     const K key = nkey;
     const u64 c = nc_;
     {
-      const u64 i2 = (win + 1) * 32 + lane;
+      const u64 i2 = (win + 1) * width + mylane;
       nkey = 0;
       nc_ = 0;
       if (win + 1 < w1 && i2 < bound) load_slot(in, i2, nkey, nc_);
@@ -869,7 +872,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         cs = __shfl_sync(0xffffffffu, lstart, l);
         cl = __shfl_sync(0xffffffffu, llen, l);
       }
-      ctup = __shfl_sync(0xffffffffu, tup, 31);
+      ctup = __shfl_sync(0xffffffffu, tup, (int)width - 1);
       if (ctup == ~0ull) cl = -1;
     } else {  // entry by entry, every check in full
       int best = INT_MAX, rs = 0, anc = 0;
@@ -1128,6 +1131,12 @@ __global__ void unpack_kernel(KeyLayout L, TableDesc t, int b, int32_t *trial, i
   }
 }
 
+// blocks of eight warps that take windows of a.win records: no more than the table can fill
+int warp_grid(const DevInfo &d, const IntroArgs &a) {
+  const u64 want = (a.in.cap + 8 * a.win - 1) / (8 * a.win), most = (u64)d.sms * d.blocks_per_sm;
+  return (int)(want < most ? (want ? want : 1) : most);
+}
+
 int grid_for(const DevInfo &d, int block) {
   int per_sm = d.blocks_per_sm * 256 / block;
   if (per_sm < 1) per_sm = 1;
@@ -1227,7 +1236,7 @@ int launch_deg8(cudaStream_t s, const DevInfo &d, const int32_t *row_ptr, int32_
 
 int launch_intro_group_warp(cudaStream_t s, const DevInfo &d, int kw, int mode,
                             const IntroArgs &a) {
-  const int grid = d.sms * d.blocks_per_sm;
+  const int grid = warp_grid(d, a);
   if (kw == 1) {
     if (mode == 1) intro_group_warp_kernel<u64, 1><<<grid, 256, 0, s>>>(a);
     else intro_group_warp_kernel<u64, 2><<<grid, 256, 0, s>>>(a);
@@ -1247,14 +1256,14 @@ int launch_nb_colour_hist(cudaStream_t s, const DevInfo &d, const GraphDev &G, i
 }
 
 int launch_intro_chain(cudaStream_t s, const DevInfo &d, int kw, const IntroArgs &a) {
-  const int grid = d.sms * d.blocks_per_sm;
+  const int grid = warp_grid(d, a);
   if (kw == 1) intro_group_warp_kernel<u64, 1, true><<<grid, 256, 0, s>>>(a);
   else intro_group_warp_kernel<u128, 1, true><<<grid, 256, 0, s>>>(a);
   return (int)cudaGetLastError();
 }
 
 int launch_intro_warp(cudaStream_t s, const DevInfo &d, int kw, int mode, const IntroArgs &a) {
-  const int grid = d.sms * d.blocks_per_sm;
+  const int grid = warp_grid(d, a);
   // a window's candidates number at most 32 * n (no bag neighbour: every vertex per entry)
   const bool narrow = (long long)a.G.n * 32 < (1ll << 31);
 #define CC_IW(K, M)                                                         \

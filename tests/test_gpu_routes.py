@@ -141,3 +141,16 @@ def test_join_routes_hubs_and_empty(ctx):
         check_tables(ctx, g, pat, oracle.colors(n, 2, pat[0], seed=8), pat[0])
     e = synth.csr_from_edges(n, np.zeros((0, 2), np.int64))
     check_tables(ctx, e, synth.pattern_A(), oracle.colors(n, 2, 9, seed=1), 9)
+
+
+# few entries go into the forget's hash table, more than 2^18 of an introduce are sorted and
+# reduced; a 3x3 grid's first forget keeps its order for the chained pair above it either way
+@pytest.mark.parametrize("pat,n,deg,trials", [
+    (("cycle", 5), 3, 2.0, 1), (("cycle", 5), 30, 6.0, 2), (("cycle", 5), 500, 7.0, 2),
+    (("cycle", 5), 1300, 8.0, 3), (("grid", 2, 3), 700, 6.0, 3), (("grid", 2, 4), 2000, 7.0, 6),
+    (("grid", 3, 3), 90, 7.0, 3), (("grid", 3, 3), 2500, 9.0, 4), (("path", 6), 9000, 5.0, 5)])
+def test_forget_routes(ctx, pat, n, deg, trials):
+    p = synth.make_pattern(pat)
+    k = p[0] + 1
+    check_tables(ctx, synth.erdos_renyi(n, min(1.0, deg / n), 3), p,
+                 oracle.colors(n, trials, k, seed=5), k)
