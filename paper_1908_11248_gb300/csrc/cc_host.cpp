@@ -716,9 +716,11 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       }
       struct SortedGuard {
         Arena &a;
-        void *p;
+        void *&p;
         ~SortedGuard() { a.release(p); }
       } sorted_guard{A, sorted};
+      void *heavy_mem = nullptr;
+      SortedGuard heavy_guard{A, heavy_mem};
       u64 total = 0, cand = 0;
       if (!planned) {
         rc = timed(x, CC_K_INTRO_COUNT, 2, [&] {
@@ -746,6 +748,20 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         const cc::NodeTable &ty = R->tables[y];
         const u64 scan = ty.hashed ? ty.cap : plan->entries[y];
         while (a.win > 4 && warps * a.win > scan) a.win >>= 1;
+        // hubs: room for the parts of their lists (8 MB at most; what does not fit is walked in
+        // place), and for the second kernel's last chunks
+        if (a.nnb == 1 && a.G.row_ptr == c->d_row_ptr && c->max_deg > cc::kHeavyList) {
+          const u64 parts = (u64)(c->max_deg + cc::kHeavyPart - 1) / cc::kHeavyPart;
+          const u64 places = std::min<u64>(1 << 20, room(plan->entries[y]) * parts);
+          heavy_mem = A.alloc((places + 1) * sizeof(u64));
+          if (heavy_mem) {
+            a.heavy_cap = places;
+            a.heavy_n = (u64 *)heavy_mem;
+            a.heavy = a.heavy_n + 1;
+            CUDA_OK(cudaMemsetAsync(a.heavy_n, 0, sizeof(u64), c->stream));
+            slack *= 2;
+          }
+        }
       }
       const u64 raw = planned ? room(plan->entries[x]) + slack : std::max<u64>(1, total);
       if (planned) check(R->d_counters + x, room(plan->entries[x]));
@@ -766,7 +782,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         if (x1 >= 0 && a.c_nnb == 1 && R->L.k <= 16 && c->max_deg < 65536)
           hist = arena_alloc<u64>(c, (size_t)R->trials * (size_t)n * 4);
         a.c_hist = hist;
-        int r = timed(x, x1 >= 0 ? CC_K_INTRO_CHAIN : CC_K_INTRO_WRITE, hist ? 2 : 1, [&] {
+        int r = timed(x, x1 >= 0 ? CC_K_INTRO_CHAIN : CC_K_INTRO_WRITE,
+                      hist || a.heavy_cap ? 2 : 1, [&] {
           if (hist) {
             const int h = cc::launch_nb_colour_hist(c->stream, c->dev, a.G, R->trials, a.c_degF,
                                                     a.c_ubit, hist, a.cand);
@@ -794,7 +811,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         a.valid = R->d_counters + x;
         a.cand = planned ? R->d_counters + 3 * N + x : nullptr;
         const bool warp = planned && a.nnb <= 1, gwarp = planned && grouped;
-        rc = timed(x, CC_K_INTRO_FUSED, 1, [&] {
+        rc = timed(x, CC_K_INTRO_FUSED, a.heavy_cap ? 2 : 1, [&] {
           return warp    ? cc::launch_intro_warp(c->stream, c->dev, R->kw, 2, a)
                  : gwarp ? cc::launch_intro_group_warp(c->stream, c->dev, R->kw, 2, a)
                          : cc::launch_intro_blk(c->stream, c->dev, R->kw, 2, grouped, block, a,

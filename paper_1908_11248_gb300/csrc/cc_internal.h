@@ -76,6 +76,10 @@ struct IntroArgs {
   uint32_t ubit;             // 1 << u, tested against G.allow
   unsigned chunk;            // warp kernels, mode 1: slots a warp reserves at a time (32..256)
   unsigned win;              // warp kernels: child entries a warp takes at a time (4..32)
+  // launch_intro_warp: the long candidate lists of a window that has many candidates are left to
+  // a second kernel, as (entry, part of its list) items, while there is room for them (heavy_cap
+  // 0: none are)
+  unsigned long long *heavy, *heavy_n, heavy_cap;
   // chained introduce (launch_intro_chain): the input is the child y of a lower introduce x1
   // whose table is not stored; the fields above describe the upper introduce x2 (its bag
   // neighbours' slots counted in y's bag), these the lower one
@@ -91,6 +95,10 @@ struct IntroArgs {
   // extensions from them instead of walking w's adjacency
   const unsigned long long *c_hist;
 };
+
+constexpr int kHeavyWindow = 2048;  // candidates of a window above which its long lists leave it
+constexpr int kHeavyList = 64;   // longest candidate list such a window keeps
+constexpr int kHeavyPart = 256;  // candidates of a longer one a warp walks at a time
 
 struct ForgetArgs {
   KeyLayout L;

@@ -533,8 +533,29 @@ __global__ void __launch_bounds__(256, 4) intro_warp_kernel(IntroArgs a) {
       const I y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += y;
     }
+    I total = __shfl_sync(0xffffffffu, incl, 31);
+    if (a.heavy_cap && total > (I)kHeavyWindow) {  // the window's long lists go to the other kernel
+      const int parts = nc > (I)kHeavyList ? (int)((nc + kHeavyPart - 1) / kHeavyPart) : 0;
+      int upto = parts;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += y;
+      }
+      u64 at = 0;
+      if (lane == 31) at = atomicAdd(a.heavy_n, (u64)upto);
+      at = __shfl_sync(0xffffffffu, at, 31) + (u64)(upto - parts);
+      const bool fits = at + (u64)parts <= a.heavy_cap;  // else the places taken stay empty
+      for (int j = 0; j < parts && at + j < a.heavy_cap; ++j)
+        a.heavy[at + j] = fits ? (base + lane) | (u64)j << 40 : ~0ull;
+      if (parts && fits) nc = 0;
+      incl = nc;
+      for (int o = 1; o < 32; o <<= 1) {
+        const I y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      total = __shfl_sync(0xffffffffu, incl, 31);
+    }
     const I excl = incl - nc;
-    const I total = __shfl_sync(0xffffffffu, incl, 31);
     if (lane == 0) examined += (u64)total;
     for (I j0 = 0; j0 < total; j0 += 32) {
       const I j = j0 + lane;
@@ -566,6 +587,79 @@ __global__ void __launch_bounds__(256, 4) intro_warp_kernel(IntroArgs a) {
         if (valid) okey = intro_out(eb, vsh, v, cv);
       }
       warp_emit<K, MODE>(a, valid, okey, ec, lane, lt, cbase, cfill, produced, fresh, full);
+    }
+  }
+  if (MODE == 1 && cfill < chunk)  // the unused tail of the warp's last chunk: holes
+    for (u64 j = cfill + lane; j < chunk; j += 32)
+      if (cbase + j < a.out.cap) store_slot(out, cbase + j, (K)0, 0ull);
+  if (full) atomicOr(a.err, kErrOverflow);
+  for (int o = 16; o > 0; o >>= 1) {
+    produced += __shfl_down_sync(0xffffffffu, produced, o);
+    fresh += __shfl_down_sync(0xffffffffu, fresh, o);
+  }
+  if (lane == 0) {
+    if (a.valid && produced) atomicAdd(a.valid, produced);
+    if (MODE == 2 && fresh) atomicAdd(a.out.count, fresh);
+    if (a.cand && examined) atomicAdd(a.cand, examined);
+  }
+}
+
+// The long candidate lists of intro_warp_kernel, one part of one list a warp.  Windows of 32
+// entries put a hub's entries, which a sorted table keeps together, into one warp: 62 000
+// candidates at 32 a step took a millisecond whatever the rest of the table held.  With the
+// lists cut into parts the five expanding introduces of a six-vertex path on a Barabasi-Albert
+// graph (n = 200 000, m = 5, largest degree 1934) went from 6.2 ms to 0.8.  A window of
+// up to kHeavyWindow candidates (64 steps) is walked in place, and so is any list of up to
+// kHeavyList, where 32 entries share steps.
+template <typename K, int MODE>
+__global__ void __launch_bounds__(256, 4) intro_heavy_kernel(IntroArgs a) {
+  const Slot<K> *in = reinterpret_cast<const Slot<K> *>(a.in.slots);
+  Slot<K> *out = reinterpret_cast<Slot<K> *>(a.out.slots);
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const u64 warps = (u64)gridDim.x * (blockDim.x / 32);
+  const u64 wid = (u64)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+  const u64 items = warp_run_failed(a.err) ? 0 : min(*a.heavy_n, a.heavy_cap);
+  const int q = MODE == 2 ? a.q : a.proj_q;
+  const int vsh = intro_vshift(a.L, a.p, q);
+  const u64 chunk = a.chunk;
+  u64 cbase = 0, cfill = chunk, produced = 0, fresh = 0, examined = 0;
+  bool full = false;
+  // the items of a batch are read one a lane, so that their chains of loads overlap
+  const int batch = (int)min((u64)32, (items + warps - 1) / warps);
+  for (u64 b0 = wid * (u64)batch; b0 < items; b0 += warps * (u64)batch) {
+    K lkey = 0;
+    u64 lc = 0;
+    int lr0 = 0, lr1 = 0;
+    if (lane < batch && b0 + lane < items && a.heavy[b0 + lane] != ~0ull) {
+      const u64 item = a.heavy[b0 + lane];
+      load_slot(in, item & ((1ull << 40) - 1ull), lkey, lc);
+      const int w = key_slot(lkey, a.L, a.nb_slot[0]);
+      lr0 = a.G.row_ptr[w] + (int)(item >> 40) * kHeavyPart;
+      lr1 = min(lr0 + kHeavyPart, a.G.row_ptr[w + 1]);
+    }
+    for (int l = 0; l < batch; ++l) {
+      const int r0 = __shfl_sync(0xffffffffu, lr0, l), r1 = __shfl_sync(0xffffffffu, lr1, l);
+      const K key = shfl_key(lkey, l);
+      const u64 c = __shfl_sync(0xffffffffu, lc, l);
+      if (r0 == r1) continue;
+      const K ob = intro_base(key, a.L, a.p, q);
+      const uint32_t cm = key_mask(key, a.L);
+      const uint8_t *col = a.G.colors + (u64)key_trial(key, a.L) * (u64)a.G.n;
+      if (lane == 0) examined += (u64)(r1 - r0);
+      for (int j0 = r0; j0 < r1; j0 += 32) {
+        bool valid = false;
+        K okey = 0;
+        if (j0 + lane < r1) {
+          const int v = __ldg(a.G.col + j0 + lane);
+          const int cv = col[v];
+          valid = !((cm >> cv) & 1u);
+          if (valid && a.degF) valid = a.G.deg8[v] >= a.degF;
+          if (valid && a.G.allow) valid = (a.G.allow[v] & a.ubit) != 0;
+          if (valid) okey = intro_out(ob, vsh, v, cv);
+        }
+        warp_emit<K, MODE>(a, valid, okey, c, lane, lt, cbase, cfill, produced, fresh, full);
+      }
     }
   }
   if (MODE == 1 && cfill < chunk)  // the unused tail of the warp's last chunk: holes
@@ -1268,7 +1362,9 @@ int launch_intro_warp(cudaStream_t s, const DevInfo &d, int kw, int mode, const 
   const bool narrow = (long long)a.G.n * 32 < (1ll << 31);
 #define CC_IW(K, M)                                                         \
   if (narrow) intro_warp_kernel<K, M, int><<<grid, 256, 0, s>>>(a);         \
-  else intro_warp_kernel<K, M, long long><<<grid, 256, 0, s>>>(a)
+  else intro_warp_kernel<K, M, long long><<<grid, 256, 0, s>>>(a);          \
+  if (a.heavy_cap)                                                          \
+    intro_heavy_kernel<K, M><<<d.sms * d.blocks_per_sm, 256, 0, s>>>(a)
   if (kw == 1) {
     if (mode == 1) {
       CC_IW(u64, 1);

@@ -154,3 +154,19 @@ def test_forget_routes(ctx, pat, n, deg, trials):
     k = p[0] + 1
     check_tables(ctx, synth.erdos_renyi(n, min(1.0, deg / n), 3), p,
                  oracle.colors(n, trials, k, seed=5), k)
+
+
+@pytest.mark.parametrize("trials", [2, 40])
+def test_hubs(ctx, trials):
+    """Stars of the degrees at which a candidate list leaves its window (65) and is cut into parts
+    (256), and of one far beyond, joined in a path: lists in parts, runs of equal keys longer than
+    a reduce block's tile and range, in hash tables (few trials) and sorted."""
+    edges, at, centres = [], 0, []
+    for d in (63, 64, 65, 255, 256, 257, 513, 6000):
+        centres.append(at)
+        edges += [(at, at + 1 + i) for i in range(d - 2 if 0 < len(centres) - 1 < 7 else d - 1)]
+        at += d
+    edges += list(zip(centres, centres[1:]))
+    g = synth.csr_from_edges(at, np.array(edges))
+    for pat in (synth.path_pattern(4), synth.star_pattern(4)):
+        check_tables(ctx, g, pat, oracle.colors(at, trials, 5, seed=2), 5)
