@@ -38,9 +38,10 @@ __device__ __forceinline__ int colour_of(const GraphDev &G, int t, int v) {
 }
 
 template <typename SK, typename K>
-__device__ bool sorted_contains(const Slot<K> *s, u64 count, const SortSpec &sp, K key) {
+__device__ bool sorted_contains(const Slot<K> *s, u64 first, u64 count, const SortSpec &sp,
+                                K key) {
   const SK q = sort_key<SK>(key, sp);
-  u64 lo = 0, hi = count;
+  u64 lo = first, hi = count;
   while (lo < hi) {
     const u64 mid = (lo + hi) >> 1;
     K km;
@@ -83,10 +84,15 @@ __device__ bool member(const EnumArgs &a, int y, K key) {
       return kk == key;
     }
     if (nd.hashed) return hash_find(s, nd.cap, key) >= 0;
-    if (nd.sorted)
-      return nd.spec.bits + nd.spec.hbits <= 64
-                 ? sorted_contains<u64>(s, nd.count, nd.spec, key)
-                 : sorted_contains<u128>(s, nd.count, nd.spec, key);
+    if (nd.sorted) {
+      const bool narrow = nd.spec.bits + nd.spec.hbits <= 64;
+      for (u64 lo = 0, hi = nd.split;; lo = hi, hi = nd.count) {
+        if (narrow ? sorted_contains<u64>(s, lo, hi, nd.spec, key)
+                   : sorted_contains<u128>(s, lo, hi, nd.spec, key))
+          return true;
+        if (hi == nd.count) return false;
+      }
+    }
     return false;
   }
   return false;

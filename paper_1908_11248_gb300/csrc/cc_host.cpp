@@ -426,6 +426,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   R->tables.assign(N, {});
   R->sizes.assign(N, 0);
   R->pairs.assign(N, 0);
+  R->runwise.assign(N, {});
   R->checks.clear();
   std::vector<bool> made(N, false);
   const int grid = cc::intro_grid(c->dev, block);
@@ -582,14 +583,15 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   };
   // sorts the records of src (scan bound *n_src, at most src_cap slots, *n of them nonempty,
   // at most cap) into a new buffer *out of cap records
-  auto sort_records = [&](int node, const cc::SortSpec &sp, const void *src, const u64 *n_src,
-                          u64 src_cap, const u64 *nn, u64 cap, void **out) -> int {
-    void *ba = A.alloc(std::max<u64>(1, cap) * rb);
-    void *bb = A.alloc(std::max<u64>(1, cap) * rb);
+  auto sort_records_of = [&](int kw, int node, const cc::SortSpec &sp, const void *src,
+                             const u64 *n_src, u64 src_cap, const u64 *nn, u64 cap,
+                             void **out) -> int {
+    void *ba = A.alloc(std::max<u64>(1, cap) * cc::slot_bytes(kw));
+    void *bb = A.alloc(std::max<u64>(1, cap) * cc::slot_bytes(kw));
     u64 *hist = arena_alloc<u64>(c, 256 * (size_t)cc::sort_grid(c->dev) + 512);
     // one-sweep scratch: tiles of the largest pass input (the scanned source or the buffers)
     cc::SweepScratch sw{};
-    sw.max_tiles = std::max(src_cap, cap) / cc::sweep_tile(R->kw) + 2;
+    sw.max_tiles = std::max(src_cap, cap) / cc::sweep_tile(kw) + 2;
     sw.ghist = arena_alloc<u64>(c, 256 * 16);
     sw.tile_ctr = arena_alloc<unsigned>(c, 16);
     sw.status = arena_alloc<u64>(c, 256 * sw.max_tiles);
@@ -607,8 +609,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     int which = 0;
     const bool sweep = R->opts.sort_sweep != 0;
     int r = timed(node, CC_K_SORT, sweep ? 2 + cc::sort_passes(sp) : 4 * cc::sort_passes(sp), [&] {
-      return cc::launch_sort_records(c->stream, c->dev, R->kw, sp, src, n_src, src_cap, nn, cap,
-                                     ba, bb, hist, &which, sweep ? &sw : nullptr);
+      return cc::launch_sort_records(c->stream, c->dev, kw, sp, src, n_src, src_cap, nn, cap, ba,
+                                     bb, hist, &which, sweep ? &sw : nullptr);
     });
     A.release(hist);
     A.release(sw.ghist);
@@ -618,9 +620,265 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     *out = which ? bb : ba;
     return r;
   };
+  auto sort_records = [&](int node, const cc::SortSpec &sp, const void *src, const u64 *n_src,
+                          u64 src_cap, const u64 *nn, u64 cap, void **out) -> int {
+    return sort_records_of(R->kw, node, sp, src, n_src, src_cap, nn, cap, out);
+  };
   // in planned mode, device word `w` must end at most `cap`
   auto check = [&](const u64 *w, u64 cap) {
     if (planned) R->checks.push_back({w, cap});
+  };
+
+  // what a node holds until it is done
+  struct Held {
+    Arena &a;
+    std::vector<void *> p;
+    ~Held() {
+      for (void *q : p) a.release(q);
+    }
+  };
+  // colours with the trials of a vertex side by side, made for the first introduce that asks
+  Held transposed{A, {}};
+  auto colours_by_vertex = [&](uint8_t **out) -> int {
+    if (transposed.p.empty()) {
+      void *t = A.alloc(std::max<size_t>(1, (size_t)R->trials * (size_t)n));
+      if (!t) return CC_ENOMEM;
+      transposed.p.push_back(t);
+      if (cc::launch_runs_colours(c->stream, c->dev, col.d_colors, n, R->trials, (uint8_t *)t))
+        return CC_ECUDA;
+      c->launches++;
+    }
+    *out = (uint8_t *)transposed.p[0];
+    return CC_OK;
+  };
+  // Introduce x (arguments a, child y) run by run, with its parent forget f when f >= 0
+  // (cc_runs.cu).  *taken: 1 if it made the table of x (or of f), 0 if the entry kernels have to;
+  // *total: the entries of x when an exact run has counted them here (else left alone).  Taken
+  // when there are trials enough for the pairs to be few beside the entries, when the child's
+  // entries come in whole runs of equal mappings, and when there is room.
+  auto run_wise = [&](int x, int y, int f, const cc::IntroArgs &a, int *taken, bool *counted,
+                      u64 *total) -> int {
+    *taken = 0;
+    *counted = false;
+    const NiceNode &nd = P.nodes[x], &ny = P.nodes[y];
+    const cc::NodeTable &ty = R->tables[y];
+    const int b_in = (int)ny.bag.size(), b_out = b_in + (f >= 0 ? 0 : 1), nb = R->L.nb;
+    const bool leaf = ny.type == 0;
+    if (R->trials < cc::kRunTrials || a.nnb != 1 || a.G.row_ptr != c->d_row_ptr ||
+        R->opts.sort_sweep != 1 || R->opts.fuse != 2 || n == 0 || b_out == 0 ||
+        (b_in + 1) * nb > 62 || R->L.k + R->L.tb > 24)
+      return CC_OK;
+    if (!leaf && (ty.hashed || ty.sort_n != b_in || ty.sort_hbits)) return CC_OK;
+    if (planned) {
+      const cc::RunSizes &r = plan->runwise[x];
+      if (plan->entries[x] <= kHashEntries || r.slots == 0 ||
+          plan->entries[x] < cc::kRunYield * r.slots)
+        return CC_OK;
+    }
+    Held held{A, {}};
+    bool short_of = false;
+    auto hold = [&](size_t bytes) {
+      void *q = A.alloc(std::max<size_t>(1, bytes));
+      if (q) held.p.push_back(q);
+      else short_of = true;
+      return q;
+    };
+    cc::RunsArgs r{};
+    r.G = a.G;
+    r.L = R->L;
+    r.trials = R->trials;
+    r.err = R->d_err;
+    r.leaf = leaf;
+    if (leaf) {
+      r.leaf_degF = df ? P.deg[ny.vertex] : 0;
+      r.leaf_ubit = 1u << ny.vertex;
+    } else {
+      r.child = desc(y);
+    }
+    r.ones = 1;
+    for (int z = y; z >= 0; z = P.nodes[z].child0)
+      if (P.nodes[z].type > 1) r.ones = 0;
+    r.b_in = b_in;
+    r.anchor = a.nb_slot[0];
+    r.p = a.p;
+    r.q = f >= 0 ? pos_in(nd.bag, P.nodes[f].vertex) : -1;
+    r.b_out = b_out;
+    r.degF = a.degF;
+    r.ubit = a.ubit;
+    uint8_t *colT = nullptr;
+    if (colours_by_vertex(&colT) != CC_OK) return CC_OK;
+    r.colT = colT;
+    // capacities: planned, or known as the exact run goes
+    u64 *w_slots = R->d_counters + 4 * N + x, *w_pairs = R->d_counters + 5 * N + x,
+        *w_more = R->d_counters + 6 * N + x, *w_runs = R->d_counters + 7 * N + x;
+    const u64 most_runs = leaf ? (u64)n : entries(y);
+    r.run_cap = leaf ? (u64)n
+                     : std::max<u64>(1, planned ? std::min(most_runs, room(plan->runwise[x].runs))
+                                                : most_runs);
+    r.n_runs = w_runs;
+    if (r.run_cap >= 1ull << 32) return CC_OK;
+    u64 *words = (u64 *)hold(4 * sizeof(u64));  // total, one, merged, -
+    u64 *scan = (u64 *)hold(cc::scan_scratch_words(c->dev) * sizeof(u64));
+    r.first = leaf ? nullptr : (u64 *)hold(r.run_cap * sizeof(u64));
+    r.packed = leaf ? nullptr : (unsigned *)hold(ty.cap * sizeof(unsigned));
+    r.deg = (unsigned *)hold(r.run_cap * sizeof(unsigned));
+    u64 *off = (u64 *)hold(r.run_cap * sizeof(u64));
+    r.off = off;
+    if (short_of) return CC_OK;
+    CUDA_OK(cudaMemsetAsync(words, 0, 4 * sizeof(u64), c->stream));
+    if (leaf) {
+      if (cc::launch_set_word(c->stream, w_runs, (u64)n)) return CC_ECUDA;
+    }
+    int rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, leaf ? 5 : 7, [&] {
+      const int e = cc::launch_runs_list(c->stream, c->dev, R->kw, r, blk);
+      return e ? e
+               : cc::launch_scan_u32(c->stream, c->dev, r.deg, r.run_cap, off, scan, r.n_runs,
+                                     w_slots);
+    });
+    if (rc) return rc;
+    check(w_runs, r.run_cap);
+    u64 slots = 0, pairs = 0;
+    if (!planned) {
+      rc = read_u64(c, w_slots, &slots);
+      if (rc) return rc;
+    } else {
+      slots = room(plan->runwise[x].slots);
+    }
+    r.pair_cap = std::max<u64>(1, slots);
+    if (r.pair_cap >= 1ull << 32) return CC_OK;
+    check(w_slots, r.pair_cap);
+    r.n_slots = w_slots;
+    r.recs = hold(r.pair_cap * 16);
+    r.prow = (unsigned *)hold(r.pair_cap * sizeof(unsigned));
+    r.pv = (int *)hold(r.pair_cap * sizeof(int));
+    if (short_of) return CC_OK;
+    r.n_pairs = w_pairs;
+    r.n_total = words;
+    r.cand = a.cand;
+    rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, 1,
+               [&] { return cc::launch_runs_pairs(c->stream, c->dev, R->kw, r); });
+    if (rc) return rc;
+    if (!planned) {
+      rc = read_u64(c, words, total);
+      if (!rc) rc = read_u64(c, w_pairs, &pairs);
+      if (rc) return rc;
+      // counted, but better (or only) done entry by entry
+      if ((f >= 0 && few(*total) && !order_handed_on(f)) || *total < cc::kRunYield * slots) {
+        *counted = f >= 0 && few(*total) && !order_handed_on(f);
+        CUDA_OK(cudaMemsetAsync(a.cand, 0, sizeof(u64), c->stream));
+        return CC_OK;
+      }
+    } else {
+      pairs = room(plan->runwise[x].pairs);
+      check(w_pairs, pairs);
+    }
+    void *sorted_pairs = nullptr;
+    cc::SortSpec fsp{};
+    if (f >= 0) {
+      fsp = forget_order(f);
+      cc::SortSpec ps = cc::rows_spec(b_out, nb);
+      for (int j = 0; j < b_out; ++j) ps.order[j] = fsp.order[j];
+      r.list_cap = std::max<u64>(1, pairs);
+      rc = sort_records_of(1, f, ps, r.recs, w_slots, r.pair_cap, w_pairs, r.list_cap,
+                           &sorted_pairs);
+      if (rc == CC_ENOMEM) return CC_OK;
+      if (rc) return rc;
+      held.p.push_back(sorted_pairs);
+      r.list = sorted_pairs;
+      r.n_list = w_pairs;
+      r.merge = 1;
+    } else {
+      r.list_cap = r.pair_cap;
+      r.list = r.recs;
+      r.n_list = w_slots;
+    }
+    const u64 windows = (r.list_cap + 31) / 32;
+    r.win_one = (unsigned *)hold(windows * sizeof(unsigned));
+    r.win_more = (unsigned *)hold(windows * sizeof(unsigned));
+    u64 *off_one = (u64 *)hold(windows * sizeof(u64));
+    u64 *off_more = (u64 *)hold(windows * sizeof(u64));
+    if (short_of) return CC_OK;
+    r.off_one = off_one;
+    r.off_more = off_more;
+    u64 *n_one = f >= 0 ? words + 1 : R->d_counters + x;
+    r.n_one = n_one;
+    r.n_more = w_more;
+    rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, 7, [&] {
+      int e = cc::launch_runs_windows(c->stream, c->dev, r);
+      if (!e) e = cc::launch_scan_u32(c->stream, c->dev, r.win_one, windows, off_one, scan, nullptr, n_one);
+      if (!e) e = cc::launch_scan_u32(c->stream, c->dev, r.win_more, windows, off_more, scan, nullptr, w_more);
+      return e;
+    });
+    if (rc) return rc;
+    u64 one = 0, more = 0, cap;
+    if (!planned) {
+      rc = read_u64(c, n_one, &one);
+      if (!rc) rc = read_u64(c, w_more, &more);
+      if (rc) return rc;
+      cap = std::max<u64>(1, one + more);
+    } else {
+      more = room(plan->runwise[x].more);
+      cap = room(plan->entries[f >= 0 ? f : x]);
+      check(w_more, more);
+      check(R->d_counters + x, room(plan->entries[x]));
+      if (f >= 0) check(R->d_counters + f, cap);
+    }
+    void *out = A.alloc(cap * rb);
+    if (!out) {
+      if (f < 0) CUDA_OK(cudaMemsetAsync(n_one, 0, sizeof(u64), c->stream));
+      return CC_OK;
+    }
+    r.out = TableDesc{out, cap, nullptr, 0};
+    r.side_cap = std::max<u64>(1, more);
+    r.side = f >= 0 ? hold(r.side_cap * rb) : nullptr;
+    if (short_of) {
+      A.release(out);
+      return CC_OK;
+    }
+    rc = timed(x, CC_K_INTRO_WRITE, 1,
+               [&] { return cc::launch_runs_write(c->stream, c->dev, R->kw, r); });
+    if (!rc && f >= 0) {
+      void *merged = r.side;
+      if (planned || more) {
+        void *srt = nullptr;
+        rc = sort_records(f, fsp, r.side, w_more, r.side_cap, w_more, r.side_cap, &srt);
+        if (!rc) {
+          held.p.push_back(srt);
+          rc = timed(f, CC_K_REDUCE, 3, [&] {
+            return cc::launch_reduce(c->stream, c->dev, R->kw, srt, w_more, r.side_cap, blk,
+                                     r.side, words + 2, &fsp, cc::sort_narrows(R->kw, fsp, 1));
+          });
+        }
+      }
+      if (!rc)
+        rc = timed(f, CC_K_REDUCE, 1, [&] {
+          return cc::launch_runs_append(c->stream, c->dev, R->kw, r, merged, words + 2,
+                                        R->d_counters + x, R->d_counters + f);
+        });
+    }
+    if (rc) {
+      A.release(out);
+      return rc == CC_ENOMEM ? CC_OK : rc;
+    }
+    const int z = f >= 0 ? f : x;
+    R->tables[z] = {out, cap, 0, true};
+    cc::NodeTable &t = R->tables[z];
+    if (f >= 0) {
+      t.sort_n = b_out;
+      for (int j = 0; j < b_out; ++j) t.sort_slots[j] = fsp.order[j];
+      t.regions = true;
+    } else {  // the child's order, then the new vertex
+      const int m = leaf ? 1 : b_in;
+      int *so = ty.regions ? t.cluster_slots : t.sort_slots;
+      for (int j = 0; j < m; ++j) {
+        const int sl = leaf ? 0 : ty.sort_slots[j];
+        so[j] = sl + (sl >= a.p ? 1 : 0);
+      }
+      so[m] = a.p;
+      (ty.regions ? t.cluster_n : t.sort_n) = m + 1;
+    }
+    *taken = 1;
+    return CC_OK;
   };
 
   for (int x = 0; x < N; ++x) {
@@ -722,7 +980,26 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       void *heavy_mem = nullptr;
       SortedGuard heavy_guard{A, heavy_mem};
       u64 total = 0, cand = 0;
-      if (!planned) {
+      bool counted = false;
+      {
+        const int f = nd.parent >= 0 && P.nodes[nd.parent].type == 2 ? nd.parent : -1;
+        int taken = 0;
+        rc = x1 >= 0 ? CC_OK : run_wise(x, y, f, a, &taken, &counted, &total);
+        if (rc) return rc;
+        if (taken) {
+          release_child(y);
+          if (f >= 0) made[f] = true;
+          if (!planned) {
+            rc = read_u64(c, R->d_counters + x, &R->sizes[x]);
+            if (!rc && f >= 0) rc = read_u64(c, R->d_counters + f, &R->sizes[f]);
+            if (rc) return rc;
+          }
+          if (f == N - 1) break;
+          continue;
+        }
+        if (counted) R->sizes[x] = total;
+      }
+      if (!planned && !counted) {
         rc = timed(x, CC_K_INTRO_COUNT, 2, [&] {
           return cc::launch_intro_blk(c->stream, c->dev, R->kw, 0, grouped, block, a, blk);
         });
@@ -978,7 +1255,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       // both are), else the one the parent likes best
       auto sorted_full = [&](int v) {
         const cc::NodeTable &t = R->tables[v];
-        return !t.hashed && t.sort_n == b && t.sort_hbits == 0;
+        return !t.hashed && t.sort_n == b && t.sort_hbits == 0 && !t.regions;
       };
       cc::SortSpec sp = forget_order(x);
       const int lead = sorted_full(z) ? z : sorted_full(y) ? y : -1;
@@ -988,13 +1265,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       sp.full = 0;
       sp.trial = 1;
       sp.bits = b * R->L.nb + R->L.tb;
-      struct Held {  // what this node holds until it is done
-        Arena &a;
-        std::vector<void *> p;
-        ~Held() {
-          for (void *q : p) a.release(q);
-        }
-      } held{A, {}};
+      Held held{A, {}};
       auto in_order = [&](int v, TableDesc *t) -> int {
         const cc::NodeTable &ty = R->tables[v];
         bool as_is = sorted_full(v);
@@ -1122,7 +1393,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
 int finish_run(Ctx *c, Run *R) {
   const int N = (int)R->sizes.size();
   int herr = 0;
-  std::vector<u64> words(4 * (size_t)N);
+  std::vector<u64> words(cc::kWords * (size_t)N);
   CUDA_OK(cudaMemcpyAsync(&herr, R->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_OK(cudaMemcpyAsync(words.data(), R->d_counters, words.size() * sizeof(u64),
                           cudaMemcpyDeviceToHost, c->stream));
@@ -1130,6 +1401,8 @@ int finish_run(Ctx *c, Run *R) {
   for (int x = 0; x < N; ++x) {
     R->sizes[x] = words[x];
     if (words[2 * N + x]) R->pairs[x] = words[2 * N + x];
+    if (words[4 * N + x])
+      R->runwise[x] = {words[4 * N + x], words[5 * N + x], words[6 * N + x], words[7 * N + x]};
   }
   for (auto &t : R->timings)
     if (t.kind == CC_K_INTRO_COUNT || t.kind == CC_K_INTRO_WRITE || t.kind == CC_K_INTRO_FUSED ||
@@ -1194,6 +1467,8 @@ int enumerate_run(Ctx *c, Run *R, uint64_t limit, int32_t *h_out, uint64_t *n_ou
     e.count = R->sizes[x];
     e.hashed = t.hashed;
     e.sorted = !t.hashed && t.sort_n == (int)nd.bag.size() && nd.type != 0;
+    // (in two regions: the entries that shared their mapping come second)
+    e.split = t.regions ? R->sizes[nd.child0] - R->runwise[nd.child0].more : e.count;
     if (e.sorted) {
       e.spec.L = R->L;
       e.spec.b = e.b;
@@ -1597,7 +1872,7 @@ int init_run(Ctx *c, int32_t pid, const cc::Coloring &col, int32_t cid, const cc
   const int N = (int)P.nodes.size();
   Arena &A = active_arena(c);
   R->home = &A == &c->arena ? nullptr : &A;
-  R->d_counters = arena_alloc<u64>(c, 4 * (size_t)N);
+  R->d_counters = arena_alloc<u64>(c, cc::kWords * (size_t)N);
   R->d_exists = arena_alloc<unsigned>(c, col.trials);
   R->d_count = arena_alloc<u64>(c, col.trials);
   R->d_err = arena_alloc<int>(c, 1);
@@ -1646,7 +1921,7 @@ int reset_run(Ctx *c, Run *R, int N) {
     cudaEventDestroy(t.stop);
   }
   R->timings.clear();
-  CUDA_OK(cudaMemsetAsync(R->d_counters, 0, 4 * (size_t)N * sizeof(u64), c->stream));
+  CUDA_OK(cudaMemsetAsync(R->d_counters, 0, cc::kWords * (size_t)N * sizeof(u64), c->stream));
   CUDA_OK(cudaMemsetAsync(R->d_exists, 0, R->trials * sizeof(unsigned), c->stream));
   CUDA_OK(cudaMemsetAsync(R->d_count, 0, R->trials * sizeof(u64), c->stream));
   return CC_OK;
@@ -1658,9 +1933,15 @@ void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t
   const size_t N = R->sizes.size();
   plan.entries.resize(N, 0);
   plan.pairs.resize(N, 0);
+  plan.runwise.resize(N);
   for (size_t x = 0; x < N; ++x) {
     plan.entries[x] = std::max(plan.entries[x], R->sizes[x]);
     plan.pairs[x] = std::max(plan.pairs[x], R->pairs[x]);
+    if (x >= R->runwise.size()) continue;  // a run put together from parts
+    cc::RunSizes &p = plan.runwise[x];
+    const cc::RunSizes &r = R->runwise[x];
+    p = {std::max(p.slots, r.slots), std::max(p.pairs, r.pairs), std::max(p.more, r.more),
+         std::max(p.runs, r.runs)};
   }
   plan.peak_bytes = std::max(plan.peak_bytes, peak);
   plan.runs++;
@@ -1794,7 +2075,7 @@ int capture_graph(Ctx *c, const std::vector<Run *> &Rs,
     S->trials = R->trials;
     S->home = &gm.sub;
     S->planned = true;
-    S->d_counters = (u64 *)gm.sub.alloc(4 * N * sizeof(u64));
+    S->d_counters = (u64 *)gm.sub.alloc(cc::kWords * N * sizeof(u64));
     S->d_exists = (unsigned *)gm.sub.alloc(R->trials * sizeof(unsigned));
     S->d_count = (u64 *)gm.sub.alloc(R->trials * sizeof(u64));
     S->d_err = (int *)gm.sub.alloc(sizeof(int));
@@ -1869,6 +2150,7 @@ int replay_graph(Ctx *c, cc::GraphSet &gs, const std::vector<Run *> &Rs) {
                             cudaMemcpyDeviceToDevice, c->stream));
     R->sizes = S->sizes;
     R->pairs = S->pairs;
+    R->runwise = S->runwise;
     R->planned = true;
     R->graphed = true;
     R->tables.assign(S->sizes.size(), {});

@@ -123,6 +123,52 @@ struct JoinArgs {
   int *err;
 };
 
+// Introduce run by run (cc_runs.cu): pairs of a run of equal mappings of the child and a candidate.
+struct RunsArgs {
+  GraphDev G;
+  KeyLayout L;
+  int trials;
+  const uint8_t *colT;  // colours, the trials of a vertex side by side
+  // the child: dense and sorted by every slot, or (leaf) one run a host vertex, its trials
+  TableDesc child;
+  int leaf, leaf_degF;
+  uint32_t leaf_ubit;
+  int ones;                    // every count of the child is 1
+  unsigned long long *n_runs;  // (a leaf's: G.n)
+  unsigned long long run_cap;
+  unsigned long long *first;   // per run: its first entry
+  unsigned *packed;            // per entry: trial << k | colour set
+  // the introduced vertex
+  int b_in, anchor;            // child bag size, slot of its one bag neighbour
+  int p, q;                    // its slot in the new bag; the slot the parent forgets (-1: none)
+  int b_out;                   // slots left
+  int degF;
+  uint32_t ubit;
+  // pairs, in the order of the runs: a run's candidates are its anchor image's neighbours
+  unsigned *deg;                   // per run: candidates
+  const unsigned long long *off;   // exclusive sums of those
+  const unsigned long long *n_slots;
+  unsigned long long pair_cap;     // below 2^32
+  void *recs;                      // per pair: (mapping with a marker bit, slot | entries << 32)
+  unsigned *prow;                  // per pair slot: its run and its candidate
+  int *pv;
+  unsigned long long *n_pairs, *n_total, *cand;  // pairs that yield entries, those entries
+  // the pairs to write: as they are, or sorted by mapping (merge)
+  const void *list;
+  const unsigned long long *n_list;
+  unsigned long long list_cap;
+  int merge;
+  unsigned *win_one, *win_more;    // per 32 pairs: entries of pairs alone with their mapping, others
+  const unsigned long long *off_one, *off_more, *n_one, *n_more;
+  TableDesc out;
+  void *side;
+  unsigned long long side_cap;
+  int *err;
+};
+// fewest trials for it, and fewest entries a pair must yield on average
+constexpr int kRunTrials = 8;
+constexpr unsigned long long kRunYield = 2;
+
 struct RootArgs {
   KeyLayout L;
   TableDesc in;
@@ -261,6 +307,8 @@ int launch_wait_probe(cudaStream_t s, const unsigned long long *flag, unsigned p
 // v = slice (mod slices), other bits from base (null: all allowed)
 int launch_slice_mask(cudaStream_t s, const DevInfo &d, const uint32_t *base, int32_t n,
                       uint32_t ubit, int32_t slices, int32_t slice, uint32_t *out);
+// *word = value, in stream order
+int launch_set_word(cudaStream_t s, unsigned long long *word, unsigned long long value);
 int launch_deg8(cudaStream_t s, const DevInfo &d, const int32_t *row_ptr, int32_t n,
                 uint8_t *deg8);
 // Grouped introduce (child sorted by bag-neighbour images), warp by warp, for planned runs;
@@ -282,6 +330,17 @@ int launch_intro_group_warp(cudaStream_t s, const DevInfo &d, int kw, int mode,
 int launch_forget(cudaStream_t s, const DevInfo &d, int kw, int block, const ForgetArgs &a);
 int launch_join(cudaStream_t s, const DevInfo &d, int kw, int phase, int block,
                 const JoinArgs &a);  // phase 0 build, 1 count pairs, 2 write
+int launch_runs_colours(cudaStream_t s, const DevInfo &d, const uint8_t *colors, int n, int T,
+                        uint8_t *colT);
+// runs of the child (blk: 2 * sort_grid(d) words) and their candidate counts
+int launch_runs_list(cudaStream_t s, const DevInfo &d, int kw, const RunsArgs &a,
+                     unsigned long long *blk);
+int launch_runs_pairs(cudaStream_t s, const DevInfo &d, int kw, const RunsArgs &a);
+int launch_runs_windows(cudaStream_t s, const DevInfo &d, const RunsArgs &a);
+int launch_runs_write(cudaStream_t s, const DevInfo &d, int kw, const RunsArgs &a);
+int launch_runs_append(cudaStream_t s, const DevInfo &d, int kw, const RunsArgs &a,
+                       const void *merged, const unsigned long long *n_merged,
+                       unsigned long long *size_x, unsigned long long *size_f);
 int prepare_join_kernels();  // once per device, as prepare_sort_kernels
 // lists a's groups and finds their ranges in b (blk: 2 * sort_grid(d) words)
 int launch_join_match(cudaStream_t s, const DevInfo &d, int kw, const JoinGroupArgs &a,
@@ -308,6 +367,7 @@ struct EnumNode {
   const void *slots;      // stored table (leaf: indexed by trial * n + v)
   unsigned long long cap, count;
   int hashed, sorted;
+  unsigned long long split;  // a sorted table in two regions: entries of the first (else count)
   SortSpec spec;          // order of a sorted table
 };
 

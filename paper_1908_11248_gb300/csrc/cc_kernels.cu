@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(256, 4) intro_heavy_kernel(IntroArgs a) {
 
 // ---- grouped introduce, warp by warp (planned capacities) -----------------------------------
 // The child comes in runs of equal images of u's bag neighbours (sorted or clustered by them).
-// Each warp takes a contiguous range of windows of 32 consecutive entries.  The first entry of
+// Each warp takes stretches of windows of 32 consecutive entries.  The first entry of
 // every run in a window leads: the warp walks the leads' anchor lists, laid end to end, 32
 // candidates at a time, keeps those adjacent to every bag neighbour's image (and passing the
 // degree filter and the allowed mappings) in a per-warp buffer, and every entry of the run then
@@ -694,8 +694,14 @@ __global__ void __launch_bounds__(256, 4) intro_heavy_kernel(IntroArgs a) {
 // and every chain of a window in sequence; end to end, a step's 32 chains belong to several
 // leads.  The closing introduce of a 4-cycle (one colouring of a
 // Barabasi-Albert graph, n = 200 000, m = 5; 27 million entries, 249 million candidates): 15.3 to
-// 10.8 ms; the three of the 2x4 grid with 13 colourings (n = 4999, m = 4): 1.47 to 1.00 ms.
+// 10.8 ms (and 5.1 with the windows spread, kGroupStretch); the three of the 2x4 grid with 13 colourings (n = 4999, m = 4): 1.47 to 1.00 ms.
 constexpr int kGroupCap = 256;  // candidate-list buffer per warp (two of them)
+// Consecutive windows a warp takes before it goes on elsewhere: long enough to carry lists, short
+// enough that a stretch of costly runs (a hub's; the region of mappings that several runs led to,
+// cc_runs.cu) is spread over the warps.  One range a warp instead: 28.6 ms for the chained
+// introduce of the 3x3 grid (Erdos-Renyi, n = 100 000, 32 colourings), 12.7 in stretches;
+// the 4-cycle's closing introduce (Barabasi-Albert, n = 200 000) 10.8 against 5.1.
+constexpr u64 kGroupStretch = 8;
 
 // true if v is in the increasing list col[lo, hi)
 __device__ __forceinline__ bool listed(const int32_t *col, int lo, int hi, int v) {
@@ -800,8 +806,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   const u64 wid = (u64)blockIdx.x * (blockDim.x / 32) + wib;
   const u64 bound = warp_run_failed(a.err) ? 0 : table_bound<K>(a.in);
   const u64 width = a.win, mylane = lane < (int)width ? (u64)lane : bound;
-  const u64 nwin = (bound + width - 1) / width, per = (nwin + warps - 1) / warps;
-  const u64 w0 = min(nwin, wid * per), w1 = min(nwin, w0 + per);
+  const u64 nwin = (bound + width - 1) / width;
   const int q = MODE == 2 ? a.q : a.proj_q;
   const int vsh = intro_vshift(a.L, a.p, q);
   const u64 n = (u64)a.G.n;
@@ -816,15 +821,18 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   // the next window's records are loaded while the current one is processed
   K nkey = 0;
   u64 nc_ = 0;
-  if (w0 < w1 && w0 * width + mylane < bound) load_slot(in, w0 * width + mylane, nkey, nc_);
-  for (u64 win = w0; win < w1; ++win) {
+  const u64 w0 = wid * kGroupStretch;
+  if (w0 < nwin && w0 * width + mylane < bound) load_slot(in, w0 * width + mylane, nkey, nc_);
+  for (u64 win = w0, follow; win < nwin; win = follow) {
     const K key = nkey;
     const u64 c = nc_;
+    follow = win + 1;
+    if (follow % kGroupStretch == 0) follow += (warps - 1) * kGroupStretch;
     {
-      const u64 i2 = (win + 1) * width + mylane;
+      const u64 i2 = follow * width + mylane;
       nkey = 0;
       nc_ = 0;
-      if (win + 1 < w1 && i2 < bound) load_slot(in, i2, nkey, nc_);
+      if (follow < nwin && i2 < bound) load_slot(in, i2, nkey, nc_);
     }
     const u64 tup = key != 0 ? nb_tuple(key, a) : ~0ull;
     const u64 up = __shfl_up_sync(0xffffffffu, tup, 1);
@@ -1100,6 +1108,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
       }
       cl = -1;  // no list to carry
     }
+    if (follow != win + 1) cl = -1;  // the next window is elsewhere
     __syncwarp();  // the buffers are rewritten by the next window
   }
   if (MODE == 1 && cfill < chunk)
@@ -1366,6 +1375,13 @@ __global__ void slice_mask_kernel(const uint32_t *base, int32_t n, uint32_t ubit
     const uint32_t m = base ? base[v] : 0xFFFFFFFFu;
     out[v] = v % slices == slice ? m : (m & ~ubit);
   }
+}
+
+__global__ void set_word_kernel(u64 *word, u64 value) { *word = value; }
+
+int launch_set_word(cudaStream_t s, unsigned long long *word, unsigned long long value) {
+  set_word_kernel<<<1, 1, 0, s>>>(word, value);
+  return (int)cudaGetLastError();
 }
 
 int launch_slice_mask(cudaStream_t s, const DevInfo &d, const uint32_t *base, int32_t n,

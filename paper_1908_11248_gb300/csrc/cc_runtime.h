@@ -151,6 +151,8 @@ struct NodeTable {
   // a bucketed order (sort_hbits > 0, see SortSpec): runs of equal images of the first m order
   // slots are contiguous only for m >= sort_min
   int sort_min = 0, sort_hbits = 0, sort_hslots = 0;
+  // sorted in two regions one after the other; every run of equal images lies in one of them
+  bool regions = false;
   // a dense table whose entries come in runs of equal images of these slots, except where an
   // append chunk or a kernel's tile ends (written in the order of a child sorted or clustered
   // by them); cluster_n == 0: no known clustering
@@ -160,10 +162,17 @@ struct NodeTable {
   unsigned long long *bound = nullptr;
 };
 
+// What an introduce taken run by run (cc_runs.cu) met: (run, candidate) pairs, those that yield
+// entries, entries of pairs that share their mapping, runs.
+struct RunSizes {
+  u64 slots = 0, pairs = 0, more = 0, runs = 0;
+};
+
 // Capacities learned from exact runs of one (pattern, graph, trials, colours, options): the
 // largest table sizes and join pair counts seen, per node.
 struct Plan {
   std::vector<u64> entries, pairs;
+  std::vector<RunSizes> runwise;  // of introduces taken run by run
   size_t peak_bytes = 0;  // largest arena use of a run beyond what it started with
   int runs = 0;
   size_t refused = 0;  // a served run of this key ran out of memory in a range this large
@@ -176,6 +185,8 @@ struct Timing {
   u64 candidates;
 };
 
+constexpr int kWords = 8;  // counter words a node
+
 struct Run {
   int32_t pattern = -1, coloring = -1;
   std::vector<Timing> timings;
@@ -184,11 +195,12 @@ struct Run {
   int kw = 1;
   int32_t trials = 0;
   std::vector<NodeTable> tables;
-  // per node, four words each: entries, chunk cursor, join pairs, candidates examined
+  // per node, kWords words: entries, chunk cursor, join pairs, candidates examined, RunSizes
   u64 *d_counters = nullptr;
   unsigned *d_exists = nullptr;
   u64 *d_count = nullptr;
   std::vector<u64> sizes, pairs;
+  std::vector<RunSizes> runwise;
   std::vector<std::pair<const u64 *, u64>> checks;  // planned runs: device word <= capacity
   bool retained = false;
   bool planned = false;

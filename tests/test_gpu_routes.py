@@ -170,3 +170,49 @@ def test_hubs(ctx, trials):
     g = synth.csr_from_edges(at, np.array(edges))
     for pat in (synth.path_pattern(4), synth.star_pattern(4)):
         check_tables(ctx, g, pat, oracle.colors(at, trials, 5, seed=2), 5)
+
+
+def hub_graph(n, seed):
+    return synth.barabasi_albert(n, 4, seed)
+
+
+# introduces run by run need 8 trials, more than 2^18 entries (planned) and two entries a pair: one
+# trial too few, the fewest, several bytes of trials; leaf, introduce and forget children; pairs
+# that share their mapping (hubs); 64- and 128-bit keys; a vertex forgotten as it comes; joins above
+@pytest.mark.parametrize("pat,n,hubs,trials,spare", [
+    (("grid", 2, 4), 1500, 1, 7, 0), (("grid", 2, 4), 1500, 1, 8, 0),
+    (("grid", 2, 4), 400, 1, 33, 1), (("grid", 3, 3), 2500, 0, 9, 0),
+    (("grid", 3, 3), 70_000, 0, 8, 0), (("cycle", 4), 4000, 1, 16, 2),
+    (("path", 5), 9000, 0, 12, 0), (("star", 5), 3000, 0, 40, 0), (("A",), 1200, 0, 10, 0),
+    (("ktree", 7, 2, 5), 700, 1, 9, 0)])
+def test_run_wise_introduces(ctx, pat, n, hubs, trials, spare):
+    p = synth.make_pattern(pat)
+    k = p[0] + spare
+    deg = 2.0 if n > 50_000 else 6.0
+    g = hub_graph(n, 3) if hubs else synth.erdos_renyi(n, deg / n, 3)
+    check_tables(ctx, g, p, oracle.colors(n, trials, k, seed=5), k)
+
+
+def test_run_wise_masks_filter_and_enumeration(ctx):
+    """Allowed mappings and no degree filter; the rows reconstructed through tables in two
+    regions."""
+    n, T = 1500, 24
+    g = hub_graph(n, 5)
+    pat = synth.cycle_pattern(4)
+    z = oracle.colors(n, T, 4, seed=7)
+    allow = np.random.default_rng(2).integers(0, 16, n).astype(np.uint32)
+    cc.cc_load_graph(ctx.h, *g)
+    cid = cc.cc_set_colors(ctx.h, z, 4)
+    for masks, df in ((None, 1), (None, 0), (allow, 1)):
+        ref = oracle.run_dp(g, pat, z, 4, degree_filter=bool(df), allow=masks)
+        pid = cc.cc_load_pattern_masked(ctx.h, *pat, masks) if masks is not None else \
+            cc.cc_load_pattern(ctx.h, *pat)
+        N, _ = cc.cc_pattern_info(ctx.h, pid)
+        want, total, _ = ref.enumerate(50_000)
+        for rep in range(2):
+            run = cc.cc_run_dp(ctx.h, pid, cid, cc.cc_default_opts(retain=1, degree_filter=df))
+            assert np.array_equal(cc.cc_count(ctx.h, run, T), ref.count)
+            assert np.array_equal(cc.cc_table_stats(ctx.h, run, N)[0], ref.node_sizes.sum(axis=0))
+            rows, got = cc.cc_enumerate(ctx.h, run, 50_000, 4)
+            assert got == total and np.array_equal(rows, want[:50_000])
+            cc.cc_release(ctx.h, run)
