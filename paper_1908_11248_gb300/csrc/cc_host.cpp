@@ -532,6 +532,24 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     *nnb2 = k2;
     return x2;
   };
+  // true if a vertex forgotten below y has all its F-neighbours among those of u in y's bag
+  // (IntroArgs::twin; with allowed mappings or the distance bound a candidate of u need not be
+  // one of that vertex)
+  auto has_twin = [&](int y, int u) {
+    uint32_t below = 0, bag = 0;
+    std::vector<int> todo{y};
+    while (!todo.empty()) {
+      const NiceNode &z = P.nodes[todo.back()];
+      todo.pop_back();
+      if (z.type == 2) below |= 1u << z.vertex;
+      if (z.child0 >= 0) todo.push_back(z.child0);
+      if (z.child1 >= 0) todo.push_back(z.child1);
+    }
+    for (int w : P.nodes[y].bag) bag |= 1u << w;
+    for (int w = 0; w < P.nF; ++w)
+      if ((below >> w & 1u) && !(bag >> w & 1u) && !(P.adj[w] & ~(P.adj[u] & bag))) return true;
+    return false;
+  };
   std::vector<int> chain_from(N, -1);  // x2 -> the x1 it runs together with
   // Few entries (default sort schedule): an introduce adds them into its forget's hash table and
   // a grouped introduce takes its child unsorted, because the dozen launches of a sort and its
@@ -951,6 +969,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       a.cand = R->d_counters + 3 * N + x;  // candidates examined (count pass, or planned)
       a.proj_q = -1;
       a.q = -1;
+      a.trials = R->trials;
       // several bag neighbours: the child must come in runs of equal images of those slots so
       // that a run shares one candidate list; sort it unless its order already starts with them
       const int grouped = R->opts.group && a.nnb >= 2 && a.nnb * R->L.nb <= 64;
@@ -971,6 +990,20 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                           R->d_counters + y, m, &sorted);
         if (rc) return rc;
         a.in = TableDesc{sorted, std::max<u64>(1, m), R->d_counters + y, 0};
+      }
+      {
+        const cc::NodeTable &ty = R->tables[y];
+        a.twin = grouped && !sorted && !ty.hashed && ty.sort_n == a.b_in && ty.sort_hbits == 0 &&
+                 !P.d_allow && !R->opts.distance_prune && has_twin(y, nd.vertex);
+      }
+      a.cols = col.d_colors;
+      a.ct = (u64)n;
+      a.cv = 1;
+      uint8_t *colT = nullptr;
+      if (planned && (grouped || x1 >= 0) && R->trials > 1 && colours_by_vertex(&colT) == CC_OK) {
+        a.cols = colT;
+        a.ct = 1;
+        a.cv = (u64)R->trials;
       }
       struct SortedGuard {
         Arena &a;
@@ -1056,14 +1089,15 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         // vertex's neighbours let entries whose runs have no upper candidate count their lower
         // extensions without walking the adjacency
         u64 *hist = nullptr;
-        if (x1 >= 0 && a.c_nnb == 1 && R->L.k <= 16 && c->max_deg < 65536)
+        if (x1 >= 0 && a.c_nnb == 1 && R->L.k <= 16 && c->max_deg < 65536 &&
+            a.cv == (u64)R->trials)
           hist = arena_alloc<u64>(c, (size_t)R->trials * (size_t)n * 4);
         a.c_hist = hist;
         int r = timed(x, x1 >= 0 ? CC_K_INTRO_CHAIN : CC_K_INTRO_WRITE,
                       hist || a.heavy_cap ? 2 : 1, [&] {
           if (hist) {
-            const int h = cc::launch_nb_colour_hist(c->stream, c->dev, a.G, R->trials, a.c_degF,
-                                                    a.c_ubit, hist, a.cand);
+            const int h = cc::launch_nb_colour_hist(c->stream, c->dev, a.G, a.cols, R->trials,
+                                                    a.c_degF, a.c_ubit, hist, a.cand);
             if (h) return h;
           }
           return x1 >= 0 ? cc::launch_intro_chain(c->stream, c->dev, R->kw, a)

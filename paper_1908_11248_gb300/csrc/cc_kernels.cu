@@ -418,6 +418,16 @@ __device__ __forceinline__ u128 shfl_key(u128 v, int src) {
   return ((u128)hi << 64) | (u128)lo;
 }
 
+// the neighbour lane's key (lane 0's, or lane 31's, is its own)
+__device__ __forceinline__ u64 shfl_up_key(u64 v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ u64 shfl_down_key(u64 v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ u128 shfl_up_key(u128 v) {
+  return ((u128)shfl_up_key((u64)(v >> 64)) << 64) | shfl_up_key((u64)v);
+}
+__device__ __forceinline__ u128 shfl_down_key(u128 v) {
+  return ((u128)shfl_down_key((u64)(v >> 64)) << 64) | shfl_down_key((u64)v);
+}
+
 // The output key of an introduce for a child entry `key` with the new vertex's field zero: the
 // vertex inserted at slot p, then slot q removed when the parent forget's projection is applied
 // (q < 0: none; q == p: the new vertex is forgotten at once, so only its colour enters the key).
@@ -715,48 +725,57 @@ __device__ __forceinline__ bool listed(const int32_t *col, int lo, int hi, int v
   return false;
 }
 
-// Per host vertex w (one thread) and every trial: counts of w's neighbours by colour, four
-// colours to a 64-bit word (16-bit fields), for the chained introduce's counted entries.
-__global__ void __launch_bounds__(256) nb_colour_hist_kernel(GraphDev G, int trials, int degF,
-                                                             uint32_t ubit, u64 *hist,
-                                                             u64 *cand) {
+// Per host vertex w (one warp) and trial (a lane): counts of w's neighbours by colour, four
+// colours to a 64-bit word (16-bit fields), for the chained introduce's counted entries.  A
+// neighbour's colours of 32 trials are one sector, and so are the counts that the entries of a
+// run (one w, one entry or more a trial) read.
+__global__ void __launch_bounds__(256) nb_colour_hist_kernel(GraphDev G, const uint8_t *colT,
+                                                             int trials, int degF, uint32_t ubit,
+                                                             u64 *hist, u64 *cand) {
   u64 seen = 0;
-  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < G.n; w += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  for (int w = blockIdx.x * 8 + (threadIdx.x >> 5); w < G.n; w += gridDim.x * 8) {
     const int r0 = G.row_ptr[w], r1 = G.row_ptr[w + 1];
-    for (int t = 0; t < trials; ++t) {
-      const uint8_t *col = G.colors + (u64)t * (u64)G.n;
+    for (int t = lane; t < trials; t += 32) {
       u64 h0 = 0, h1 = 0, h2 = 0, h3 = 0;
       for (int r = r0; r < r1; ++r) {
         const int v = __ldg(G.col + r);
         if (degF && G.deg8[v] < degF) continue;
         if (G.allow && !(G.allow[v] & ubit)) continue;
-        const int c = col[v];
+        const int c = colT[(u64)v * (u64)trials + (u64)t];
         const u64 one = 1ull << (16 * (c & 3));
         h0 += (c >> 2) == 0 ? one : 0;
         h1 += (c >> 2) == 1 ? one : 0;
         h2 += (c >> 2) == 2 ? one : 0;
         h3 += (c >> 2) == 3 ? one : 0;
       }
-      u64 *o = hist + ((u64)t * (u64)G.n + (u64)w) * 4;
+      u64 *o = hist + ((u64)w * (u64)trials + (u64)t) * 4;
       reinterpret_cast<ulonglong2 *>(o)[0] = make_ulonglong2(h0, h1);
       reinterpret_cast<ulonglong2 *>(o)[1] = make_ulonglong2(h2, h3);
     }
-    seen += (u64)(r1 - r0) * (u64)trials;
+    if (lane == 0) seen += (u64)(r1 - r0) * (u64)trials;
   }
   for (int o = 16; o > 0; o >>= 1) seen += __shfl_down_sync(0xffffffffu, seen, o);
   if ((threadIdx.x & 31) == 0 && seen) atomicAdd(cand, seen);
 }
 
-// x1's extensions of an entry with colour set cm from the colour counts of its anchor image
-__device__ __forceinline__ u64 hist_count(const u64 *h, uint32_t cm, int k) {
-  const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2 *>(h));
-  const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2 *>(h) + 1);
-  const u64 w[4] = {a.x, a.y, b.x, b.y};
+// x1's extensions of an entry from the colour counts of its anchor's image (slot `slot`): the sum
+// of the 16-bit fields of the colours outside its set (at most a degree, below 65536)
+template <typename K>
+__device__ __forceinline__ u64 chain_counted(const IntroArgs &a, K key, int slot) {
+  const u64 w = (u64)key_slot(key, a.L, slot);
+  const u64 *h = a.c_hist + (w * (u64)a.trials + (u64)key_trial(key, a.L)) * 4;
+  const ulonglong2 lo = __ldg(reinterpret_cast<const ulonglong2 *>(h));
+  const ulonglong2 hi = __ldg(reinterpret_cast<const ulonglong2 *>(h) + 1);
+  const u64 word[4] = {lo.x, lo.y, hi.x, hi.y};
+  const uint32_t free = ~key_mask(key, a.L) & ((1u << a.L.k) - 1u);
   u64 sum = 0;
 #pragma unroll
-  for (int c = 0; c < 16; ++c)
-    if (c < k && !((cm >> c) & 1u)) sum += (w[c >> 2] >> (16 * (c & 3))) & 0xFFFFull;
-  return sum;
+  for (int q = 0; q < 4; ++q) {  // four bits of `free` spread over the four fields
+    const u64 bits = ((u64)(free >> (4 * q) & 15u) * 0x0000200040008001ull) & 0x0001000100010001ull;
+    sum += word[q] & bits * 0xFFFFull;
+  }
+  return sum * 0x0001000100010001ull >> 48;
 }
 
 // x1's candidates of one y entry (chained introduce): the adjacency list of the bag neighbour
@@ -809,7 +828,6 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   const u64 nwin = (bound + width - 1) / width;
   const int q = MODE == 2 ? a.q : a.proj_q;
   const int vsh = intro_vshift(a.L, a.p, q);
-  const u64 n = (u64)a.G.n;
   const u64 chunk = a.chunk;
   u64 cbase = 0, cfill = chunk;
   u64 produced = 0, fresh = 0, examined = 0, produced1 = 0;
@@ -835,8 +853,40 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
       if (follow < nwin && i2 < bound) load_slot(in, i2, nkey, nc_);
     }
     const u64 tup = key != 0 ? nb_tuple(key, a) : ~0ull;
-    const u64 up = __shfl_up_sync(0xffffffffu, tup, 1);
-    const bool lead = key != 0 && (lane == 0 ? (cl < 0 || tup != ctup) : up != tup);
+    // entries that can have a candidate (see IntroArgs::twin), and those that start a list
+    bool live = key != 0;
+    if (a.twin) {
+      const u64 i = win * width + lane;
+      const K g = key >> a.L.k;
+      K gp = shfl_up_key(g), gn = shfl_down_key(g);
+      K other;
+      u64 ignored;
+      if (lane == 0) {
+        gp = ~(K)0;
+        if (key != 0 && i > 0) {
+          load_slot(in, i - 1, other, ignored);
+          gp = other >> a.L.k;
+        }
+      }
+      if (lane == (int)width - 1) {
+        gn = ~(K)0;
+        if (key != 0 && i + 1 < bound) {
+          load_slot(in, i + 1, other, ignored);
+          gn = other >> a.L.k;
+        }
+      }
+      live = live && (g == gp || g == gn);
+    }
+    const unsigned lives = __ballot_sync(0xffffffffu, live);
+    if (!lives && (!CHAIN || a.c_hist)) {  // nothing to extend: x1's entries are only counted
+      if (CHAIN && key != 0)
+        produced1 += chain_counted(a, key, a.c_nb_slot[0]);
+      if (follow != win + 1) cl = -1;
+      continue;
+    }
+    const int before = lives & lt ? 31 - __clz(lives & lt) : 0;
+    const u64 up = __shfl_sync(0xffffffffu, tup, before);
+    const bool lead = live && (lives & lt ? up != tup : cl < 0 || tup != ctup);
     const unsigned leads = __ballot_sync(0xffffffffu, lead);
     const int nbuf = cb ^ 1;  // the new lists go where the carried one is not
     int *nb_base = bufs + nbuf * kGroupCap;
@@ -869,9 +919,10 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
       }
       // a run of one entry needs no candidate whose colour that entry already has (the run of
       // the window's last entry may go on in the next window)
-      const bool single = lead && lane + 1 < (int)width && (leads >> (lane + 1) & 1u);
+      const unsigned after = lives & ~(lt | 1u << lane);
+      const bool single = lead && after && (leads & after & (~after + 1u));
       const uint32_t lcm = single ? key_mask(key, a.L) : 0;
-      const u64 lrow = key != 0 ? (u64)key_trial(key, a.L) * n : 0;
+      const u64 lrow = key != 0 ? (u64)key_trial(key, a.L) * a.ct : 0;
       int incl = d1;
       for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -905,7 +956,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         int v = 0;
         if (j < total) {
           v = __ldg(a.G.col + ers + (j - eex));
-          ok = !ecm || !((ecm >> a.G.colors[erow + (u64)v]) & 1u);
+          ok = !ecm || !((ecm >> a.cols[erow + (u64)v * a.cv]) & 1u);
           if (ok) ok = (a.degF == 0 || a.G.deg8[v] >= a.degF) &&
                        (!a.G.allow || (a.G.allow[v] & a.ubit));
           if (a.nnb > 2) {
@@ -945,11 +996,11 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         s0 = cs;
         n0 = cl < 0 ? 0 : cl;
       }
-      if (key == 0) n0 = 0;
+      if (!live) n0 = 0;
       int nmax = n0;
       for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
       const uint32_t cm = key_mask(key, a.L);
-      const u64 crow = key != 0 ? (u64)key_trial(key, a.L) * n : 0;
+      const u64 crow = key != 0 ? (u64)key_trial(key, a.L) * a.ct : 0;
       if constexpr (CHAIN) {
         // every x1 extension (entry, v1) of this entry is counted; those with a nonempty u2 list
         // are extended by it at once
@@ -959,13 +1010,11 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         // extend one of its x1 entries (the set only grows with v1's colour)
         int nv = 0;
         for (int r = 0; r < nmax; ++r)
-          if (r < n0 && !((cm >> a.G.colors[crow + (u64)lst[s0 + r]]) & 1u)) ++nv;
+          if (r < n0 && !((cm >> a.cols[crow + (u64)lst[s0 + r] * a.cv]) & 1u)) ++nv;
         if (a.c_hist && key != 0 && nv == 0) {
           // none: the entry's x1 extensions are only counted, from the colour counts of its
           // anchor image
-          const u64 w1 = (u64)key_slot(key, a.L, a.c_nb_slot[anc1]);
-          produced1 += hist_count(a.c_hist + ((u64)key_trial(key, a.L) * n + w1) * 4, cm,
-                                  a.L.k);
+          produced1 += chain_counted(a, key, a.c_nb_slot[anc1]);
           d1 = 0;
         }
         if (nv == 0) n0 = 0;  // no pair can be valid
@@ -982,7 +1031,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
           int v1 = 0, cv1 = 0;
           if (j < d1) {
             v1 = __ldg(a.G.col + r1 + j);
-            cv1 = a.G.colors[crow + (u64)v1];
+            cv1 = a.cols[crow + (u64)v1 * a.cv];
             ok1 = chain_ok(a, key, cm, v1, cv1, anc1);
           }
           produced1 += ok1 ? 1u : 0u;
@@ -997,7 +1046,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
             K okey = 0;
             if (pair && r < n0) {
               const int v = lst[s0 + r];
-              const int cv = a.G.colors[crow + (u64)v];
+              const int cv = a.cols[crow + (u64)v * a.cv];
               valid = !((cm1 >> cv) & 1u);
               if (valid) okey = intro_out(intro_base(k1, a.L, a.p, q), vsh, v, cv);
             }
@@ -1011,7 +1060,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         K okey = 0;
         if (r < n0) {
           const int v = lst[s0 + r];
-          const int cv = a.G.colors[crow + (u64)v];
+          const int cv = a.cols[crow + (u64)v * a.cv];
           valid = !((cm >> cv) & 1u);
           // most candidates of a closing step clash in colour: the output key is built only
           // for the valid ones
@@ -1026,8 +1075,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         cs = __shfl_sync(0xffffffffu, lstart, l);
         cl = __shfl_sync(0xffffffffu, llen, l);
       }
-      ctup = __shfl_sync(0xffffffffu, tup, (int)width - 1);
-      if (ctup == ~0ull) cl = -1;
+      if (lives) ctup = __shfl_sync(0xffffffffu, tup, 31 - __clz(lives));
     } else {  // entry by entry, every check in full
       int best = INT_MAX, rs = 0, anc = 0;
       if (key != 0)
@@ -1040,11 +1088,11 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
             anc = j;
           }
         }
-      const int nc = key != 0 ? best : 0;
+      const int nc = live ? best : 0;
       int nmax = nc;
       for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
       const uint32_t cm = key_mask(key, a.L);
-      const u64 crow = key != 0 ? (u64)key_trial(key, a.L) * n : 0;
+      const u64 crow = key != 0 ? (u64)key_trial(key, a.L) * a.ct : 0;
       if constexpr (CHAIN) {
         // every x1 extension, then every u2 candidate of the entry's own anchor list with all
         // of x2's checks
@@ -1062,7 +1110,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
           int v1 = 0, cv1 = 0;
           if (j < d1) {
             v1 = __ldg(a.G.col + r1 + j);
-            cv1 = a.G.colors[crow + (u64)v1];
+            cv1 = a.cols[crow + (u64)v1 * a.cv];
             ok1 = chain_ok(a, key, cm, v1, cv1, anc1);
           }
           produced1 += ok1 ? 1u : 0u;
@@ -1076,7 +1124,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
             K okey = 0;
             if (pair && r < nc) {
               const int v = __ldg(a.G.col + rs + r);
-              const int cv = a.G.colors[crow + (u64)v];
+              const int cv = a.cols[crow + (u64)v * a.cv];
               valid = !((cm1 >> cv) & 1u);
               if (valid && a.degF) valid = a.G.deg8[v] >= a.degF;
               if (valid && a.G.allow) valid = (a.G.allow[v] & a.ubit) != 0;
@@ -1096,7 +1144,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
         K okey = 0;
         if (j < nc) {
           const int v = __ldg(a.G.col + rs + j);
-          const int cv = a.G.colors[crow + (u64)v];
+          const int cv = a.cols[crow + (u64)v * a.cv];
           valid = !((cm >> cv) & 1u);
           if (valid && a.degF) valid = a.G.deg8[v] >= a.degF;
           if (valid && a.G.allow) valid = (a.G.allow[v] & a.ubit) != 0;
@@ -1409,11 +1457,11 @@ int launch_intro_group_warp(cudaStream_t s, const DevInfo &d, int kw, int mode,
   return (int)cudaGetLastError();
 }
 
-int launch_nb_colour_hist(cudaStream_t s, const DevInfo &d, const GraphDev &G, int trials,
-                          int degF, uint32_t ubit, unsigned long long *hist,
-                          unsigned long long *cand) {
-  const int grid = std::max(1, std::min(d.sms * 8, (G.n + 255) / 256));
-  nb_colour_hist_kernel<<<grid, 256, 0, s>>>(G, trials, degF, ubit, hist, cand);
+int launch_nb_colour_hist(cudaStream_t s, const DevInfo &d, const GraphDev &G,
+                          const uint8_t *colT, int trials, int degF, uint32_t ubit,
+                          unsigned long long *hist, unsigned long long *cand) {
+  const int grid = std::max(1, std::min(d.sms * 8, (G.n + 7) / 8));
+  nb_colour_hist_kernel<<<grid, 256, 0, s>>>(G, colT, trials, degF, ubit, hist, cand);
   return (int)cudaGetLastError();
 }
 

@@ -17,8 +17,8 @@
 // bytes each (trial and colour set) from L2.  What is left is the write of the result.
 // Introduce, sort and reduce of the first forget of the 3x3 grid (Erdos-Renyi, n = 100 000, degree
 // 10, 32 colourings; 221 million entries of 11 million pairs): 3.1 + 16.7 + 2.7 ms entry by entry,
-// 4.5 ms here.  Of the three big ones of the 2x4 grid (Barabasi-Albert, n = 20 000, 64 colourings;
-// 159, 154 and 90 million entries): 40 ms entry by entry, 13 here.
+// 4.4 ms here.  Of the three big ones of the 2x4 grid (Barabasi-Albert, n = 20 000, 64 colourings;
+// 159, 154 and 90 million entries): 40 ms entry by entry, 11 here.
 //
 // With fewer than kRunTrials trials, or fewer than kRunYield entries a pair, a pair's record is no
 // smaller than what it stands for, and the entry kernels take the node.
@@ -183,9 +183,10 @@ __global__ void __launch_bounds__(256) runs_pairs_kernel(RunsArgs a) {
         const uint8_t *cr = a.colT + r * (u64)T;
         for (int t = 0; t < T; ++t) cnt += cv[t] != cr[t];
       } else {
-        for (u64 e = e0; e < e1; ++e) {
+#pragma unroll 8
+        for (u64 e = e0; e < e1; ++e) {  // (unrolled: the loads of eight entries overlap)
           const uint32_t pk = __ldg(a.packed + e);
-          cnt += !((pk & cmask) >> cv[pk >> k] & 1u);
+          cnt += !((pk & cmask) >> __ldg(cv + (pk >> k)) & 1u);
         }
       }
     }
@@ -260,11 +261,13 @@ __global__ void __launch_bounds__(256) runs_windows_kernel(RunsArgs a) {
   }
 }
 
-// Writes the entries of the listed pairs: a warp takes 32 pairs, lays their runs end to end and
-// tests 32 entries a step; as the offsets are exact, its results are one stretch of the output
-// (and one of the side buffer).
+// Writes the entries of the listed pairs: a warp takes 32 pairs, and 32 entries of their runs a
+// step, of one run or (short runs) of several laid end to end; as the offsets are exact, its
+// results are one stretch of the output (and one of the side buffer).
+constexpr int kRunLong = 20;  // entries a run from which pairs are written one after the other
+
 template <typename K>
-__global__ void __launch_bounds__(256, 4) runs_write_kernel(RunsArgs a) {
+__global__ void __launch_bounds__(256, 5) runs_write_kernel(RunsArgs a) {
   const Slot<K> *in = reinterpret_cast<const Slot<K> *>(a.child.slots);
   Slot<K> *out = reinterpret_cast<Slot<K> *>(a.out.slots);
   Slot<K> *side = reinterpret_cast<Slot<K> *>(a.side);
@@ -310,27 +313,17 @@ __global__ void __launch_bounds__(256, 4) runs_write_kernel(RunsArgs a) {
     }
     const int excl = incl - len, total = __shfl_sync(0xffffffffu, incl, 31);
     u64 at = a.off_one[w], at2 = a.off_more[w];
-    for (int x0 = 0; x0 < total; x0 += 32) {
-      const int x = x0 + lane;
-      int lo = 0, hi = 31;  // owner: smallest lane with incl > x
-#pragma unroll
-      for (int step = 0; step < 5; ++step) {
-        const int mid = (lo + hi) >> 1;
-        const int y = __shfl_sync(0xffffffffu, incl, mid);
-        if (y > x) hi = mid;
-        else lo = mid + 1;
-      }
-      const u64 oe = __shfl_sync(0xffffffffu, e0, lo), ophi = __shfl_sync(0xffffffffu, phi, lo);
-      const int ox = __shfl_sync(0xffffffffu, excl, lo), ov = __shfl_sync(0xffffffffu, v, lo);
-      bool ok = false;
+    // one step: the lane's entry, if any, of a pair (its run's entries from oe on, or leaf vertex oe)
+    auto step = [&](bool have, u64 oe, int x, u64 ophi, int ov, bool mine) {
       uint32_t t = 0, m = 0;
+      bool ok = false;
       u64 e = 0;
-      if (x < total) {
+      if (have) {
         if (a.leaf) {
-          t = (uint32_t)(x - ox);
+          t = (uint32_t)x;
           m = 1u << a.colT[oe * (u64)T + t];
         } else {
-          e = oe + (u64)(x - ox);
+          e = oe + (u64)x;
           const uint32_t pk = __ldg(a.packed + e);
           t = pk >> k;
           m = pk & cmask;
@@ -339,7 +332,6 @@ __global__ void __launch_bounds__(256, 4) runs_write_kernel(RunsArgs a) {
         ok = !(m & c);
         m |= c;
       }
-      const bool mine = ones >> lo & 1u;
       const unsigned b1 = __ballot_sync(0xffffffffu, ok && mine);
       const unsigned b2 = __ballot_sync(0xffffffffu, ok && !mine);
       if (ok) {
@@ -356,6 +348,31 @@ __global__ void __launch_bounds__(256, 4) runs_write_kernel(RunsArgs a) {
       }
       at += __popc(b1);
       at2 += __popc(b2);
+    };
+    if (total >= 32 * kRunLong) {  // long runs: one pair after the other, 32 of its entries a step
+      for (unsigned todo = __ballot_sync(0xffffffffu, len > 0); todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const u64 oe = __shfl_sync(0xffffffffu, e0, l), ophi = __shfl_sync(0xffffffffu, phi, l);
+        const int ol = __shfl_sync(0xffffffffu, len, l), ov = __shfl_sync(0xffffffffu, v, l);
+        const bool mine = ones >> l & 1u;
+#pragma unroll 4
+        for (int x0 = 0; x0 < ol; x0 += 32) step(x0 + lane < ol, oe, x0 + lane, ophi, ov, mine);
+      }
+      continue;
+    }
+    for (int x0 = 0; x0 < total; x0 += 32) {  // short ones end to end
+      const int x = x0 + lane;
+      int lo = 0, hi = 31;  // owner: smallest lane with incl > x
+#pragma unroll
+      for (int i5 = 0; i5 < 5; ++i5) {
+        const int mid = (lo + hi) >> 1;
+        const int y = __shfl_sync(0xffffffffu, incl, mid);
+        if (y > x) hi = mid;
+        else lo = mid + 1;
+      }
+      const u64 oe = __shfl_sync(0xffffffffu, e0, lo), ophi = __shfl_sync(0xffffffffu, phi, lo);
+      const int ox = __shfl_sync(0xffffffffu, excl, lo), ov = __shfl_sync(0xffffffffu, v, lo);
+      step(x < total, oe, x - ox, ophi, ov, ones >> lo & 1u);
     }
   }
   if (full) atomicOr(a.err, kErrOverflow);
@@ -417,8 +434,8 @@ int launch_runs_windows(cudaStream_t s, const DevInfo &d, const RunsArgs &a) {
 }
 
 int launch_runs_write(cudaStream_t s, const DevInfo &d, int kw, const RunsArgs &a) {
-  if (kw == 1) runs_write_kernel<u64><<<sort_grid(d), 256, 0, s>>>(a);
-  else runs_write_kernel<u128><<<sort_grid(d), 256, 0, s>>>(a);
+  if (kw == 1) runs_write_kernel<u64><<<d.sms * 10, 256, 0, s>>>(a);
+  else runs_write_kernel<u128><<<d.sms * 10, 256, 0, s>>>(a);
   return (int)cudaGetLastError();
 }
 

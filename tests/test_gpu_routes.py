@@ -216,3 +216,25 @@ def test_run_wise_masks_filter_and_enumeration(ctx):
             rows, got = cc.cc_enumerate(ctx.h, run, 50_000, 4)
             assert got == total and np.array_equal(rows, want[:50_000])
             cc.cc_release(ctx.h, run)
+
+
+def theta(n_mid):
+    """Two vertices joined through n_mid middle ones: every middle vertex is the others' twin."""
+    e = [(u, 2 + i) for i in range(n_mid) for u in (0, 1)]
+    bags = [[0, 1, 2 + i] for i in range(n_mid)]
+    return 2 + n_mid, np.array(e, np.int32), (bags, [i + 1 for i in range(n_mid - 1)] + [-1])
+
+
+# an entry alone with its mapping and trial has no candidate when a forgotten vertex could have
+# been the candidate's (4-cycles, theta graphs, the first square of a grid; chained in the 3x3
+# grid), and may have one when not (5-cycles, a triangle with a tail)
+@pytest.mark.parametrize("name", ["C4", "theta3", "theta4", "grid24", "grid33", "C5", "B"])
+@pytest.mark.parametrize("trials", [2, 9])
+def test_twin_rule(ctx, name, trials):
+    pat = {"C4": synth.cycle_pattern(4), "theta3": theta(3), "theta4": theta(4),
+           "grid24": synth.grid_pattern(2, 4), "grid33": synth.grid_pattern(3, 3),
+           "C5": synth.cycle_pattern(5), "B": synth.pattern_B()}[name]
+    n = 2600 if trials == 2 else 700
+    g = hub_graph(n, 9) if name not in ("grid33", "C5", "B") else \
+        synth.erdos_renyi(n, 9.0 / n, 9)
+    check_tables(ctx, g, pat, oracle.colors(n, trials, pat[0], seed=5), pat[0])
