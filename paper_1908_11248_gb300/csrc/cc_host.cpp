@@ -682,15 +682,15 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     const cc::NodeTable &ty = R->tables[y];
     const int b_in = (int)ny.bag.size(), b_out = b_in + (f >= 0 ? 0 : 1), nb = R->L.nb;
     const bool leaf = ny.type == 0;
-    if (R->trials < cc::kRunTrials || a.nnb != 1 || a.G.row_ptr != c->d_row_ptr ||
-        R->opts.sort_sweep != 1 || R->opts.fuse != 2 || n == 0 || b_out == 0 ||
-        (b_in + 1) * nb > 62 || R->L.k + R->L.tb > 24)
+    if (((f >= 0 || leaf) && R->trials < cc::kRunTrials) || a.nnb > 1 ||
+        a.G.row_ptr != c->d_row_ptr || R->opts.sort_sweep != 1 || R->opts.fuse != 2 || n == 0 ||
+        b_out < (f >= 0 ? 2 : 1) || (b_in + 1) * nb > 62 || R->L.k + R->L.tb > 24)
       return CC_OK;
     if (!leaf && (ty.hashed || ty.sort_n != b_in || ty.sort_hbits)) return CC_OK;
     if (planned) {
       const cc::RunSizes &r = plan->runwise[x];
       if (plan->entries[x] <= kHashEntries || r.slots == 0 ||
-          plan->entries[x] < cc::kRunYield * r.slots)
+          plan->entries[x] < cc::kRunYield * r.slots || 2 * r.more > plan->entries[x])
         return CC_OK;
     }
     Held held{A, {}};
@@ -717,7 +717,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     for (int z = y; z >= 0; z = P.nodes[z].child0)
       if (P.nodes[z].type > 1) r.ones = 0;
     r.b_in = b_in;
-    r.anchor = a.nb_slot[0];
+    r.anchor = a.nnb ? a.nb_slot[0] : -1;
     r.p = a.p;
     r.q = f >= 0 ? pos_in(nd.bag, P.nodes[f].vertex) : -1;
     r.b_out = b_out;
@@ -833,6 +833,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       rc = read_u64(c, n_one, &one);
       if (!rc) rc = read_u64(c, w_more, &more);
       if (rc) return rc;
+      if (2 * more > one + more) {  // most entries would be sorted after all
+        CUDA_OK(cudaMemsetAsync(a.cand, 0, sizeof(u64), c->stream));
+        return CC_OK;
+      }
       cap = std::max<u64>(1, one + more);
     } else {
       more = room(plan->runwise[x].more);
@@ -1049,6 +1053,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       const bool warp_path = planned && (a.nnb <= 1 || grouped);
       a.chunk = 256;
       a.win = 32;
+      a.stretch = 8;
       u64 slack = chunk_slack;
       if (warp_path) {
         const u64 warps = (u64)c->dev.sms * c->dev.blocks_per_sm * 8;
@@ -1058,6 +1063,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         const cc::NodeTable &ty = R->tables[y];
         const u64 scan = ty.hashed ? ty.cap : plan->entries[y];
         while (a.win > 4 && warps * a.win > scan) a.win >>= 1;
+        // grouped windows differ more in cost (hubs): sixteen a warp, if not of fewer than 8 entries
+        // (with several trials a window of 8 would hold less than a run)
+        while (grouped && R->trials == 1 && a.win > 8 && warps * a.win * 16 > scan) a.win >>= 1;
+        while (a.stretch > 1 && warps * a.win * 16 * a.stretch > scan) a.stretch >>= 1;
         // hubs: room for the parts of their lists (8 MB at most; what does not fit is walked in
         // place), and for the second kernel's last chunks
         if (a.nnb == 1 && a.G.row_ptr == c->d_row_ptr && c->max_deg > cc::kHeavyList) {

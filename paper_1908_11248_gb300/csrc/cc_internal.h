@@ -76,6 +76,7 @@ struct IntroArgs {
   uint32_t ubit;             // 1 << u, tested against G.allow
   unsigned chunk;            // warp kernels, mode 1: slots a warp reserves at a time (32..256)
   unsigned win;              // warp kernels: child entries a warp takes at a time (4..32)
+  unsigned stretch;          // grouped kernels: consecutive windows a warp takes (1, 2, 4 or 8)
   // launch_intro_warp: the long candidate lists of a window that has many candidates are left to
   // a second kernel, as (entry, part of its list) items, while there is room for them (heavy_cap
   // 0: none are)
@@ -110,7 +111,7 @@ struct IntroArgs {
   int twin;
 };
 
-constexpr int kHeavyWindow = 2048;  // candidates of a window above which its long lists leave it
+constexpr int kHeavyWindow = 64;  // candidates an entry above which a window's long lists leave it
 constexpr int kHeavyList = 64;   // longest candidate list such a window keeps
 constexpr int kHeavyPart = 256;  // candidates of a longer one a warp walks at a time
 
@@ -153,12 +154,13 @@ struct RunsArgs {
   unsigned long long *first;   // per run: its first entry
   unsigned *packed;            // per entry: trial << k | colour set
   // the introduced vertex
-  int b_in, anchor;            // child bag size, slot of its one bag neighbour
+  int b_in, anchor;            // child bag size, slot of its one bag neighbour (-1: it has none)
   int p, q;                    // its slot in the new bag; the slot the parent forgets (-1: none)
   int b_out;                   // slots left
   int degF;
   uint32_t ubit;
-  // pairs, in the order of the runs: a run's candidates are its anchor image's neighbours
+  // pairs, in the order of the runs: a run's candidates are its anchor image's neighbours, or
+  // every host vertex
   unsigned *deg;                   // per run: candidates
   const unsigned long long *off;   // exclusive sums of those
   const unsigned long long *n_slots;
@@ -179,7 +181,7 @@ struct RunsArgs {
   unsigned long long side_cap;
   int *err;
 };
-// fewest trials for it, and fewest entries a pair must yield on average
+// fewest trials for it below a forget or above a leaf, and fewest entries a pair must yield
 constexpr int kRunTrials = 8;
 constexpr unsigned long long kRunYield = 2;
 

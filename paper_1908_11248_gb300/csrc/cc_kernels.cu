@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(256, 4) intro_warp_kernel(IntroArgs a) {
       if (lane >= o) incl += y;
     }
     I total = __shfl_sync(0xffffffffu, incl, 31);
-    if (a.heavy_cap && total > (I)kHeavyWindow) {  // the window's long lists go to the other kernel
+    if (a.heavy_cap && total > (I)(kHeavyWindow * a.win)) {  // the window's long lists go to the other kernel
       const int parts = nc > (I)kHeavyList ? (int)((nc + kHeavyPart - 1) / kHeavyPart) : 0;
       int upto = parts;
       for (int o = 1; o < 32; o <<= 1) {
@@ -619,8 +619,8 @@ __global__ void __launch_bounds__(256, 4) intro_warp_kernel(IntroArgs a) {
 // candidates at 32 a step took a millisecond whatever the rest of the table held.  With the
 // lists cut into parts the five expanding introduces of a six-vertex path on a Barabasi-Albert
 // graph (n = 200 000, m = 5, largest degree 1934) went from 6.2 ms to 0.8.  A window of
-// up to kHeavyWindow candidates (64 steps) is walked in place, and so is any list of up to
-// kHeavyList, where 32 entries share steps.
+// up to kHeavyWindow candidates an entry (64 steps for 32 entries, 8 for the 4 of a small table) is
+// walked in place, and so is any list of up to kHeavyList, where the entries share steps.
 template <typename K, int MODE>
 __global__ void __launch_bounds__(256, 4) intro_heavy_kernel(IntroArgs a) {
   const Slot<K> *in = reinterpret_cast<const Slot<K> *>(a.in.slots);
@@ -704,14 +704,16 @@ __global__ void __launch_bounds__(256, 4) intro_heavy_kernel(IntroArgs a) {
 // and every chain of a window in sequence; end to end, a step's 32 chains belong to several
 // leads.  The closing introduce of a 4-cycle (one colouring of a
 // Barabasi-Albert graph, n = 200 000, m = 5; 27 million entries, 249 million candidates): 15.3 to
-// 10.8 ms (and 5.1 with the windows spread, kGroupStretch); the three of the 2x4 grid with 13 colourings (n = 4999, m = 4): 1.47 to 1.00 ms.
+// 10.8 ms (and 5.1 with the windows spread, IntroArgs::stretch); the three of the 2x4 grid with 13 colourings (n = 4999, m = 4): 1.47 to 1.00 ms.
 constexpr int kGroupCap = 256;  // candidate-list buffer per warp (two of them)
-// Consecutive windows a warp takes before it goes on elsewhere: long enough to carry lists, short
-// enough that a stretch of costly runs (a hub's; the region of mappings that several runs led to,
+// IntroArgs::stretch, the consecutive windows a warp takes before it goes on elsewhere (1, 2, 4, 8): long
+// enough to carry lists, short enough that a stretch of costly runs (a hub's; the region of mappings that several runs led to,
 // cc_runs.cu) is spread over the warps.  One range a warp instead: 28.6 ms for the chained
 // introduce of the 3x3 grid (Erdos-Renyi, n = 100 000, 32 colourings), 12.7 in stretches;
-// the 4-cycle's closing introduce (Barabasi-Albert, n = 200 000) 10.8 against 5.1.
-constexpr u64 kGroupStretch = 8;
+// the 4-cycle's closing introduce (Barabasi-Albert, n = 200 000) 10.8 against 5.1.  A table that
+// gives a warp few windows has shorter stretches, and with one colouring, whose runs are short,
+// smaller windows too: the closing introduce of the 4-cycle over 2.1 million entries
+// (Barabasi-Albert, n = 20 000) went from 0.52 to 0.15 ms.
 
 // true if v is in the increasing list col[lo, hi)
 __device__ __forceinline__ bool listed(const int32_t *col, int lo, int hi, int v) {
@@ -839,13 +841,13 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   // the next window's records are loaded while the current one is processed
   K nkey = 0;
   u64 nc_ = 0;
-  const u64 w0 = wid * kGroupStretch;
+  const u64 stretch = CHAIN ? 8 : a.stretch, w0 = wid * stretch;
   if (w0 < nwin && w0 * width + mylane < bound) load_slot(in, w0 * width + mylane, nkey, nc_);
   for (u64 win = w0, follow; win < nwin; win = follow) {
     const K key = nkey;
     const u64 c = nc_;
     follow = win + 1;
-    if (follow % kGroupStretch == 0) follow += (warps - 1) * kGroupStretch;
+    if ((follow & (stretch - 1)) == 0) follow += (warps - 1) * stretch;
     {
       const u64 i2 = follow * width + mylane;
       nkey = 0;

@@ -20,8 +20,13 @@
 // 4.4 ms here.  Of the three big ones of the 2x4 grid (Barabasi-Albert, n = 20 000, 64 colourings;
 // 159, 154 and 90 million entries): 40 ms entry by entry, 11 here.
 //
-// With fewer than kRunTrials trials, or fewer than kRunYield entries a pair, a pair's record is no
-// smaller than what it stands for, and the entry kernels take the node.
+// Below a join the result's order saves a sort of its own.  With fewer than kRunYield entries a
+// pair, a pair's record is no smaller than what it stands for; where most mappings have several
+// origins (a forget that leaves one vertex) most entries would be sorted in the side buffer after
+// all: the entry kernels take those nodes, and those of fewer than kRunTrials trials below a forget
+// or above a leaf.  The 9-vertex tree (Barabasi-Albert, n = 20 000, 4 colourings), whose stored
+// introduces yield 15 to 100 entries a pair: 8.5 to 7.8 ms a run; a batch of partial k-trees with
+// 4 colourings is the same with the line at 4 trials as at 8 (9.07 and 8.99 ms).
 #include <algorithm>
 #include <cstdint>
 
@@ -134,10 +139,13 @@ __global__ void __launch_bounds__(256) runs_degree_kernel(RunsArgs a) {
     if (!a.leaf) {
       K key;
       u64 c;
-      load_slot(in, a.first[r], key, c);
-      w = key_slot(key, a.L, a.anchor);
+      if (a.anchor >= 0) {
+        load_slot(in, a.first[r], key, c);
+        w = key_slot(key, a.L, a.anchor);
+      }
     }
-    if (!a.leaf || leaf_ok(a, w)) d = (unsigned)(a.G.row_ptr[w + 1] - a.G.row_ptr[w]);
+    if (!a.leaf || leaf_ok(a, w))
+      d = a.anchor < 0 ? (unsigned)a.G.n : (unsigned)(a.G.row_ptr[w + 1] - a.G.row_ptr[w]);
     a.deg[r] = d;
   }
 }
@@ -174,8 +182,8 @@ __global__ void __launch_bounds__(256) runs_pairs_kernel(RunsArgs a) {
       load_slot(in, e0, key, c);
       phi = phi_bits(key, a);
     }
-    const int w = (int)(phi >> (a.anchor * nb) & vm);
-    const int v = __ldg(a.G.col + a.G.row_ptr[w] + (int)(j - a.off[r]));
+    int v = (int)(j - a.off[r]);
+    if (a.anchor >= 0) v = __ldg(a.G.col + a.G.row_ptr[(int)(phi >> (a.anchor * nb) & vm)] + v);
     unsigned cnt = 0;
     if ((a.degF == 0 || a.G.deg8[v] >= a.degF) && (!a.G.allow || (a.G.allow[v] & a.ubit))) {
       const uint8_t *cv = a.colT + (u64)v * (u64)T;

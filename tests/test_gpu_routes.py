@@ -179,12 +179,13 @@ def hub_graph(n, seed):
 # introduces run by run need 8 trials, more than 2^18 entries (planned) and two entries a pair: one
 # trial too few, the fewest, several bytes of trials; leaf, introduce and forget children; pairs
 # that share their mapping (hubs); 64- and 128-bit keys; a vertex forgotten as it comes; joins above
+# (one trial is enough where nothing is forgotten); a vertex without a bag neighbour
 @pytest.mark.parametrize("pat,n,hubs,trials,spare", [
     (("grid", 2, 4), 1500, 1, 7, 0), (("grid", 2, 4), 1500, 1, 8, 0),
     (("grid", 2, 4), 400, 1, 33, 1), (("grid", 3, 3), 2500, 0, 9, 0),
     (("grid", 3, 3), 70_000, 0, 8, 0), (("cycle", 4), 4000, 1, 16, 2),
     (("path", 5), 9000, 0, 12, 0), (("star", 5), 3000, 0, 40, 0), (("A",), 1200, 0, 10, 0),
-    (("ktree", 7, 2, 5), 700, 1, 9, 0)])
+    (("ktree", 7, 2, 5), 700, 1, 9, 0), (("A",), 5000, 0, 1, 0), (("D",), 230, 0, 9, 0)])
 def test_run_wise_introduces(ctx, pat, n, hubs, trials, spare):
     p = synth.make_pattern(pat)
     k = p[0] + spare
