@@ -559,7 +559,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   // (0.21 and 0.2), but then without the order that a grouped introduce above could use.
   // Small windows (IntroArgs::win) go with it: 29 000 entries whose lists are built one by one
   // take 0.36 ms in 900 warps of 32 entries, 0.09 ms in 7000 warps of 4.
-  const bool hash_few = R->opts.sort_sweep == 1;
+  const bool hash_few = R->opts.sort_sweep == 1 && !R->frugal;
   auto few = [&](u64 e) { return hash_few && e <= kHashEntries; };
   // true if an introduce above forget f hands f's order on to a grouped introduce above it
   auto order_handed_on = [&](int f) {
@@ -658,6 +658,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   // colours with the trials of a vertex side by side, made for the first introduce that asks
   Held transposed{A, {}};
   auto colours_by_vertex = [&](uint8_t **out) -> int {
+    if (R->frugal) return CC_ENOMEM;
     if (transposed.p.empty()) {
       void *t = A.alloc(std::max<size_t>(1, (size_t)R->trials * (size_t)n));
       if (!t) return CC_ENOMEM;
@@ -678,6 +679,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                       u64 *total) -> int {
     *taken = 0;
     *counted = false;
+    if (R->frugal) return CC_OK;
     const NiceNode &nd = P.nodes[x], &ny = P.nodes[y];
     const cc::NodeTable &ty = R->tables[y];
     const int b_in = (int)ny.bag.size(), b_out = b_in + (f >= 0 ? 0 : 1), nb = R->L.nb;
@@ -1069,7 +1071,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         while (a.stretch > 1 && warps * a.win * 16 * a.stretch > scan) a.stretch >>= 1;
         // hubs: room for the parts of their lists (8 MB at most; what does not fit is walked in
         // place), and for the second kernel's last chunks
-        if (a.nnb == 1 && a.G.row_ptr == c->d_row_ptr && c->max_deg > cc::kHeavyList) {
+        if (a.nnb == 1 && !R->frugal && a.G.row_ptr == c->d_row_ptr &&
+            c->max_deg > cc::kHeavyList) {
           const u64 parts = (u64)(c->max_deg + cc::kHeavyPart - 1) / cc::kHeavyPart;
           const u64 places = std::min<u64>(1 << 20, room(plan->entries[y]) * parts);
           heavy_mem = A.alloc((places + 1) * sizeof(u64));
@@ -1288,7 +1291,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                  [&] { return cc::launch_forget(c->stream, c->dev, R->kw, block, a); });
       if (rc) return rc;
       release_child(y);
-    } else if (R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
+    } else if (!R->frugal && R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
                entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries) {
       // join, group by group (cc_join.cu)
       const int b = (int)nd.bag.size();
@@ -1991,7 +1994,10 @@ void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t
 }
 
 // Runs the nodes on the context's stream: planned when a plan exists (repeated exactly if the
-// plan proves too small), exact otherwise; then reads the results and updates the plan.
+// plan proves too small), exact otherwise; then reads the results and updates the plan.  A run
+// that nothing could make smaller (its tables are kept, or it is a single trial) and that runs
+// out of memory is repeated without the routes that hold scratch beside the tables (Run::frugal),
+// so that a context in which the tables just fit still counts them; the plan remembers it.
 int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long long> &key,
                bool exact_only) {
   const Pattern &P = c->patterns.at(R->pattern);
@@ -2001,6 +2007,7 @@ int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long l
   auto pl = c->plans.find(key);
   R->planned = !exact_only && pl != c->plans.end() && pl->second.runs > 0;
   R->graphed = false;
+  R->frugal = pl != c->plans.end() && pl->second.frugal;
   Arena &A = active_arena(c);
   const size_t base = A.in_use();
   A.reset_high_water();
@@ -2017,6 +2024,14 @@ int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long l
   } else {
     rc = run_nodes(c, R, P, col, nullptr);
     if (!rc) rc = finish_run(c, R);
+  }
+  if (rc == CC_ENOMEM && !R->frugal && (R->retained || R->trials == 1)) {
+    R->frugal = true;
+    rc = reset_run(c, R, N);
+    A.reset_high_water();
+    if (!rc) rc = run_nodes(c, R, P, col, nullptr);
+    if (!rc) rc = finish_run(c, R);
+    if (!rc) c->plans[key].frugal = true;
   }
   if (rc) return rc;
   update_plan(c, key, R, A.high_water() - base);
@@ -2118,6 +2133,7 @@ int capture_graph(Ctx *c, const std::vector<Run *> &Rs,
     S->trials = R->trials;
     S->home = &gm.sub;
     S->planned = true;
+    S->frugal = c->plans.at(keys[m]).frugal;
     S->d_counters = (u64 *)gm.sub.alloc(cc::kWords * N * sizeof(u64));
     S->d_exists = (unsigned *)gm.sub.alloc(R->trials * sizeof(unsigned));
     S->d_count = (u64 *)gm.sub.alloc(R->trials * sizeof(u64));

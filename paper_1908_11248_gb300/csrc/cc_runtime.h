@@ -175,6 +175,7 @@ struct Plan {
   std::vector<RunSizes> runwise;  // of introduces taken run by run
   size_t peak_bytes = 0;  // largest arena use of a run beyond what it started with
   int runs = 0;
+  bool frugal = false;  // its runs leave out the routes that hold scratch beside the tables
   size_t refused = 0;  // a served run of this key ran out of memory in a range this large
   int slices = 0;      // a single trial of this key fitted once split into this many slices
 };
@@ -206,6 +207,7 @@ struct Run {
   bool planned = false;
   bool graphed = false;
   bool streamed = false;  // its trials ran in chunks (all at once did not fit)
+  bool frugal = false;    // no route that holds scratch beside the tables (see run_direct)
   int sliced = 0;         // most slices one of its trials was split into (0: none)
   u64 *d_blk = nullptr;  // per-run scratch: block counts and bases, pair counters
   int *d_err = nullptr;  // per-run device error word

@@ -239,3 +239,37 @@ def test_twin_rule(ctx, name, trials):
     g = hub_graph(n, 9) if name not in ("grid33", "C5", "B") else \
         synth.erdos_renyi(n, 9.0 / n, 9)
     check_tables(ctx, g, pat, oracle.colors(n, trials, pat[0], seed=5), pat[0])
+
+
+# routes with scratch beside the tables (introduces run by run, joins group by group) and hubs, kept
+# and not, from rooms that hold little more than the graph to ones that hold everything twice
+@pytest.mark.parametrize("pat,n,trials", [(("grid", 2, 4), 1500, 9), (("A",), 4000, 1)])
+@pytest.mark.parametrize("retain", [0, 1])
+def test_every_arena_size(pat, n, trials, retain):
+    """Whatever the room, a run (planned from exact runs, or exact) counts what the oracle does or
+    ends with CC_ENOMEM; only a run that keeps its tables, or a slice too many, ever does."""
+    p = synth.make_pattern(pat)
+    g = hub_graph(n, 3)
+    z = oracle.colors(n, trials, p[0], seed=5)
+    ref = oracle.run_dp(g, p, z, p[0])
+    fitted = 0
+    mb = 2.0
+    while mb < 1024:
+        with cc.Context(arena_bytes=int(mb * 2 ** 20)) as c:
+            cc.cc_load_graph(c.h, *g)
+            pid = cc.cc_load_pattern(c.h, *p)
+            cid = cc.cc_set_colors(c.h, z, p[0])
+            opts = cc.cc_default_opts(retain=retain, max_slices=8)
+            for _ in range(3):
+                try:
+                    run = cc.cc_run_dp(c.h, pid, cid, opts)
+                except cc.CCError as ex:
+                    assert ex.code == cc.CC_ENOMEM, mb
+                    break
+                assert np.array_equal(cc.cc_count(c.h, run, trials), ref.count), mb
+                assert np.array_equal(cc.cc_decide(c.h, run, trials), ref.exists), mb
+                cc.cc_release(c.h, run)
+            else:
+                fitted += 1
+        mb *= 1.2
+    assert fitted
