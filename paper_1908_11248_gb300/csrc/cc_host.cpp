@@ -561,6 +561,16 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   // take 0.36 ms in 900 warps of 32 entries, 0.09 ms in 7000 warps of 4.
   const bool hash_few = R->opts.sort_sweep == 1 && !R->frugal;
   auto few = [&](u64 e) { return hash_few && e <= kHashEntries; };
+  // true if a mapping of forget f that only one (mapping below, candidate) pair leads to has no
+  // candidate in the introduce above (cc_runs.cu), and no caller sees f's table
+  auto lone_dead = [&](int f) {
+    const int g = P.nodes[f].parent;
+    if (R->opts.retain || g < 0 || P.nodes[g].type != 1 || P.d_allow || R->opts.distance_prune)
+      return false;
+    uint32_t bag = 0;
+    for (int w : P.nodes[f].bag) bag |= 1u << w;
+    return !(P.adj[P.nodes[f].vertex] & ~(P.adj[P.nodes[g].vertex] & bag));
+  };
   // true if an introduce above forget f hands f's order on to a grouped introduce above it
   auto order_handed_on = [&](int f) {
     const int g = P.nodes[f].parent, h = g >= 0 ? P.nodes[g].parent : -1;
@@ -723,6 +733,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     r.p = a.p;
     r.q = f >= 0 ? pos_in(nd.bag, P.nodes[f].vertex) : -1;
     r.b_out = b_out;
+    r.drop = f >= 0 && lone_dead(f);
+    if (r.drop) r.kept = cursor + f;
     r.degF = a.degF;
     r.ubit = a.ubit;
     uint8_t *colT = nullptr;
@@ -839,13 +851,13 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         CUDA_OK(cudaMemsetAsync(a.cand, 0, sizeof(u64), c->stream));
         return CC_OK;
       }
-      cap = std::max<u64>(1, one + more);
+      cap = std::max<u64>(1, r.drop ? more : one + more);
     } else {
       more = room(plan->runwise[x].more);
-      cap = room(plan->entries[f >= 0 ? f : x]);
+      cap = r.drop ? more : room(plan->entries[f >= 0 ? f : x]);
       check(w_more, more);
       check(R->d_counters + x, room(plan->entries[x]));
-      if (f >= 0) check(R->d_counters + f, cap);
+      if (f >= 0) check(R->d_counters + f, room(plan->entries[f]));
     }
     void *out = A.alloc(cap * rb);
     if (!out) {
@@ -870,7 +882,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
           held.p.push_back(srt);
           rc = timed(f, CC_K_REDUCE, 3, [&] {
             return cc::launch_reduce(c->stream, c->dev, R->kw, srt, w_more, r.side_cap, blk,
-                                     r.side, words + 2, &fsp, cc::sort_narrows(R->kw, fsp, 1));
+                                     r.drop ? out : r.side, words + 2, &fsp, cc::sort_narrows(R->kw, fsp, 1));
           });
         }
       }
@@ -891,6 +903,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       t.sort_n = b_out;
       for (int j = 0; j < b_out; ++j) t.sort_slots[j] = fsp.order[j];
       t.regions = true;
+      t.dropped = r.drop;
+      if (r.drop) t.bound = r.kept;
     } else {  // the child's order, then the new vertex
       const int m = leaf ? 1 : b_in;
       int *so = ty.regions ? t.cluster_slots : t.sort_slots;
@@ -991,11 +1005,12 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         sp.bits = a.nnb * R->L.nb;
         const cc::NodeTable &ty = R->tables[y];
         const u64 m = entries(y);
+        u64 *live = ty.dropped ? ty.bound : R->d_counters + y;  // nonempty entries
         check(R->d_counters + y, m);
-        rc = sort_records(x, sp, ty.slots, ty.hashed ? c->d_ones : desc(y).count, ty.cap,
-                          R->d_counters + y, m, &sorted);
+        rc = sort_records(x, sp, ty.slots, ty.hashed ? c->d_ones : desc(y).count, ty.cap, live, m,
+                          &sorted);
         if (rc) return rc;
-        a.in = TableDesc{sorted, std::max<u64>(1, m), R->d_counters + y, 0};
+        a.in = TableDesc{sorted, std::max<u64>(1, m), live, 0};
       }
       {
         const cc::NodeTable &ty = R->tables[y];
@@ -1063,7 +1078,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         slack = warps * a.chunk;
         // fewer entries a window while that puts more of the GPU's warps to work
         const cc::NodeTable &ty = R->tables[y];
-        const u64 scan = ty.hashed ? ty.cap : plan->entries[y];
+        const u64 scan = ty.hashed ? ty.cap : std::min(ty.cap, plan->entries[y]);
         while (a.win > 4 && warps * a.win > scan) a.win >>= 1;
         // grouped windows differ more in cost (hubs): sixteen a warp, if not of fewer than 8 entries
         // (with several trials a window of 8 would hold less than a run)

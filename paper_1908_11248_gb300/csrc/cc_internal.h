@@ -179,6 +179,10 @@ struct RunsArgs {
   TableDesc out;
   void *side;
   unsigned long long side_cap;
+  // the entries of pairs alone with their mapping are counted and not written; *kept: entries that
+  // are (`out` then holds the merged side entries)
+  int drop;
+  unsigned long long *kept;
   int *err;
 };
 // fewest trials for it below a forget or above a leaf, and fewest entries a pair must yield

@@ -153,6 +153,9 @@ struct NodeTable {
   int sort_min = 0, sort_hbits = 0, sort_hslots = 0;
   // sorted in two regions one after the other; every run of equal images lies in one of them
   bool regions = false;
+  // entries that no candidate extends were counted and not written (RunsArgs::drop): `bound` of them
+  // are here
+  bool dropped = false;
   // a dense table whose entries come in runs of equal images of these slots, except where an
   // append chunk or a kernel's tile ends (written in the order of a child sorted or clustered
   // by them); cluster_n == 0: no known clustering
