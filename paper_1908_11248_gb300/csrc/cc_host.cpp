@@ -427,6 +427,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   R->sizes.assign(N, 0);
   R->pairs.assign(N, 0);
   R->runwise.assign(N, {});
+  R->starved = false;
   R->checks.clear();
   std::vector<bool> made(N, false);
   const int grid = cc::intro_grid(c->dev, block);
@@ -684,7 +685,9 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   // (cc_runs.cu).  *taken: 1 if it made the table of x (or of f), 0 if the entry kernels have to;
   // *total: the entries of x when an exact run has counted them here (else left alone).  Taken
   // when there are trials enough for the pairs to be few beside the entries, when the child's
-  // entries come in whole runs of equal mappings, and when there is room.
+  // entries come in whole runs of equal mappings, and when there is room; in a planned run, when
+  // the last exact run that tried it went through (a plan of one that did not has no room for the
+  // entries that share their mapping).
   auto run_wise = [&](int x, int y, int f, const cc::IntroArgs &a, int *taken, bool *counted,
                       u64 *total) -> int {
     *taken = 0;
@@ -701,7 +704,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (!leaf && (ty.hashed || ty.sort_n != b_in || ty.sort_hbits)) return CC_OK;
     if (planned) {
       const cc::RunSizes &r = plan->runwise[x];
-      if (plan->entries[x] <= kHashEntries || r.slots == 0 ||
+      if (r.state != cc::Runwise::kDone || plan->entries[x] <= kHashEntries || r.slots == 0 ||
           plan->entries[x] < cc::kRunYield * r.slots || 2 * r.more > plan->entries[x])
         return CC_OK;
     }
@@ -713,6 +716,18 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       else short_of = true;
       return q;
     };
+    // on every way out: how far the attempt came
+    struct Outcome {
+      Run &run;
+      cc::RunSizes &r;
+      const int &taken;
+      const bool &short_of;
+      bool exact;
+      ~Outcome() {
+        r.state = taken ? cc::Runwise::kDone : exact ? cc::Runwise::kLeft : r.state;
+        if (exact && !taken && short_of) run.starved = true;
+      }
+    } outcome{*R, R->runwise[x], *taken, short_of, !planned};
     cc::RunsArgs r{};
     r.G = a.G;
     r.L = R->L;
@@ -738,7 +753,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     r.degF = a.degF;
     r.ubit = a.ubit;
     uint8_t *colT = nullptr;
-    if (colours_by_vertex(&colT) != CC_OK) return CC_OK;
+    if (colours_by_vertex(&colT) != CC_OK) {
+      short_of = true;
+      return CC_OK;
+    }
     r.colT = colT;
     // capacities: planned, or known as the exact run goes
     u64 *w_slots = R->d_counters + 4 * N + x, *w_pairs = R->d_counters + 5 * N + x,
@@ -813,7 +831,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       r.list_cap = std::max<u64>(1, pairs);
       rc = sort_records_of(1, f, ps, r.recs, w_slots, r.pair_cap, w_pairs, r.list_cap,
                            &sorted_pairs);
-      if (rc == CC_ENOMEM) return CC_OK;
+      if (rc == CC_ENOMEM) {
+        short_of = true;
+        return CC_OK;
+      }
       if (rc) return rc;
       held.p.push_back(sorted_pairs);
       r.list = sorted_pairs;
@@ -861,6 +882,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     }
     void *out = A.alloc(cap * rb);
     if (!out) {
+      short_of = true;
       if (f < 0) CUDA_OK(cudaMemsetAsync(n_one, 0, sizeof(u64), c->stream));
       return CC_OK;
     }
@@ -894,7 +916,9 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     }
     if (rc) {
       A.release(out);
-      return rc == CC_ENOMEM ? CC_OK : rc;
+      if (rc != CC_ENOMEM) return rc;
+      short_of = true;
+      return CC_OK;
     }
     const int z = f >= 0 ? f : x;
     R->tables[z] = {out, cap, 0, true};
@@ -1463,7 +1487,8 @@ int finish_run(Ctx *c, Run *R) {
     R->sizes[x] = words[x];
     if (words[2 * N + x]) R->pairs[x] = words[2 * N + x];
     if (words[4 * N + x])
-      R->runwise[x] = {words[4 * N + x], words[5 * N + x], words[6 * N + x], words[7 * N + x]};
+      R->runwise[x] = {words[4 * N + x], words[5 * N + x], words[6 * N + x], words[7 * N + x],
+                       R->runwise[x].state};
   }
   for (auto &t : R->timings)
     if (t.kind == CC_K_INTRO_COUNT || t.kind == CC_K_INTRO_WRITE || t.kind == CC_K_INTRO_FUSED ||
@@ -1988,6 +2013,10 @@ int reset_run(Ctx *c, Run *R, int N) {
   return CC_OK;
 }
 
+bool plan_ready(const cc::Plan &plan, size_t room) {
+  return plan.runs > 0 && !(plan.starved && room / 2 >= plan.starved);
+}
+
 // Folds a finished run's sizes into the plan of its key.
 void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t peak) {
   cc::Plan &plan = c->plans[key];
@@ -2002,8 +2031,9 @@ void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t
     cc::RunSizes &p = plan.runwise[x];
     const cc::RunSizes &r = R->runwise[x];
     p = {std::max(p.slots, r.slots), std::max(p.pairs, r.pairs), std::max(p.more, r.more),
-         std::max(p.runs, r.runs)};
+         std::max(p.runs, r.runs), r.state != cc::Runwise::kUntried ? r.state : p.state};
   }
+  if (!R->planned) plan.starved = R->starved ? std::max<size_t>(1, R->room) : 0;
   plan.peak_bytes = std::max(plan.peak_bytes, peak);
   plan.runs++;
 }
@@ -2020,10 +2050,11 @@ int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long l
   int rc = reset_run(c, R, N);
   if (rc) return rc;
   auto pl = c->plans.find(key);
-  R->planned = !exact_only && pl != c->plans.end() && pl->second.runs > 0;
+  Arena &A = active_arena(c);
+  R->room = A.free_bytes();
+  R->planned = !exact_only && pl != c->plans.end() && plan_ready(pl->second, R->room);
   R->graphed = false;
   R->frugal = pl != c->plans.end() && pl->second.frugal;
-  Arena &A = active_arena(c);
   const size_t base = A.in_use();
   A.reset_high_water();
   if (R->planned) {
@@ -2073,7 +2104,7 @@ void drop_all_graphs(Ctx *c) {
 bool graph_eligible(Ctx *c, const Run *R, const std::vector<long long> &key) {
   if (!R->opts.use_graph || R->opts.retain || R->opts.profile) return false;
   auto pl = c->plans.find(key);
-  return pl != c->plans.end() && pl->second.runs > 0;
+  return pl != c->plans.end() && plan_ready(pl->second, c->arena.free_bytes());
 }
 
 // Captures the planned runs of Rs as one CUDA graph: member m runs on branch stream m (on the

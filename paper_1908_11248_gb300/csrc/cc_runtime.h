@@ -166,9 +166,12 @@ struct NodeTable {
 };
 
 // What an introduce taken run by run (cc_runs.cu) met: (run, candidate) pairs, those that yield
-// entries, entries of pairs that share their mapping, runs.
+// entries, entries of pairs that share their mapping, runs.  An attempt that was left early has
+// written the first of them only.
+enum class Runwise : uint8_t { kUntried, kDone, kLeft };
 struct RunSizes {
   u64 slots = 0, pairs = 0, more = 0, runs = 0;
+  Runwise state = Runwise::kUntried;
 };
 
 // Capacities learned from exact runs of one (pattern, graph, trials, colours, options): the
@@ -178,6 +181,9 @@ struct Plan {
   std::vector<RunSizes> runwise;  // of introduces taken run by run
   size_t peak_bytes = 0;  // largest arena use of a run beyond what it started with
   int runs = 0;
+  // room in which the last exact run left an introduce run by run for want of memory (0: in none):
+  // with twice that room the key is planned anew
+  size_t starved = 0;
   bool frugal = false;  // its runs leave out the routes that hold scratch beside the tables
   size_t refused = 0;  // a served run of this key ran out of memory in a range this large
   int slices = 0;      // a single trial of this key fitted once split into this many slices
@@ -211,6 +217,8 @@ struct Run {
   bool graphed = false;
   bool streamed = false;  // its trials ran in chunks (all at once did not fit)
   bool frugal = false;    // no route that holds scratch beside the tables (see run_direct)
+  size_t room = 0;        // free arena bytes when it started
+  bool starved = false;   // an introduce run by run was left for want of memory (exact runs)
   int sliced = 0;         // most slices one of its trials was split into (0: none)
   u64 *d_blk = nullptr;  // per-run scratch: block counts and bases, pair counters
   int *d_err = nullptr;  // per-run device error word
@@ -306,6 +314,8 @@ int reset_run(Ctx *c, Run *R, int N);
 int run_nodes(Ctx *c, Run *R, const Pattern &P, const Coloring &col, const Plan *plan);
 // Reads the run's error word, sizes and capacity checks (waits for the context's stream).
 int finish_run(Ctx *c, Run *R);
+// True if runs of the plan's key can be planned in this much room.
+bool plan_ready(const Plan &plan, size_t room);
 // Folds a finished run's sizes (and its arena peak) into the plan of its key.
 void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t peak);
 // Runs R to completion on the context's stream: planned if a plan exists and exact_only is

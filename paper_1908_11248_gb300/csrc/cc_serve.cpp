@@ -210,8 +210,9 @@ Outcome issue(Server *S, Ctx *c, ServeSlot &sl, const ServeQuery &q, bool alone)
   if (!rc) {
     bool exact = true;
     auto pl = c->plans.find(sl.key);
+    const bool known = pl != c->plans.end() && rt::plan_ready(pl->second, sl.sub.free_bytes());
     const bool split = pl != c->plans.end() && pl->second.slices > 0 && q.limit == 0;
-    if (!q.exact && !split && q.limit == 0 && pl != c->plans.end() && pl->second.runs > 0) {
+    if (!q.exact && !split && q.limit == 0 && known) {
       exact = false;
       rc = rt::reset_run(c, sl.run.get(), (int)P.nodes.size());
       if (!rc) rc = rt::run_nodes(c, sl.run.get(), P, sl.view, &pl->second);
@@ -235,11 +236,9 @@ Outcome issue(Server *S, Ctx *c, ServeSlot &sl, const ServeQuery &q, bool alone)
       // planned with its tables kept when it asks for embeddings
       {
         std::lock_guard<std::mutex> g2(S->mu);
-        if (q.limit == 0 || q.exact || pl == c->plans.end() || pl->second.runs == 0)
-          S->exact_runs++;
+        if (q.limit == 0 || q.exact || !known) S->exact_runs++;
       }
-      const bool planned_enum = q.limit > 0 && !q.exact && pl != c->plans.end() &&
-                                pl->second.runs > 0;
+      const bool planned_enum = q.limit > 0 && !q.exact && known;
       if (split && alone) {
         rc = rt::run_split(c, sl.run.get(), sl.view);
       } else if (split) {

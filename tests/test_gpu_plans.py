@@ -1,0 +1,106 @@
+"""What a plan remembers: whether later runs of its key go the same way whatever colouring or room the
+first ones had.  Results are whole numbers, compared for equality."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+cc = pytest.importorskip("paper_1908_11248_gb300")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+
+    __graft_entry__.build()
+
+
+def five_layers(size, deg, seed):
+    """Five layers in a ring, every vertex with `deg` neighbours in the layer on either side: coloured
+    by layer, half of an entry's candidates have a free colour."""
+    rng = np.random.default_rng(seed)
+    at, edges = np.arange(size), []
+    for a in range(5):
+        to = rng.permutation(size)
+        for shift in rng.choice(size, deg, replace=False):
+            edges.append(np.stack([a * size + at, (a + 1) % 5 * size + to[(at + shift) % size]], 1))
+    return synth.csr_from_edges(5 * size, np.concatenate(edges))
+
+
+def test_planned_when_pairs_yield_about_two_entries():
+    """Two colourings of one key, one just below the two entries a (run, candidate) pair at which
+    introduces are taken run by run and one at it: once planned, every run is."""
+    size, trials = 1600, 8
+    g = five_layers(size, 4, 1)
+    layer = np.repeat(np.arange(5), size).astype(np.uint8)
+    full = np.zeros((trials, 5 * size), np.uint8)
+    full[:4] = layer
+    fewer = full.copy()
+    fewer[0, :160] = 4  # some of the first layer coloured as the last
+    pat = synth.cycle_pattern(5)
+    want = {w: oracle.run_dp(g, pat, z, 5) for w, z in (("full", full), ("fewer", fewer))}
+    with cc.Context(arena_bytes=8 << 30) as c:
+        cc.cc_load_graph(c.h, *g)
+        pid = cc.cc_load_pattern(c.h, *pat)
+        N, _ = cc.cc_pattern_info(c.h, pid)
+        ids = {"full": cc.cc_set_colors(c.h, full, 5), "fewer": cc.cc_set_colors(c.h, fewer, 5)}
+        modes = []
+        for w in ("fewer", "full", "fewer", "fewer", "full"):
+            run = cc.cc_run_dp(c.h, pid, ids[w], cc.cc_default_opts())
+            modes.append(cc.cc_run_mode(c.h, run))
+            assert np.array_equal(cc.cc_count(c.h, run, trials), want[w].count)
+            assert np.array_equal(cc.cc_table_stats(c.h, run, N)[0],
+                                  want[w].node_sizes.sum(axis=0))
+            cc.cc_release(c.h, run)
+        assert modes == ["exact"] + ["planned"] * 4
+
+
+def kinds(c, pid, cid, trials, want, **opt):
+    """Mode of a run and the (node, kernel kind) list of its launches; its counts are checked."""
+    run = cc.cc_run_dp(c.h, pid, cid, cc.cc_default_opts(profile=1, max_slices=8, **opt))
+    assert np.array_equal(cc.cc_count(c.h, run, trials), want.count)
+    mode = cc.cc_run_mode(c.h, run)
+    node, kind, _, _ = cc.cc_run_timings(c.h, run)
+    cc.cc_release(c.h, run)
+    return mode, list(zip(node.tolist(), kind.tolist()))
+
+
+# many colourings: introduces run by run, which hold pairs beside the tables
+@pytest.mark.parametrize("pat,n,trials,retain,room_mb", [(("grid", 2, 4), 1500, 9, 0, 1024)])
+def test_little_room_once_is_not_remembered(pat, n, trials, retain, room_mb):
+    """A key whose first runs had only part of the arena (another colouring held the rest) runs, once
+    that is given back, by the same kernels as a key that had all of it from the start."""
+    p = synth.make_pattern(pat)
+    g = synth.barabasi_albert(n, 4, 3)
+    z = oracle.colors(n, trials, p[0], seed=5)
+    want = oracle.run_dp(g, p, z, p[0])
+    with cc.Context(arena_bytes=room_mb << 20) as c:
+        cc.cc_load_graph(c.h, *g)
+        cid = cc.cc_set_colors(c.h, z, p[0])
+        pid = cc.cc_load_pattern(c.h, *p)
+        for _ in range(2):
+            ref = kinds(c, pid, cid, trials, want, retain=retain)
+        assert ref[0] == "planned"
+        _, used, size = cc.cc_context_stats(c.h)
+        left, tight = size - used, 0
+        while left > 4 << 20:
+            left = int(left / 1.07)
+            used = cc.cc_context_stats(c.h)[1]
+            held = cc.cc_color(c.h, 1, (size - used - left) // n, p[0])
+            pid = cc.cc_load_pattern(c.h, *p)  # a key of its own
+            try:
+                first = [kinds(c, pid, cid, trials, want, retain=retain) for _ in range(2)]
+            except cc.CCError as ex:
+                assert ex.code == cc.CC_ENOMEM
+                first = [("none", [])]
+            cc.cc_release_colors(c.h, held)
+            if first[0][0] == "exact":
+                tight += first[-1] != ref
+                for _ in range(3):
+                    last = kinds(c, pid, cid, trials, want, retain=retain)
+                assert last == ref, left >> 20
+        assert tight
