@@ -395,6 +395,12 @@ int read_u64(Ctx *c, const u64 *d, u64 *h) {
   return CC_OK;
 }
 
+// two words with one wait
+int read_two(Ctx *c, const u64 *d0, u64 *h0, const u64 *d1, u64 *h1) {
+  CUDA_OK(cudaMemcpyAsync(h0, d0, sizeof(u64), cudaMemcpyDeviceToHost, c->stream));
+  return read_u64(c, d1, h1);
+}
+
 int pos_in(const std::vector<int32_t> &bag, int u) {
   return (int)(std::lower_bound(bag.begin(), bag.end(), u) - bag.begin());
 }
@@ -533,11 +539,9 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     *nnb2 = k2;
     return x2;
   };
-  // true if a vertex forgotten below y has all its F-neighbours among those of u in y's bag
-  // (IntroArgs::twin; with allowed mappings or the distance bound a candidate of u need not be
-  // one of that vertex)
-  auto has_twin = [&](int y, int u) {
-    uint32_t below = 0, bag = 0;
+  // the vertices forgotten at y or below it
+  auto forgotten_below = [&](int y) {
+    uint32_t below = 0;
     std::vector<int> todo{y};
     while (!todo.empty()) {
       const NiceNode &z = P.nodes[todo.back()];
@@ -546,6 +550,14 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       if (z.child0 >= 0) todo.push_back(z.child0);
       if (z.child1 >= 0) todo.push_back(z.child1);
     }
+    return below;
+  };
+  // true if a vertex forgotten below y has all its F-neighbours among those of u in y's bag
+  // (IntroArgs::twin; with allowed mappings or the distance bound a candidate of u need not be
+  // one of that vertex)
+  auto has_twin = [&](int y, int u) {
+    const uint32_t below = forgotten_below(y);
+    uint32_t bag = 0;
     for (int w : P.nodes[y].bag) bag |= 1u << w;
     for (int w = 0; w < P.nF; ++w)
       if ((below >> w & 1u) && !(bag >> w & 1u) && !(P.adj[w] & ~(P.adj[u] & bag))) return true;
@@ -767,7 +779,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                                                 : most_runs);
     r.n_runs = w_runs;
     if (r.run_cap >= 1ull << 32) return CC_OK;
-    u64 *words = (u64 *)hold(4 * sizeof(u64));  // total, one, merged, -
+    u64 *words = (u64 *)hold(4 * sizeof(u64));  // total, one, merged, most
     u64 *scan = (u64 *)hold(cc::scan_scratch_words(c->dev) * sizeof(u64));
     r.first = leaf ? nullptr : (u64 *)hold(r.run_cap * sizeof(u64));
     r.packed = leaf ? nullptr : (unsigned *)hold(ty.cap * sizeof(unsigned));
@@ -775,6 +787,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     u64 *off = (u64 *)hold(r.run_cap * sizeof(u64));
     r.off = off;
     if (short_of) return CC_OK;
+    r.n_most = words + 3;
     CUDA_OK(cudaMemsetAsync(words, 0, 4 * sizeof(u64), c->stream));
     if (leaf) {
       if (cc::launch_set_word(c->stream, w_runs, (u64)n)) return CC_ECUDA;
@@ -789,8 +802,15 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     check(w_runs, r.run_cap);
     u64 slots = 0, pairs = 0;
     if (!planned) {
-      rc = read_u64(c, w_slots, &slots);
+      u64 most = 0;
+      rc = read_two(c, w_slots, &slots, words + 3, &most);
       if (rc) return rc;
+      // Entries to expect if colours are drawn at random: a candidate's is none of the s colours of
+      // an entry in (k - s) of k cases.  Too few a pair: nothing is listed that the entry kernels
+      // would do again.  (First run of the six-cycle, Erdos-Renyi, n = 6000, 8 colourings: 8.65 ms
+      // with the pairs of such nodes counted and given up, 7.57 so; 7.55 by the entry kernels alone.)
+      const u64 s = ny.bag.size() + __builtin_popcount(forgotten_below(y)), k = R->L.k;
+      if (most * (k - s) < cc::kRunYield * slots * k) return CC_OK;
     } else {
       slots = room(plan->runwise[x].slots);
     }
@@ -809,12 +829,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                [&] { return cc::launch_runs_pairs(c->stream, c->dev, R->kw, r); });
     if (rc) return rc;
     if (!planned) {
-      rc = read_u64(c, words, total);
-      if (!rc) rc = read_u64(c, w_pairs, &pairs);
+      rc = read_two(c, words, total, w_pairs, &pairs);
       if (rc) return rc;
-      // counted, but better (or only) done entry by entry
-      if ((f >= 0 && few(*total) && !order_handed_on(f)) || *total < cc::kRunYield * slots) {
-        *counted = f >= 0 && few(*total) && !order_handed_on(f);
+      if (f >= 0 && few(*total) && !order_handed_on(f)) {  // counted, but better done entry by entry
+        *counted = true;
         CUDA_OK(cudaMemsetAsync(a.cand, 0, sizeof(u64), c->stream));
         return CC_OK;
       }
@@ -865,13 +883,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (rc) return rc;
     u64 one = 0, more = 0, cap;
     if (!planned) {
-      rc = read_u64(c, n_one, &one);
-      if (!rc) rc = read_u64(c, w_more, &more);
+      rc = read_two(c, n_one, &one, w_more, &more);
       if (rc) return rc;
-      if (2 * more > one + more) {  // most entries would be sorted after all
-        CUDA_OK(cudaMemsetAsync(a.cand, 0, sizeof(u64), c->stream));
-        return CC_OK;
-      }
       cap = std::max<u64>(1, r.drop ? more : one + more);
     } else {
       more = room(plan->runwise[x].more);

@@ -162,6 +162,7 @@ struct RunsArgs {
   // pairs, in the order of the runs: a run's candidates are its anchor image's neighbours, or
   // every host vertex
   unsigned *deg;                   // per run: candidates
+  unsigned long long *n_most;      // sum over the runs of candidates times entries
   const unsigned long long *off;   // exclusive sums of those
   const unsigned long long *n_slots;
   unsigned long long pair_cap;     // below 2^32

@@ -31,7 +31,8 @@
 // pair, a pair's record is no smaller than what it stands for; where most mappings have several
 // origins (a forget that leaves one vertex) most entries would be sorted in the side buffer after
 // all: the entry kernels take those nodes, and those of fewer than kRunTrials trials below a forget
-// or above a leaf.  The 9-vertex tree (Barabasi-Albert, n = 20 000, 4 colourings), whose stored
+// or above a leaf.  An exact run, which knows neither, goes by what the runs' lengths and random
+// colours let it expect, before any pair is listed; what it has counted it also writes.  The 9-vertex tree (Barabasi-Albert, n = 20 000, 4 colourings), whose stored
 // introduces yield 15 to 100 entries a pair: 8.5 to 7.8 ms a run; a batch of partial k-trees with
 // 4 colourings is the same with the line at 4 trials as at 8 (9.07 and 8.99 ms).
 #include <algorithm>
@@ -134,12 +135,16 @@ __device__ __forceinline__ bool leaf_ok(const RunsArgs &a, int v) {
          (!a.G.allow || (a.G.allow[v] & a.leaf_ubit));
 }
 
-// candidates of every run: the neighbours of its anchor's image
+// candidates of every run (the neighbours of its anchor's image), and in all the candidates of its
+// entries, the most entries there can be
 template <typename K>
 __global__ void __launch_bounds__(256) runs_degree_kernel(RunsArgs a) {
+  __shared__ u64 s_red[8];
   const Slot<K> *in = reinterpret_cast<const Slot<K> *>(a.child.slots);
   const bool failed = block_run_failed(a.err);
   const u64 runs = failed ? 0 : run_count(a);
+  const u64 n_in = a.leaf || failed ? 0 : child_bound<K>(a);
+  u64 most = 0;
   for (u64 r = blockIdx.x * 256ull + threadIdx.x; r < runs; r += gridDim.x * 256ull) {
     unsigned d = 0;
     int w = (int)r;
@@ -154,7 +159,10 @@ __global__ void __launch_bounds__(256) runs_degree_kernel(RunsArgs a) {
     if (!a.leaf || leaf_ok(a, w))
       d = a.anchor < 0 ? (unsigned)a.G.n : (unsigned)(a.G.row_ptr[w + 1] - a.G.row_ptr[w]);
     a.deg[r] = d;
+    most += d * (a.leaf ? (u64)a.trials : (r + 1 < runs ? a.first[r + 1] : n_in) - a.first[r]);
   }
+  most = block_sum<256>(most, s_red);
+  if (threadIdx.x == 0 && most) atomicAdd(a.n_most, most);
 }
 
 // One thread a pair: its record (the mapping it leads to with a marker bit above, its slot and

@@ -104,3 +104,40 @@ def test_little_room_once_is_not_remembered(pat, n, trials, retain, room_mb):
                     last = kinds(c, pid, cid, trials, want, retain=retain)
                 assert last == ref, left >> 20
         assert tight
+
+
+# the six-cycle: one introduce that is expected to yield just more than two entries a pair and yields
+# just fewer, one that is expected to yield fewer; the partial 2-tree: most mappings have several origins
+@pytest.mark.parametrize("pat,n,hubs,trials", [(("cycle", 6), 1500, 0, 8),
+                                               (("ktree", 7, 2, 5), 700, 1, 9)])
+def test_exact_runs_write_what_they_count(pat, n, hubs, trials):
+    """An exact run lists and counts a node's (run, candidate) pairs, or sorts them, only where it also
+    writes their entries: nothing is counted for the entry kernels to do again."""
+    p = synth.make_pattern(pat)
+    g = synth.barabasi_albert(n, 4, 3) if hubs else synth.erdos_renyi(n, 8 / n, 3)
+    z = oracle.colors(n, trials, p[0], seed=100)
+    want = oracle.run_dp(g, p, z, p[0])
+    with cc.Context(arena_bytes=8 << 30) as c:
+        cc.cc_load_graph(c.h, *g)
+        pid = cc.cc_load_pattern(c.h, *p)
+        N, _ = cc.cc_pattern_info(c.h, pid)
+        nodes = cc.cc_pattern_nodes(c.h, pid, p[0])
+        cid = cc.cc_set_colors(c.h, z, p[0])
+        for mode in ("exact", "planned"):
+            run = cc.cc_run_dp(c.h, pid, cid, cc.cc_default_opts(profile=1))
+            assert cc.cc_run_mode(c.h, run) == mode
+            assert np.array_equal(cc.cc_count(c.h, run, trials), want.count)
+            assert np.array_equal(cc.cc_table_stats(c.h, run, N)[0], want.node_sizes.sum(axis=0))
+            node, kind, _, _ = cc.cc_run_timings(c.h, run)
+            cc.cc_release(c.h, run)
+            if mode == "planned":
+                break
+            made = {(x, cc.KERNEL_KINDS[k]): int(((node == x) & (kind == k)).sum())
+                    for x, k in zip(node.tolist(), kind.tolist())}
+            for f, nd in enumerate(nodes):
+                if nd[0] == cc.FORGET and nodes[nd[1]][0] == cc.INTRODUCE:
+                    # pairs and side entries are sorted and reduced; else at most the runs are listed
+                    # before the entries are counted
+                    sorts, reduces = made.get((f, "sort"), 0), made.get((f, "reduce"), 0)
+                    assert sorts == reduces, f
+                    assert made.get((nd[1], "intro_count"), 0) <= (3 if sorts == 2 else 2), f
