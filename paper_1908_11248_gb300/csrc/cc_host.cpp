@@ -720,26 +720,32 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
           plan->entries[x] < cc::kRunYield * r.slots || 2 * r.more > plan->entries[x])
         return CC_OK;
     }
-    Held held{A, {}};
+    // On every way out: how far the attempt came; of one that was left nothing stays, neither a
+    // capacity to keep to nor its scratch in the run's peak (which later runs reserve).
     bool short_of = false;
+    struct Outcome {
+      Run &run;
+      Arena &arena;
+      cc::RunSizes &r;
+      const int &taken;
+      const bool &short_of;
+      bool exact;
+      size_t checks, peak;
+      ~Outcome() {
+        r.state = taken ? cc::Runwise::kDone : exact ? cc::Runwise::kLeft : r.state;
+        if (taken) return;
+        if (exact && short_of) run.starved = true;
+        run.checks.resize(checks);
+        arena.set_high_water(peak);
+      }
+    } outcome{*R, A, R->runwise[x], *taken, short_of, !planned, R->checks.size(), A.high_water()};
+    Held held{A, {}};
     auto hold = [&](size_t bytes) {
       void *q = A.alloc(std::max<size_t>(1, bytes));
       if (q) held.p.push_back(q);
       else short_of = true;
       return q;
     };
-    // on every way out: how far the attempt came
-    struct Outcome {
-      Run &run;
-      cc::RunSizes &r;
-      const int &taken;
-      const bool &short_of;
-      bool exact;
-      ~Outcome() {
-        r.state = taken ? cc::Runwise::kDone : exact ? cc::Runwise::kLeft : r.state;
-        if (exact && !taken && short_of) run.starved = true;
-      }
-    } outcome{*R, R->runwise[x], *taken, short_of, !planned};
     cc::RunsArgs r{};
     r.G = a.G;
     r.L = R->L;
@@ -824,7 +830,6 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (short_of) return CC_OK;
     r.n_pairs = w_pairs;
     r.n_total = words;
-    r.cand = a.cand;
     rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, 1,
                [&] { return cc::launch_runs_pairs(c->stream, c->dev, R->kw, r); });
     if (rc) return rc;
@@ -833,7 +838,6 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       if (rc) return rc;
       if (f >= 0 && few(*total) && !order_handed_on(f)) {  // counted, but better done entry by entry
         *counted = true;
-        CUDA_OK(cudaMemsetAsync(a.cand, 0, sizeof(u64), c->stream));
         return CC_OK;
       }
     } else {
@@ -933,6 +937,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       short_of = true;
       return CC_OK;
     }
+    if (R->opts.profile)  // candidates examined: every pair
+      CUDA_OK(cudaMemcpyAsync(a.cand, w_slots, sizeof(u64), cudaMemcpyDeviceToDevice, c->stream));
     const int z = f >= 0 ? f : x;
     R->tables[z] = {out, cap, 0, true};
     cc::NodeTable &t = R->tables[z];

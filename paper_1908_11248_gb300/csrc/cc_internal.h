@@ -169,7 +169,7 @@ struct RunsArgs {
   void *recs;                      // per pair: (mapping with a marker bit, slot | entries << 32)
   unsigned *prow;                  // per pair slot: its run and its candidate
   int *pv;
-  unsigned long long *n_pairs, *n_total, *cand;  // pairs that yield entries, those entries
+  unsigned long long *n_pairs, *n_total;  // pairs that yield entries, those entries
   // the pairs to write: as they are, or sorted by mapping (merge)
   const void *list;
   const unsigned long long *n_list;

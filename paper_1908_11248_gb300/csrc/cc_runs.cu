@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256) runs_pairs_kernel(RunsArgs a) {
   Slot<u64> *recs = reinterpret_cast<Slot<u64> *>(a.recs);
   const bool failed = block_run_failed(a.err);
   const u64 runs = failed ? 0 : run_count(a);
-  const u64 slots = failed ? 0 : *a.n_slots, pairs = min(slots, a.pair_cap);
+  const u64 pairs = failed ? 0 : min(*a.n_slots, a.pair_cap);
   const u64 n_in = a.leaf || failed ? 0 : child_bound<K>(a);
   const int T = a.trials, k = a.L.k, nb = a.L.nb;
   const uint32_t cmask = (uint32_t)((1ull << k) - 1ull);
@@ -236,7 +236,6 @@ __global__ void __launch_bounds__(256) runs_pairs_kernel(RunsArgs a) {
   if (threadIdx.x == 0 && valid) atomicAdd(a.n_pairs, valid);
   total = block_sum<256>(total, s_red);
   if (threadIdx.x == 0 && total) atomicAdd(a.n_total, total);
-  if (a.cand && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.cand, slots);
 }
 
 // pairs to write; a list with more than its room is not read at all (the run is repeated)

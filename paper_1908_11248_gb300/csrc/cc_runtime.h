@@ -96,6 +96,7 @@ class Arena {
   size_t in_use() const { return inuse_; }
   size_t high_water() const { return hw_; }
   void reset_high_water() { hw_ = inuse_; }
+  void set_high_water(size_t bytes) { hw_ = std::max(bytes, inuse_); }
   size_t largest_free() const {
     size_t s = 0;
     for (auto &f : free_) s = std::max(s, f.second);
