@@ -434,6 +434,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   R->pairs.assign(N, 0);
   R->runwise.assign(N, {});
   R->starved = false;
+  if (planned) R->learn_pairs = false;
   R->checks.clear();
   std::vector<bool> made(N, false);
   const int grid = cc::intro_grid(c->dev, block);
@@ -962,6 +963,159 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     return CC_OK;
   };
 
+  // Join x of two children sorted by (mapping, trial), group by group (cc_join.cu).  *taken: 0 if
+  // its scratch or its result does not fit, after which the children are what they were or sorted.
+  auto join_groups = [&](int x, int *taken) -> int {
+    *taken = 0;
+    const NiceNode &nd = P.nodes[x];
+    const int b = (int)nd.bag.size();
+    int y = nd.child0, z = nd.child1;
+    if (entries(y) > entries(z)) std::swap(y, z);  // y's groups look theirs up in z
+    // the order both must have: that of a child sorted by all its slots (the larger one's if
+    // both are), else the one the parent likes best
+    auto sorted_full = [&](int v) {
+      const cc::NodeTable &t = R->tables[v];
+      return !t.hashed && t.sort_n == b && t.sort_hbits == 0 && !t.regions;
+    };
+    cc::SortSpec sp = forget_order(x);
+    const int lead = sorted_full(z) ? z : sorted_full(y) ? y : -1;
+    if (lead >= 0)
+      for (int j = 0; j < b; ++j) sp.order[j] = R->tables[lead].sort_slots[j];
+    sp.nsl = b;
+    sp.full = 0;
+    sp.trial = 1;
+    sp.bits = b * R->L.nb + R->L.tb;
+    Held held{A, {}};
+    auto in_order = [&](int v, TableDesc *t) -> int {
+      const cc::NodeTable &ty = R->tables[v];
+      bool as_is = sorted_full(v);
+      for (int j = 0; j < b && as_is; ++j) as_is = ty.sort_slots[j] == sp.order[j];
+      *t = desc(v);
+      if (as_is) return CC_OK;
+      const u64 m = entries(v);
+      void *s = nullptr;
+      check(R->d_counters + v, m);
+      const int r = sort_records(x, sp, ty.slots, ty.hashed ? c->d_ones : t->count, ty.cap,
+                                 R->d_counters + v, m, &s);
+      if (r) {
+        A.release(s);
+        return r;
+      }
+      *t = TableDesc{s, std::max<u64>(1, m), R->d_counters + v, 0};
+      if (R->opts.retain) {
+        held.p.push_back(s);
+        return CC_OK;
+      }
+      release_child(v);  // the sorted records take the table's place
+      R->tables[v] = {s, t->cap, 0, true};
+      R->tables[v].sort_n = b;
+      for (int j = 0; j < b; ++j) R->tables[v].sort_slots[j] = sp.order[j];
+      return CC_OK;
+    };
+    cc::JoinGroupArgs a{};
+    a.G = G;
+    a.L = R->L;
+    a.sp = sp;
+    a.bag = b;
+    a.err = R->d_err;
+    int r = in_order(y, &a.a);
+    if (!r) r = in_order(z, &a.b);
+    if (r) return r == CC_ENOMEM ? CC_OK : r;
+    bool short_of = false;
+    auto hold = [&](size_t bytes) {
+      void *q = A.alloc(bytes);
+      if (q) held.p.push_back(q);
+      else short_of = true;
+      return q;
+    };
+    a.groups = (u64 *)hold(sizeof(u64));
+    a.first = (u64 *)hold(a.a.cap * sizeof(u64));
+    a.blo = (u64 *)hold(a.a.cap * sizeof(u64));
+    a.blen = (unsigned *)hold(a.a.cap * sizeof(unsigned));
+    a.cnt = (unsigned *)hold(a.a.cap * sizeof(unsigned));
+    u64 *off = (u64 *)hold(a.a.cap * sizeof(u64));
+    u64 *scan = (u64 *)hold(cc::scan_scratch_words(c->dev) * sizeof(u64));
+    if (short_of) return CC_OK;
+    a.off = off;
+    r = timed(x, CC_K_JOIN_BUILD, 4,
+              [&] { return cc::launch_join_match(c->stream, c->dev, R->kw, a, blk); });
+    if (r) return r;
+    r = timed(x, CC_K_JOIN_COUNT, 4, [&] {
+      const int e = cc::launch_join_groups(c->stream, c->dev, R->kw, 0, a);
+      return e ? e : cc::launch_scan_u32(c->stream, c->dev, a.cnt, a.a.cap, off, scan, a.groups,
+                                         R->d_counters + x);
+    });
+    if (r) return r;
+    u64 total = planned ? room(plan->entries[x]) : 0;
+    if (!planned) r = read_u64(c, R->d_counters + x, &total);
+    if (r) return r;
+    const u64 cap = std::max<u64>(1, total);
+    void *p = A.alloc(cap * rb);
+    if (!p) {  // (the hash table's counter starts at 0)
+      CUDA_OK(cudaMemsetAsync(R->d_counters + x, 0, sizeof(u64), c->stream));
+      return CC_OK;
+    }
+    R->tables[x] = {p, cap, 0, true};
+    R->tables[x].sort_n = b;
+    for (int j = 0; j < b; ++j) R->tables[x].sort_slots[j] = sp.order[j];
+    check(R->d_counters + x, cap);
+    a.out = desc(x);
+    r = timed(x, CC_K_JOIN_WRITE, 1,
+              [&] { return cc::launch_join_groups(c->stream, c->dev, R->kw, 1, a); });
+    *taken = !r;
+    return r;
+  };
+
+  // Join x through hash tables: the smaller child's entries chained by (mapping, trial), the other's
+  // probing the chains.
+  auto join_hashed = [&](int x) -> int {
+    const NiceNode &nd = P.nodes[x];
+    int rc = CC_OK;
+    int y = nd.child0, z = nd.child1;
+    if (entries(y) > entries(z)) std::swap(y, z);  // chain the smaller child
+    u64 icap = hash_cap(entries(y), lf);
+    u64 bound_y = R->tables[y].hashed || planned ? R->tables[y].cap : R->sizes[y];
+    void *index = A.alloc(icap * cc::index_slot_bytes(R->kw));
+    u64 *next = arena_alloc<u64>(c, std::max<u64>(1, bound_y));
+    if (!index || !next) {
+      A.release(index);
+      A.release(next);
+      return CC_ENOMEM;
+    }
+    CUDA_OK(cudaMemsetAsync(index, 0, icap * cc::index_slot_bytes(R->kw), c->stream));
+    u64 *pairs = pairs_dev + x;
+    cc::JoinArgs a{};
+    a.G = G;
+    a.L = R->L;
+    a.build = desc(y);
+    a.probe = desc(z);
+    a.b = (int)nd.bag.size();
+    a.index = index;
+    a.index_cap = icap;
+    a.next = next;
+    a.pairs = pairs;
+    a.err = R->d_err;
+    rc = timed(x, CC_K_JOIN_BUILD, 1,
+               [&] { return cc::launch_join(c->stream, c->dev, R->kw, 0, block, a); });
+    u64 np = 0;
+    if (!rc && !planned) {
+      rc = timed(x, CC_K_JOIN_COUNT, 1,
+                 [&] { return cc::launch_join(c->stream, c->dev, R->kw, 1, block, a); });
+      if (!rc) rc = read_u64(c, pairs, &np);
+      R->pairs[x] = np;
+    }
+    if (planned) np = room(plan->pairs[x]);
+    if (!rc) rc = new_hash(x, np);
+    if (!rc) {
+      a.out = desc(x);
+      rc = timed(x, CC_K_JOIN_WRITE, 1,
+                 [&] { return cc::launch_join(c->stream, c->dev, R->kw, 2, block, a); });
+    }
+    A.release(index);
+    A.release(next);
+    return rc;
+  };
+
   for (int x = 0; x < N; ++x) {
     if (made[x]) continue;
     const NiceNode &nd = P.nodes[x];
@@ -1349,138 +1503,25 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
                  [&] { return cc::launch_forget(c->stream, c->dev, R->kw, block, a); });
       if (rc) return rc;
       release_child(y);
-    } else if (!R->frugal && R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
-               entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries) {
-      // join, group by group (cc_join.cu)
-      const int b = (int)nd.bag.size();
-      int y = nd.child0, z = nd.child1;
-      if (entries(y) > entries(z)) std::swap(y, z);  // y's groups look theirs up in z
-      // the order both must have: that of a child sorted by all its slots (the larger one's if
-      // both are), else the one the parent likes best
-      auto sorted_full = [&](int v) {
-        const cc::NodeTable &t = R->tables[v];
-        return !t.hashed && t.sort_n == b && t.sort_hbits == 0 && !t.regions;
-      };
-      cc::SortSpec sp = forget_order(x);
-      const int lead = sorted_full(z) ? z : sorted_full(y) ? y : -1;
-      if (lead >= 0)
-        for (int j = 0; j < b; ++j) sp.order[j] = R->tables[lead].sort_slots[j];
-      sp.nsl = b;
-      sp.full = 0;
-      sp.trial = 1;
-      sp.bits = b * R->L.nb + R->L.tb;
-      Held held{A, {}};
-      auto in_order = [&](int v, TableDesc *t) -> int {
-        const cc::NodeTable &ty = R->tables[v];
-        bool as_is = sorted_full(v);
-        for (int j = 0; j < b && as_is; ++j) as_is = ty.sort_slots[j] == sp.order[j];
-        *t = desc(v);
-        if (as_is) return CC_OK;
-        const u64 m = entries(v);
-        void *s = nullptr;
-        check(R->d_counters + v, m);
-        const int r = sort_records(x, sp, ty.slots, ty.hashed ? c->d_ones : t->count, ty.cap,
-                                   R->d_counters + v, m, &s);
-        held.p.push_back(s);
-        if (r) return r;
-        *t = TableDesc{s, std::max<u64>(1, m), R->d_counters + v, 0};
-        release_child(v);
-        return CC_OK;
-      };
-      cc::JoinGroupArgs a{};
-      a.G = G;
-      a.L = R->L;
-      a.sp = sp;
-      a.bag = b;
-      a.err = R->d_err;
-      rc = in_order(y, &a.a);
-      if (!rc) rc = in_order(z, &a.b);
-      if (rc) return rc;
-      auto hold = [&](size_t bytes) {
-        held.p.push_back(A.alloc(bytes));
-        return held.p.back();
-      };
-      a.groups = (u64 *)hold(sizeof(u64));
-      a.first = (u64 *)hold(a.a.cap * sizeof(u64));
-      a.blo = (u64 *)hold(a.a.cap * sizeof(u64));
-      a.blen = (unsigned *)hold(a.a.cap * sizeof(unsigned));
-      a.cnt = (unsigned *)hold(a.a.cap * sizeof(unsigned));
-      u64 *off = (u64 *)hold(a.a.cap * sizeof(u64));
-      u64 *scan = (u64 *)hold(cc::scan_scratch_words(c->dev) * sizeof(u64));
-      for (void *q : held.p)
-        if (!q) return CC_ENOMEM;
-      a.off = off;
-      rc = timed(x, CC_K_JOIN_BUILD, 4,
-                 [&] { return cc::launch_join_match(c->stream, c->dev, R->kw, a, blk); });
-      if (rc) return rc;
-      rc = timed(x, CC_K_JOIN_COUNT, 4, [&] {
-        const int r = cc::launch_join_groups(c->stream, c->dev, R->kw, 0, a);
-        return r ? r : cc::launch_scan_u32(c->stream, c->dev, a.cnt, a.a.cap, off, scan, a.groups,
-                                           R->d_counters + x);
-      });
-      if (rc) return rc;
-      u64 total = planned ? room(plan->entries[x]) : 0;
-      if (!planned) rc = read_u64(c, R->d_counters + x, &total);
-      if (rc) return rc;
-      const u64 cap = std::max<u64>(1, total);
-      void *p = A.alloc(cap * rb);
-      if (!p) return CC_ENOMEM;
-      R->tables[x] = {p, cap, 0, true};
-      R->tables[x].sort_n = b;
-      for (int j = 0; j < b; ++j) R->tables[x].sort_slots[j] = sp.order[j];
-      check(R->d_counters + x, cap);
-      a.out = desc(x);
-      rc = timed(x, CC_K_JOIN_WRITE, 1,
-                 [&] { return cc::launch_join_groups(c->stream, c->dev, R->kw, 1, a); });
-      if (rc) return rc;
-      release_child(y);
-      release_child(z);
-    } else {  // join through hash tables
-      int y = nd.child0, z = nd.child1;
-      if (entries(y) > entries(z)) std::swap(y, z);  // chain the smaller child
-      u64 icap = hash_cap(entries(y), lf);
-      u64 bound_y = R->tables[y].hashed || planned ? R->tables[y].cap : R->sizes[y];
-      void *index = A.alloc(icap * cc::index_slot_bytes(R->kw));
-      u64 *next = arena_alloc<u64>(c, std::max<u64>(1, bound_y));
-      if (!index || !next) {
-        A.release(index);
-        A.release(next);
-        return CC_ENOMEM;
+    } else {  // join: group by group, or through hash tables
+      int joined = 0;
+      if (!R->frugal && !R->learn_pairs && R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
+          entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries) {
+        rc = join_groups(x, &joined);
+        if (rc) return rc;
       }
-      CUDA_OK(cudaMemsetAsync(index, 0, icap * cc::index_slot_bytes(R->kw), c->stream));
-      u64 *pairs = pairs_dev + x;
-      cc::JoinArgs a{};
-      a.G = G;
-      a.L = R->L;
-      a.build = desc(y);
-      a.probe = desc(z);
-      a.b = (int)nd.bag.size();
-      a.index = index;
-      a.index_cap = icap;
-      a.next = next;
-      a.pairs = pairs;
-      a.err = R->d_err;
-      rc = timed(x, CC_K_JOIN_BUILD, 1,
-                 [&] { return cc::launch_join(c->stream, c->dev, R->kw, 0, block, a); });
-      u64 np = 0;
-      if (!rc && !planned) {
-        rc = timed(x, CC_K_JOIN_COUNT, 1,
-                   [&] { return cc::launch_join(c->stream, c->dev, R->kw, 1, block, a); });
-        if (!rc) rc = read_u64(c, pairs, &np);
-        R->pairs[x] = np;
+      if (!joined) {
+        // the matching pairs of a join that exact runs made group by group are not known: the exact
+        // run that follows counts them
+        if (planned && !plan->pairs[x] && plan->entries[x]) {
+          R->learn_pairs = true;
+          return CC_ENOMEM;
+        }
+        rc = join_hashed(x);
+        if (rc) return rc;
       }
-      if (planned) np = room(plan->pairs[x]);
-      if (!rc) rc = new_hash(x, np);
-      if (!rc) {
-        a.out = desc(x);
-        rc = timed(x, CC_K_JOIN_WRITE, 1,
-                   [&] { return cc::launch_join(c->stream, c->dev, R->kw, 2, block, a); });
-      }
-      A.release(index);
-      A.release(next);
-      if (rc) return rc;
-      release_child(y);
-      release_child(z);
+      release_child(nd.child0);
+      release_child(nd.child1);
     }
     if (!planned) {
       rc = read_u64(c, R->d_counters + x, &R->sizes[x]);

@@ -166,3 +166,48 @@ def test_exact_runs_write_what_they_count(pat, n, hubs, trials):
                     sorts, reduces = made.get((f, "sort"), 0), made.get((f, "reduce"), 0)
                     assert sorts == reduces, f
                     assert made.get((nd[1], "intro_count"), 0) <= (3 if sorts == 2 else 2), f
+
+
+def test_join_without_room_to_sort():
+    """A join of a large unsorted child with a small one (allowed mappings) where sorting the large one
+    does not fit: it goes through hash tables, whose need is the small child's, in the same run."""
+    n, trials, k = 16_000, 7, 6
+    nF, edges, _ = synth.star_pattern(4)
+    pat = nF, edges, ([[0, i] for i in range(1, 4)], [-1, 0, 0])
+    g = synth.erdos_renyi(n, 8 / n, 6)
+    z = oracle.colors(n, trials, k, seed=5)
+    allow = np.full(n, 0b1011, np.uint32)
+    allow[::1000] |= 0b0100  # vertex 2 on a few host vertices
+    want = oracle.run_dp(g, pat, z, k, allow=allow)
+    with cc.Context(arena_bytes=1 << 30) as c:
+        cc.cc_load_graph(c.h, *g)
+        cid = cc.cc_set_colors(c.h, z, k)
+        pid = cc.cc_load_pattern_masked(c.h, *pat, allow)
+        nodes = cc.cc_pattern_nodes(c.h, pid, nF)
+        join = [x for x, nd in enumerate(nodes) if nd[0] == cc.JOIN]
+        assert len(join) == 1
+        sizes = want.node_sizes.sum(axis=0)
+        large = max(int(sizes[nodes[join[0]][1]]), int(sizes[nodes[join[0]][2]]))
+        assert large > 1 << 21
+        _, used, size = cc.cc_context_stats(c.h)
+        hashed, was_planned = 0, True
+        parts = list(range(60, 19, -2))  # the room in tenths of the large table's records
+        pids = [cc.cc_load_pattern_masked(c.h, *pat, allow) for _ in parts]  # a key each
+        for part, pid in zip(parts, pids):
+            left = 16 * large * part // 10
+            used = cc.cc_context_stats(c.h)[1]
+            held = cc.cc_color(c.h, 1, (size - used - left) // n, k)
+            for rep in range(4):
+                run = cc.cc_run_dp(c.h, pid, cid, cc.cc_default_opts(profile=1))
+                mode = cc.cc_run_mode(c.h, run)
+                assert np.array_equal(cc.cc_count(c.h, run, trials), want.count)
+                assert np.array_equal(cc.cc_table_stats(c.h, run, len(nodes))[0], sizes)
+                node, kind, _, _ = cc.cc_run_timings(c.h, run)
+                cc.cc_release(c.h, run)
+                assert mode in ("exact", "planned"), part
+                groups = (node == join[0]) & (kind == cc.KERNEL_KINDS.index("join_count"))
+                hashed += mode == "planned" and not groups.any()
+            assert was_planned or mode == "exact", part  # planned down to some room
+            was_planned = mode == "planned"
+            cc.cc_release_colors(c.h, held)
+        assert hashed
