@@ -434,6 +434,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   R->pairs.assign(N, 0);
   R->runwise.assign(N, {});
   R->starved = false;
+  R->beside = 0;
   if (planned) R->learn_pairs = false;
   R->checks.clear();
   std::vector<bool> made(N, false);
@@ -687,6 +688,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       void *t = A.alloc(std::max<size_t>(1, (size_t)R->trials * (size_t)n));
       if (!t) return CC_ENOMEM;
       transposed.p.push_back(t);
+      R->beside = (size_t)R->trials * (size_t)n;
       if (cc::launch_runs_colours(c->stream, c->dev, col.d_colors, n, R->trials, (uint8_t *)t))
         return CC_ECUDA;
       c->launches++;
@@ -1340,7 +1342,12 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         fuse = 1;
       if (fuse == 1) {  // add projected entries into the forget's hash table
         rc = new_hash(f, planned ? room(plan->entries[f]) : total);
-        if (rc) return rc;
+        if (rc == CC_ENOMEM && R->opts.fuse == 2) fuse = 2;  // no room for it: sorted after all
+        else if (rc) return rc;
+        else if (R->opts.fuse == 2)
+          R->tables[f].beside = (size_t)(R->tables[f].cap - std::min(R->tables[f].cap, raw)) * rb;
+      }
+      if (fuse == 1) {
         a.out = desc(f);
         a.q = pos_in(nd.bag, P.nodes[f].vertex);
         a.valid = R->d_counters + x;
@@ -2098,11 +2105,20 @@ void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t
   plan.runs++;
 }
 
+// True if run R, out of memory, held at least what it lacked in what a frugal run does without:
+// hash tables of few entries (larger than the sorted records) and transposed colours.  The other
+// routes with scratch beside the tables have given it up by themselves.
+bool held_beside(const Run *R, const Arena &A) {
+  size_t bytes = R->beside;
+  for (const auto &t : R->tables) bytes += t.beside;
+  return bytes > 0 && A.lacked() <= bytes;
+}
+
 // Runs the nodes on the context's stream: planned when a plan exists (repeated exactly if the
 // plan proves too small), exact otherwise; then reads the results and updates the plan.  A run
 // that nothing could make smaller (its tables are kept, or it is a single trial) and that runs
-// out of memory is repeated without the routes that hold scratch beside the tables (Run::frugal),
-// so that a context in which the tables just fit still counts them; the plan remembers it.
+// out of memory for what it holds beside the tables is repeated without that (Run::frugal), so
+// that a context in which the tables just fit still counts them; the plan remembers it.
 int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long long> &key,
                bool exact_only) {
   const Pattern &P = c->patterns.at(R->pattern);
@@ -2131,7 +2147,7 @@ int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long l
     rc = run_nodes(c, R, P, col, nullptr);
     if (!rc) rc = finish_run(c, R);
   }
-  if (rc == CC_ENOMEM && !R->frugal && (R->retained || R->trials == 1)) {
+  if (rc == CC_ENOMEM && !R->frugal && (R->retained || R->trials == 1) && held_beside(R, A)) {
     R->frugal = true;
     rc = reset_run(c, R, N);
     A.reset_high_water();
@@ -2327,9 +2343,9 @@ int run_sliced(Ctx *c, Run *R, const cc::Coloring &view, int32_t t0,
                const std::vector<long long> &ckey, int s0);
 
 // Trials [t0, t0 + nt) of run R as a run of their own over their rows of the colouring; if
-// they do not fit either, each half in turn, and a single trial in slices (run_sliced).
-// Per-trial results do not depend on the other trials, so the chunk's exists flags and counts
-// are R's, and table sizes add over chunks.
+// they do not fit either, each half in turn, and a single trial in slices (run_sliced; at once
+// if it is all of R, which did not fit).  Per-trial results do not depend on the other trials, so
+// the chunk's exists flags and counts are R's, and table sizes add over chunks.
 int run_chunk(Ctx *c, Run *R, const cc::Coloring &col, int32_t t0, int32_t nt) {
   cc::Coloring view;
   view.trials = nt;
@@ -2340,9 +2356,10 @@ int run_chunk(Ctx *c, Run *R, const cc::Coloring &col, int32_t t0, int32_t nt) {
   int rc = init_run(c, R->pattern, view, -1, &R->opts, S, key);
   if (rc) return rc;
   auto pl = c->plans.find(key);
-  if (nt == 1 && pl != c->plans.end() && pl->second.slices > 0) {  // known not to fit whole
+  const int slices = pl != c->plans.end() ? pl->second.slices : 0;
+  if (nt == 1 && (slices > 0 || R->trials == 1)) {  // known not to fit whole
     free_run(c, S.get());
-    return run_sliced(c, R, view, t0, key, pl->second.slices);
+    return run_sliced(c, R, view, t0, key, slices > 0 ? slices : 2);
   }
   rc = run_direct(c, S.get(), view, key, false);
   if (!rc) {

@@ -29,7 +29,7 @@ class Arena {
     size_ = size;
     free_.clear();
     used_.clear();
-    inuse_ = hw_ = top_ = 0;
+    inuse_ = hw_ = top_ = lacked_ = 0;
     if (size) free_[0] = size;
   }
   void *alloc(size_t bytes) {
@@ -46,8 +46,12 @@ class Arena {
       if (off + bytes > top_) top_ = off + bytes;
       return base_ + off;
     }
+    const size_t have = free_bytes();
+    lacked_ = bytes > have ? bytes - have : 0;
     return nullptr;
   }
+  // bytes that the last block refused was larger than all that was free (0: in pieces, it was not)
+  size_t lacked() const { return lacked_; }
   void release(void *p) {
     if (!p) return;
     size_t off = (char *)p - base_;
@@ -105,7 +109,7 @@ class Arena {
 
  private:
   char *base_ = nullptr;
-  size_t size_ = 0, inuse_ = 0, hw_ = 0, top_ = 0;
+  size_t size_ = 0, inuse_ = 0, hw_ = 0, top_ = 0, lacked_ = 0;
   std::map<size_t, size_t> free_, used_;
 };
 
@@ -164,6 +168,8 @@ struct NodeTable {
   int cluster_slots[kMaxBag] = {};
   // scan bound of a dense table written in chunks (holes up to it); null: the entry counter
   unsigned long long *bound = nullptr;
+  // a hash table of few entries: its bytes beyond those of the sorted records in its place
+  size_t beside = 0;
 };
 
 // What an introduce taken run by run (cc_runs.cu) met: (run, candidate) pairs, those that yield
@@ -218,6 +224,7 @@ struct Run {
   bool graphed = false;
   bool streamed = false;  // its trials ran in chunks (all at once did not fit)
   bool frugal = false;    // no route that holds scratch beside the tables (see run_direct)
+  size_t beside = 0;      // bytes of transposed colours
   size_t room = 0;        // free arena bytes when it started
   bool starved = false;   // an introduce run by run was left for want of memory (exact runs)
   bool learn_pairs = false;  // a planned attempt had to join through hash tables without knowing how

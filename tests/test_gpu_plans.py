@@ -211,3 +211,33 @@ def test_join_without_room_to_sort():
             was_planned = mode == "planned"
             cc.cc_release_colors(c.h, held)
         assert hashed
+
+
+@pytest.mark.parametrize("retain", [0, 1])
+@pytest.mark.parametrize("pat", [("A",), ("cycle", 5)])
+def test_run_that_does_not_fit_is_tried_once(pat, retain):
+    """A single trial too large for the room (and not to be sliced) ends with CC_ENOMEM after one
+    attempt; a second one is made only where what the first held beside its tables is what it
+    lacked, which is rare."""
+    p = synth.make_pattern(pat)
+    n = 20_000
+    g = synth.barabasi_albert(n, 4, 3)
+    z = oracle.colors(n, 1, p[0], seed=5)
+    opts = cc.cc_default_opts(retain=retain, max_slices=1)
+    full, spent = 0, []
+    mb = 4096.0
+    while mb > 8:
+        with cc.Context(arena_bytes=int(mb * 2 ** 20)) as c:
+            cc.cc_load_graph(c.h, *g)
+            pid = cc.cc_load_pattern(c.h, *p)
+            cid = cc.cc_set_colors(c.h, z, p[0])
+            before = cc.cc_context_stats(c.h)[0]
+            try:
+                cc.cc_run_dp(c.h, pid, cid, opts)
+                full = full or cc.cc_context_stats(c.h)[0] - before
+            except cc.CCError as ex:
+                assert ex.code == cc.CC_ENOMEM
+                spent.append(cc.cc_context_stats(c.h)[0] - before)
+        mb /= 1.2
+    assert full and spent
+    assert np.mean([s > full for s in spent]) < 0.25, (full, spent)
