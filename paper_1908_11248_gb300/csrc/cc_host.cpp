@@ -2117,10 +2117,12 @@ bool held_beside(const Run *R, const Arena &A) {
 // Runs the nodes on the context's stream: planned when a plan exists (repeated exactly if the
 // plan proves too small), exact otherwise; then reads the results and updates the plan.  A run
 // that nothing could make smaller (its tables are kept, or it is a single trial) and that runs
-// out of memory for what it holds beside the tables is repeated without that (Run::frugal), so
-// that a context in which the tables just fit still counts them; the plan remembers it.
+// out of memory for what it holds beside the tables is at last repeated without that
+// (Run::frugal), so that a context in which the tables just fit still counts them.  The plan
+// remembers in how much room: with more of it (another run released, graphs given back, the
+// server's other queries done) the key runs as any other.
 int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long long> &key,
-               bool exact_only) {
+               bool exact_only, bool last) {
   const Pattern &P = c->patterns.at(R->pattern);
   const int N = (int)P.nodes.size();
   int rc = reset_run(c, R, N);
@@ -2130,7 +2132,7 @@ int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long l
   R->room = A.free_bytes();
   R->planned = !exact_only && pl != c->plans.end() && plan_ready(pl->second, R->room);
   R->graphed = false;
-  R->frugal = pl != c->plans.end() && pl->second.frugal;
+  R->frugal = pl != c->plans.end() && R->room <= pl->second.frugal[R->retained];
   const size_t base = A.in_use();
   A.reset_high_water();
   if (R->planned) {
@@ -2147,13 +2149,14 @@ int run_direct(Ctx *c, Run *R, const cc::Coloring &col, const std::vector<long l
     rc = run_nodes(c, R, P, col, nullptr);
     if (!rc) rc = finish_run(c, R);
   }
-  if (rc == CC_ENOMEM && !R->frugal && (R->retained || R->trials == 1) && held_beside(R, A)) {
+  if (rc == CC_ENOMEM && last && !R->frugal && (R->retained || R->trials == 1) &&
+      held_beside(R, A)) {
     R->frugal = true;
     rc = reset_run(c, R, N);
     A.reset_high_water();
     if (!rc) rc = run_nodes(c, R, P, col, nullptr);
     if (!rc) rc = finish_run(c, R);
-    if (!rc) c->plans[key].frugal = true;
+    if (!rc) c->plans[key].frugal[R->retained] = R->room;
   }
   if (rc) return rc;
   update_plan(c, key, R, A.high_water() - base);
@@ -2255,7 +2258,6 @@ int capture_graph(Ctx *c, const std::vector<Run *> &Rs,
     S->trials = R->trials;
     S->home = &gm.sub;
     S->planned = true;
-    S->frugal = c->plans.at(keys[m]).frugal;
     S->d_counters = (u64 *)gm.sub.alloc(cc::kWords * N * sizeof(u64));
     S->d_exists = (unsigned *)gm.sub.alloc(R->trials * sizeof(unsigned));
     S->d_count = (u64 *)gm.sub.alloc(R->trials * sizeof(u64));
@@ -2271,6 +2273,7 @@ int capture_graph(Ctx *c, const std::vector<Run *> &Rs,
     c->stream = M > 1 ? c->branches[m] : main;
     c->active = &gm.sub;
     rc = reset_run(c, S, (int)N);
+    S->frugal = gm.sub.free_bytes() <= c->plans.at(keys[m]).frugal[0];
     if (!rc) rc = run_nodes(c, S, P, view, &c->plans.at(keys[m]));
     c->stream = origin;
     c->active = nullptr;
@@ -2361,7 +2364,7 @@ int run_chunk(Ctx *c, Run *R, const cc::Coloring &col, int32_t t0, int32_t nt) {
     free_run(c, S.get());
     return run_sliced(c, R, view, t0, key, slices > 0 ? slices : 2);
   }
-  rc = run_direct(c, S.get(), view, key, false);
+  rc = run_direct(c, S.get(), view, key, false, true);
   if (!rc) {
     if (cudaMemcpyAsync(R->d_exists + t0, S->d_exists, nt * sizeof(unsigned),
                         cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess ||
@@ -2430,7 +2433,7 @@ int run_sliced(Ctx *c, Run *R, const cc::Coloring &view, int32_t t0,
       key.push_back(-2);
       key.push_back(s);
       key.push_back(i);
-      rc = run_direct(c, S.get(), view, key, false);
+      rc = run_direct(c, S.get(), view, key, false, true);
       u64 hc = 0;
       unsigned he = 0;
       if (!rc &&
@@ -2496,10 +2499,10 @@ int run_split(Ctx *c, Run *R, const cc::Coloring &col) {
 // trials together do not fit.
 int run_one(Ctx *c, Run *R, const std::vector<long long> &key) {
   const cc::Coloring &col = c->colorings.at(R->coloring);
-  int rc = run_direct(c, R, col, key, false);
+  int rc = run_direct(c, R, col, key, false, c->graphs.empty());
   if (rc == CC_ENOMEM && !c->graphs.empty()) {
     drop_all_graphs(c);
-    rc = run_direct(c, R, col, key, false);
+    rc = run_direct(c, R, col, key, false, true);
   }
   if (rc == CC_ENOMEM && !R->retained) rc = run_split(c, R, col);
   return rc;
@@ -2516,6 +2519,14 @@ int run_graphed(Ctx *c, const std::vector<Run *> &Rs,
     gkey.push_back(-1);
   }
   auto it = c->graphs.find(gkey);
+  if (it != c->graphs.end())  // captured in little room, and there is more now: captured anew
+    for (size_t m = 0; m < Rs.size(); ++m)
+      if (it->second->members[m].shadow->frugal &&
+          c->arena.largest_free() > c->plans.at(keys[m]).frugal[0]) {
+        drop_graph(c, gkey);
+        it = c->graphs.end();
+        break;
+      }
   if (it == c->graphs.end()) {
     std::unique_ptr<cc::GraphSet> gs;
     int rc = capture_graph(c, Rs, keys, gs);

@@ -191,7 +191,10 @@ struct Plan {
   // room in which the last exact run left an introduce run by run for want of memory (0: in none):
   // with twice that room the key is planned anew
   size_t starved = 0;
-  bool frugal = false;  // its runs leave out the routes that hold scratch beside the tables
+  // room in which a run of this key ran out of memory and then fitted without the routes that
+  // hold memory beside the tables (0: none did): runs with no more room leave them out at once.
+  // Of runs that keep no tables, of runs that do.
+  size_t frugal[2] = {0, 0};
   size_t refused = 0;  // a served run of this key ran out of memory in a range this large
   int slices = 0;      // a single trial of this key fitted once split into this many slices
 };
@@ -223,7 +226,7 @@ struct Run {
   bool planned = false;
   bool graphed = false;
   bool streamed = false;  // its trials ran in chunks (all at once did not fit)
-  bool frugal = false;    // no route that holds scratch beside the tables (see run_direct)
+  bool frugal = false;    // no route that holds memory beside the tables (see run_direct)
   size_t beside = 0;      // bytes of transposed colours
   size_t room = 0;        // free arena bytes when it started
   bool starved = false;   // an introduce run by run was left for want of memory (exact runs)
@@ -329,9 +332,11 @@ bool plan_ready(const Plan &plan, size_t room);
 // Folds a finished run's sizes (and its arena peak) into the plan of its key.
 void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t peak);
 // Runs R to completion on the context's stream: planned if a plan exists and exact_only is
-// false (exactly again if it proves too small), else exactly; updates the plan.
+// false (exactly again if it proves too small), else exactly; updates the plan.  `last`: no memory
+// can be had by waiting or by giving something back, so a run that lacks some may go without the
+// routes that hold memory beside the tables.
 int run_direct(Ctx *c, Run *R, const Coloring &col, const std::vector<long long> &key,
-               bool exact_only);
+               bool exact_only, bool last);
 // Runs R (tables not kept) after it ran out of memory: its trials in halves, and a single trial
 // split by the image of one pattern vertex into slices that fit (results exact; table sizes add
 // over chunks and slices).

@@ -244,7 +244,7 @@ Outcome issue(Server *S, Ctx *c, ServeSlot &sl, const ServeQuery &q, bool alone)
       } else if (split) {
         rc = CC_ENOMEM;  // wait until it runs alone
       } else {
-        rc = rt::run_direct(c, sl.run.get(), sl.view, sl.key, !planned_enum);
+        rc = rt::run_direct(c, sl.run.get(), sl.view, sl.key, !planned_enum, alone);
         if (rc == CC_ENOMEM && alone && q.limit == 0) {
           {
             std::lock_guard<std::mutex> g2(S->mu);

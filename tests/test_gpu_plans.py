@@ -92,14 +92,16 @@ def kinds(c, pid, cid, trials, want, cand, **opt):
 
 
 # many colourings: introduces run by run, which hold pairs beside the tables, and (in the partial
-# 2-tree, where most mappings have several origins) more than the entry kernels would
+# 2-tree, where most mappings have several origins) more than the entry kernels would; one: forgets
+# of few entries, whose hash tables are larger than sorted records
 @pytest.mark.parametrize("pat,n,trials,retain,room_mb", [
-    (("grid", 2, 4), 1500, 9, 0, 1024), (("ktree", 7, 2, 5), 700, 9, 0, 512)])
+    (("grid", 2, 4), 1500, 9, 0, 1024), (("ktree", 7, 2, 5), 700, 9, 0, 512),
+    (("A",), 4000, 1, 1, 1024), (("path", 8), 3000, 1, 1, 128)])
 def test_little_room_once_is_not_remembered(pat, n, trials, retain, room_mb):
     """A key whose first runs had only part of the arena (another colouring held the rest) runs, once
     that is given back, by the same kernels as a key that had all of it from the start."""
     p = synth.make_pattern(pat)
-    g = synth.barabasi_albert(n, 4, 3)
+    g = synth.barabasi_albert(n, 4, 3) if pat[0] != "path" else synth.erdos_renyi(n, 6 / n, 3)
     z = oracle.colors(n, trials, p[0], seed=5)
     want = oracle.run_dp(g, p, z, p[0])
     with cc.Context(arena_bytes=room_mb << 20) as c:
@@ -129,6 +131,50 @@ def test_little_room_once_is_not_remembered(pat, n, trials, retain, room_mb):
                     last = kinds(c, pid, cid, trials, want, cand, retain=retain)
                 assert last == ref, left >> 20
         assert tight
+
+
+def test_graphs_give_way_before_routes():
+    """A run whose tables fit only without the routes that hold memory beside them, while a captured
+    graph holds some, takes the graph's memory and keeps the routes."""
+    p, n = synth.path_pattern(8), 3000
+    g = synth.erdos_renyi(n, 6 / n, 3)
+    z = oracle.colors(n, 1, 8, seed=5)
+    want = oracle.run_dp(g, p, z, 8)
+    with cc.Context(arena_bytes=256 << 20) as c:
+        cc.cc_load_graph(c.h, *g)
+        cid = cc.cc_set_colors(c.h, z, 8)
+        ref = kinds(c, cc.cc_load_pattern(c.h, *p), cid, 1, want, {}, retain=1)
+        other = cc.cc_load_pattern(c.h, *synth.path_pattern(6))
+        many = cc.cc_color(c.h, 2, 8, 6)
+        for mode in ("exact", "graph"):
+            run = cc.cc_run_dp(c.h, other, many, cc.cc_default_opts(use_graph=1))
+            assert cc.cc_run_mode(c.h, run) == mode
+            cc.cc_release(c.h, run)
+        _, used, size = cc.cc_context_stats(c.h)
+        # (kept tables fit 19 MB without those routes and 23 MB with them)
+        cc.cc_color(c.h, 1, (size - used - (41 << 19)) // n, 8)
+        assert kinds(c, cc.cc_load_pattern(c.h, *p), cid, 1, want, {}, retain=1) == ref
+
+
+def test_kept_tables_do_not_slow_runs_that_keep_none():
+    """Kept tables fit only without the routes that hold memory beside them; runs of the same key that
+    keep none do not go without."""
+    p, n = synth.path_pattern(8), 3000
+    g = synth.erdos_renyi(n, 6 / n, 3)
+    z = oracle.colors(n, 1, 8, seed=5)
+    want = oracle.run_dp(g, p, z, 8)
+    with cc.Context(arena_bytes=256 << 20) as c:
+        cc.cc_load_graph(c.h, *g)
+        cid = cc.cc_set_colors(c.h, z, 8)
+        _, used, size = cc.cc_context_stats(c.h)
+        cc.cc_color(c.h, 1, (size - used - (41 << 19)) // n, 8)
+        alone, both = cc.cc_load_pattern(c.h, *p), cc.cc_load_pattern(c.h, *p)
+        for _ in range(2):
+            ref = kinds(c, alone, cid, 1, want, {})
+        assert ref[0] == "planned"
+        kept = kinds(c, both, cid, 1, want, {}, retain=1)
+        assert kept[0] == "exact" and kept[1] != kinds(c, alone, cid, 1, want, {})[1]
+        assert kinds(c, both, cid, 1, want, {}) == ref
 
 
 # the six-cycle: one introduce that is expected to yield just more than two entries a pair and yields
