@@ -215,6 +215,7 @@ Outcome issue(Server *S, Ctx *c, ServeSlot &sl, const ServeQuery &q, bool alone)
     if (!q.exact && !split && q.limit == 0 && known) {
       exact = false;
       rc = rt::reset_run(c, sl.run.get(), (int)P.nodes.size());
+      sl.run->frugal = sl.sub.free_bytes() <= pl->second.frugal[0];
       if (!rc) rc = rt::run_nodes(c, sl.run.get(), P, sl.view, &pl->second);
       if (!rc && cudaEventRecord(sl.done, sl.stream) != cudaSuccess) rc = CC_ECUDA;
       if (rc == CC_ENOMEM)  // the planned capacities need more than this range

@@ -287,3 +287,37 @@ def test_run_that_does_not_fit_is_tried_once(pat, retain):
         mb /= 1.2
     assert full and spent
     assert np.mean([s > full for s in spent]) < 0.25, (full, spent)
+
+
+@pytest.mark.parametrize("limit", [0, 50])
+def test_served_in_little_room(limit):
+    """Queries of one key under budgets from one that holds its tables twice down to one that does not
+    hold them: the oracle's counts (whole, or in slices), or CC_ENOMEM for kept tables."""
+    p, n = synth.path_pattern(8), 3000
+    g = synth.erdos_renyi(n, 6 / n, 3)
+    want = [oracle.run_dp(g, p, oracle.colors(n, 1, 8, seed=s), 8) for s in range(3)]
+    first = want[0].enumerate(limit)[0][:limit] if limit else None
+    whole = 0
+    with cc.Context(arena_bytes=256 << 20) as c:
+        cc.cc_load_graph(c.h, *g)
+        budget = 48 << 20
+        while budget > 12 << 20:
+            pid = cc.cc_load_pattern(c.h, *p)  # a key of its own
+            cc.cc_serve_start(c.h, budget, 2)
+            try:
+                for s in (0, 1, 2, 0):
+                    ticket = cc.cc_serve_submit(c.h, pid, s, 1, 8, limit)
+                    done = False
+                    while not done:
+                        done, status, counts, _, _, rows = cc.cc_serve_poll(c.h, ticket, 1, limit, 8)
+                    if status:
+                        assert limit and status == cc.CC_ENOMEM, budget
+                        continue
+                    assert np.array_equal(counts, want[s].count), budget
+                    if limit and s == 0:
+                        assert np.array_equal(rows, first), budget
+                whole += cc.cc_serve_stats(c.h)["sliced"] == 0 and not status
+            finally:
+                cc.cc_serve_stop(c.h)
+            budget = int(budget / 1.08)
+    assert whole
