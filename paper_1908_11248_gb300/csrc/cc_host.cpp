@@ -774,9 +774,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     r.degF = a.degF;
     r.ubit = a.ubit;
     uint8_t *colT = nullptr;
-    if (colours_by_vertex(&colT) != CC_OK) {
-      short_of = true;
-      return CC_OK;
+    int rc = colours_by_vertex(&colT);
+    if (rc) {
+      short_of = rc == CC_ENOMEM;
+      return short_of ? CC_OK : rc;
     }
     r.colT = colT;
     // capacities: planned, or known as the exact run goes
@@ -801,7 +802,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (leaf) {
       if (cc::launch_set_word(c->stream, w_runs, (u64)n)) return CC_ECUDA;
     }
-    int rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, leaf ? 5 : 7, [&] {
+    rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, leaf ? 5 : 7, [&] {
       const int e = cc::launch_runs_list(c->stream, c->dev, R->kw, r, blk);
       return e ? e
                : cc::launch_scan_u32(c->stream, c->dev, r.deg, r.run_cap, off, scan, r.n_runs,
@@ -883,8 +884,12 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     r.n_more = w_more;
     rc = timed(x, planned ? CC_K_INTRO_WRITE : CC_K_INTRO_COUNT, 7, [&] {
       int e = cc::launch_runs_windows(c->stream, c->dev, r);
-      if (!e) e = cc::launch_scan_u32(c->stream, c->dev, r.win_one, windows, off_one, scan, nullptr, n_one);
-      if (!e) e = cc::launch_scan_u32(c->stream, c->dev, r.win_more, windows, off_more, scan, nullptr, w_more);
+      if (!e)
+        e = cc::launch_scan_u32(c->stream, c->dev, r.win_one, windows, off_one, scan, nullptr,
+                                n_one);
+      if (!e)
+        e = cc::launch_scan_u32(c->stream, c->dev, r.win_more, windows, off_more, scan, nullptr,
+                                w_more);
       return e;
     });
     if (rc) return rc;
@@ -924,7 +929,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
           held.p.push_back(srt);
           rc = timed(f, CC_K_REDUCE, 3, [&] {
             return cc::launch_reduce(c->stream, c->dev, R->kw, srt, w_more, r.side_cap, blk,
-                                     r.drop ? out : r.side, words + 2, &fsp, cc::sort_narrows(R->kw, fsp, 1));
+                                     r.drop ? out : r.side, words + 2, &fsp,
+                                     cc::sort_narrows(R->kw, fsp, 1));
           });
         }
       }
@@ -1220,10 +1226,14 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       a.ct = (u64)n;
       a.cv = 1;
       uint8_t *colT = nullptr;
-      if (planned && (grouped || x1 >= 0) && R->trials > 1 && colours_by_vertex(&colT) == CC_OK) {
-        a.cols = colT;
-        a.ct = 1;
-        a.cv = (u64)R->trials;
+      if (planned && (grouped || x1 >= 0) && R->trials > 1) {
+        rc = colours_by_vertex(&colT);
+        if (rc && rc != CC_ENOMEM) return rc;
+        if (!rc) {
+          a.cols = colT;
+          a.ct = 1;
+          a.cv = (u64)R->trials;
+        }
       }
       struct SortedGuard {
         Arena &a;
