@@ -544,7 +544,8 @@ __global__ void __launch_bounds__(256, 4) intro_warp_kernel(IntroArgs a) {
       if (lane >= o) incl += y;
     }
     I total = __shfl_sync(0xffffffffu, incl, 31);
-    if (a.heavy_cap && total > (I)(kHeavyWindow * a.win)) {  // the window's long lists go to the other kernel
+    // the window's long lists go to the other kernel
+    if (a.heavy_cap && total > (I)(kHeavyWindow * a.win)) {
       const int parts = nc > (I)kHeavyList ? (int)((nc + kHeavyPart - 1) / kHeavyPart) : 0;
       int upto = parts;
       for (int o = 1; o < 32; o <<= 1) {
@@ -702,17 +703,18 @@ __global__ void __launch_bounds__(256, 4) intro_heavy_kernel(IntroArgs a) {
 // What bounds it is the chain of dependent loads of a candidate (row pointers, neighbour, colour,
 // degree, a binary search).  One lead after the other left a third of the lanes with a candidate
 // and every chain of a window in sequence; end to end, a step's 32 chains belong to several
-// leads.  The closing introduce of a 4-cycle (one colouring of a
-// Barabasi-Albert graph, n = 200 000, m = 5; 27 million entries, 249 million candidates): 15.3 to
-// 10.8 ms (and 5.1 with the windows spread, IntroArgs::stretch); the three of the 2x4 grid with 13 colourings (n = 4999, m = 4): 1.47 to 1.00 ms.
+// leads.  The closing introduce of a 4-cycle (one colouring of a Barabasi-Albert graph, n = 200 000,
+// m = 5; 27 million entries, 249 million candidates): 15.3 to 10.8 ms (and 5.1 with the windows
+// spread, IntroArgs::stretch); the three of the 2x4 grid with 13 colourings (n = 4999, m = 4): 1.47
+// to 1.00 ms.
 constexpr int kGroupCap = 256;  // candidate-list buffer per warp (two of them)
-// IntroArgs::stretch, the consecutive windows a warp takes before it goes on elsewhere (1, 2, 4, 8): long
-// enough to carry lists, short enough that a stretch of costly runs (a hub's; the region of mappings that several runs led to,
-// cc_runs.cu) is spread over the warps.  One range a warp instead: 28.6 ms for the chained
-// introduce of the 3x3 grid (Erdos-Renyi, n = 100 000, 32 colourings), 12.7 in stretches;
-// the 4-cycle's closing introduce (Barabasi-Albert, n = 200 000) 10.8 against 5.1.  A table that
-// gives a warp few windows has shorter stretches, and with one colouring, whose runs are short,
-// smaller windows too: the closing introduce of the 4-cycle over 2.1 million entries
+// IntroArgs::stretch, the consecutive windows a warp takes before it goes on elsewhere (1, 2, 4, 8):
+// long enough to carry lists, short enough that a stretch of costly runs (a hub's; the region of
+// mappings that several runs led to, cc_runs.cu) is spread over the warps.  One range a warp instead:
+// 28.6 ms for the chained introduce of the 3x3 grid (Erdos-Renyi, n = 100 000, 32 colourings), 12.7
+// in stretches; the 4-cycle's closing introduce (Barabasi-Albert, n = 200 000) 10.8 against 5.1.  A
+// table that gives a warp few windows has shorter stretches, and with one colouring, whose runs are
+// short, smaller windows too: the closing introduce of the 4-cycle over 2.1 million entries
 // (Barabasi-Albert, n = 20 000) went from 0.52 to 0.15 ms.
 
 // true if v is in the increasing list col[lo, hi)
@@ -932,7 +934,13 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
       }
       const int excl = incl - d1, total = __shfl_sync(0xffffffffu, incl, 31);
       overflow = __any_sync(0xffffffffu, d1 > (1 << 25));  // (sums of 32 lists stay below 2^31)
-      if (lane == 0) examined += (u64)total;
+      if (overflow) {
+        u64 all = (u64)d1;
+        for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+        if (lane == 0) examined += all;
+      } else if (lane == 0) {
+        examined += (u64)total;
+      }
       for (int j0 = 0; j0 < total && !overflow; j0 += 32) {
         const int j = j0 + lane;
         int lo = 0, hi = 31;  // owner: smallest lane with incl > j
