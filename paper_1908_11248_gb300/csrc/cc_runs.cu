@@ -32,9 +32,10 @@
 // origins (a forget that leaves one vertex) most entries would be sorted in the side buffer after
 // all: the entry kernels take those nodes, and those of fewer than kRunTrials trials below a forget
 // or above a leaf.  An exact run, which knows neither, goes by what the runs' lengths and random
-// colours let it expect, before any pair is listed; what it has counted it also writes.  The 9-vertex tree (Barabasi-Albert, n = 20 000, 4 colourings), whose stored
-// introduces yield 15 to 100 entries a pair: 8.5 to 7.8 ms a run; a batch of partial k-trees with
-// 4 colourings is the same with the line at 4 trials as at 8 (9.07 and 8.99 ms).
+// colours let it expect, before any pair is listed; what it has counted it also writes.  The
+// 9-vertex tree (Barabasi-Albert, n = 20 000, 4 colourings), whose stored introduces yield 15 to
+// 100 entries a pair: 8.5 to 7.8 ms a run; a batch of partial k-trees with 4 colourings is the same
+// with the line at 4 trials as at 8 (9.07 and 8.99 ms).
 #include <algorithm>
 #include <cstdint>
 
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(256, 5) runs_write_kernel(RunsArgs a) {
     }
     const int excl = incl - len, total = __shfl_sync(0xffffffffu, incl, 31);
     u64 at = a.off_one[w], at2 = a.off_more[w];
-    // one step: the lane's entry, if any, of a pair (its run's entries from oe on, or leaf vertex oe)
+    // one step: the lane's entry, if any, of a pair (its run's entries from oe on; leaf vertex oe)
     auto step = [&](bool have, u64 oe, int x, u64 ophi, int ov, bool mine) {
       uint32_t t = 0, m = 0;
       bool ok = false;

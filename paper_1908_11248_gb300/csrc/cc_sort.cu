@@ -898,7 +898,8 @@ __global__ void __launch_bounds__(BLOCK) reduce_write_kernel(const void *src, co
       }
     }
     __syncthreads();
-    for (int l = tid + (open ? 0 : 1); l < total; l += BLOCK) put(cursor - 1 + l, s_key[l], s_cnt[l]);
+    for (int l = tid + (open ? 0 : 1); l < total; l += BLOCK)
+      put(cursor - 1 + l, s_key[l], s_cnt[l]);
     if (total || open) {
       open = true;
       osum = s_osum;
