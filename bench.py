@@ -206,11 +206,17 @@ GROUPS = {"color": "colour", "leaf": "leaf", "intro_count": "introduce",
 
 
 # device kernels (by function name) grouped by the node rule they implement, for the DRAM-traffic
-# summary of an ncu capture; kernels of no node rule (graph set-up, enumeration) are "other"
+# summary of an ncu capture; kernels of no node rule (graph set-up, enumeration, scans that several
+# rules share) are "other"
 KERNEL_GROUPS = {
     "color_kernel": "colour", "leaf_kernel": "leaf",
     "intro_kernel": "introduce", "intro_warp_kernel": "introduce",
     "intro_group_warp_kernel": "introduce", "nb_colour_hist_kernel": "introduce",
+    "intro_heavy_kernel": "introduce", "runs_colours_kernel": "introduce",
+    "runs_count_kernel": "introduce", "runs_scan_kernel": "introduce",
+    "runs_list_kernel": "introduce", "runs_degree_kernel": "introduce",
+    "runs_pairs_kernel": "introduce", "runs_windows_kernel": "introduce",
+    "runs_write_kernel": "introduce", "runs_append_kernel": "forget",
     "sort_hist_kernel": "forget", "row_scan_kernel": "forget", "digit_base_kernel": "forget",
     "sort_scatter_kernel": "forget", "sweep_hist_kernel": "forget",
     "sweep_bases_kernel": "forget", "sweep_pass_kernel": "forget",
@@ -220,7 +226,9 @@ KERNEL_GROUPS = {
     "part_cursor_kernel": "forget", "part_split_kernel": "forget",
     "part_local_kernel": "forget",
     "join_build_kernel": "join", "join_probe_kernel": "join",
-    "join_group_kernel": "join", "root_kernel": "root",
+    "join_heads_count_kernel": "join", "join_heads_scan_kernel": "join",
+    "join_heads_list_kernel": "join", "join_match_kernel": "join", "join_group_kernel": "join",
+    "root_kernel": "root",
 }
 
 

@@ -135,3 +135,23 @@ def test_forest_hom_counts_against_brute_force():
                 assert got[shape] <= brute and got[shape] >= 0.5 * brute, (t, shape)
             else:
                 assert got[shape] == brute, (t, shape, got[shape], brute)
+
+
+def test_every_kernel_has_a_group():
+    """Every device kernel is counted under the node rule it serves, or is one of those that serve
+    none or several (graph set-up, dumps, enumeration, shared scans)."""
+    import pathlib
+    import re
+
+    import paper_1908_11248_gb300 as cc
+
+    none = {"deg8_kernel", "set_word_kernel", "slice_mask_kernel", "unpack_kernel",
+            "wait_probe_kernel", "scan_blocks_kernel", "block_sums_kernel", "scan_small_kernel",
+            "block_scan_kernel", "enum_init_kernel", "enum_step_kernel"}
+    found = set()
+    for f in sorted((pathlib.Path(cc.__file__).parent / "csrc").glob("*.cu")):
+        for part in f.read_text().split("__global__")[1:]:
+            found.add(re.search(r"(\w+_kernel)\(", part).group(1))
+    rows = {k for k in found if k.startswith("rows_")}
+    assert set(bench.KERNEL_GROUPS) <= found
+    assert found - set(bench.KERNEL_GROUPS) == none | rows
