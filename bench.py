@@ -197,6 +197,20 @@ def algorithmic_bytes(kind, node, nodes, sizes, cand, n, T, k):
     return 0
 
 
+def step_bytes(node, kind, cand, nodes, sizes, n, T, k):
+    """algorithmic_bytes of every launch of one step.  A node rule that runs as several timed launches
+    (an introduce run by run, a forget that sorts pairs and then the entries that share a mapping, a
+    join that matches, counts and writes) moves its bytes once: the first launch of a kind at a node
+    has them, and of a join's the one that writes."""
+    out, seen = [], set()
+    for x, kn, c in zip(node, kind, cand):
+        first = (int(x), kn) not in seen
+        seen.add((int(x), kn))
+        out.append(algorithmic_bytes(kn, int(x), nodes, sizes, c, n, T, k)
+                   if first and kn not in ("join_build", "join_count") else 0)
+    return out
+
+
 # kernel kinds grouped by the node rule they implement (Section 3.1)
 GROUPS = {"color": "colour", "leaf": "leaf", "intro_count": "introduce",
           "intro_write": "introduce", "intro_chain": "introduce",
@@ -604,11 +618,11 @@ def dp_leg(cc, torch, name, args, rank, dist, tune=True, enum_limit=0, sampler=N
         sizes, total = cc.cc_table_stats(h, run, len(nodes))
         node, kind, ms, cand = cc.cc_run_timings(h, run)
         groups = {}
-        for i in range(len(node)):
-            kn = cc.KERNEL_KINDS[int(kind[i])]
+        kinds = [cc.KERNEL_KINDS[int(x)] for x in kind]
+        for kn, moved in zip(kinds, step_bytes(node, kinds, cand, nodes, sizes, n, T, k)):
             g2 = groups.setdefault(GROUPS.get(kn, kn), {"launches": 0, "bytes": 0})
             g2["launches"] += 1
-            g2["bytes"] += algorithmic_bytes(kn, int(node[i]), nodes, sizes, cand[i], n, T, k)
+            g2["bytes"] += moved
         with open(capture, "w") as f:
             json.dump({"workload": name, "trials": T, "sources": source_hash(),
                        "opts": out["config"]["opts"], "entries": int(total),
@@ -635,12 +649,12 @@ def dp_leg(cc, torch, name, args, rank, dist, tune=True, enum_limit=0, sampler=N
         entries += total
         modes.add(cc.cc_run_mode(h, run))
         node, kind, ms, cand = cc.cc_run_timings(h, run)
-        for i in range(len(node)):
-            kn = cc.KERNEL_KINDS[int(kind[i])]
-            d = kern.setdefault(kn, {"launches": 0, "ms": 0.0, "bytes": 0})
+        kinds = [cc.KERNEL_KINDS[int(x)] for x in kind]
+        for i, moved in enumerate(step_bytes(node, kinds, cand, nodes, sizes, n, T, k)):
+            d = kern.setdefault(kinds[i], {"launches": 0, "ms": 0.0, "bytes": 0})
             d["launches"] += 1
             d["ms"] += float(ms[i])
-            d["bytes"] += algorithmic_bytes(kn, int(node[i]), nodes, sizes, cand[i], n, T, k)
+            d["bytes"] += moved
         cc.cc_release(h, run)
         cc.cc_release_colors(h, cid)
     torch.cuda.synchronize()

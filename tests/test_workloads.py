@@ -155,3 +155,19 @@ def test_every_kernel_has_a_group():
     rows = {k for k in found if k.startswith("rows_")}
     assert set(bench.KERNEL_GROUPS) <= found
     assert found - set(bench.KERNEL_GROUPS) == none | rows
+
+
+def test_step_bytes_counts_a_rule_once():
+    """An introduce run by run (four launches), its forget (pairs and side entries sorted and
+    reduced) and a join group by group move their tables once."""
+    # leaf 0, introduce 1, forget 1, and a join of that table with itself
+    nodes = [(0, -1, -1, 0, [0]), (1, 0, -1, 1, [0, 1]), (2, 1, -1, 0, [1]), (3, 2, 2, -1, [1])]
+    sizes, k = [10, 1000, 70, 30], 3
+    s1, s2 = bench.slot_bytes(1, k), bench.slot_bytes(2, k)
+    kinds = ["intro_write"] * 2 + ["sort"] + ["intro_write"] * 2 + ["sort", "reduce", "reduce",
+                                                                     "join_build", "join_count",
+                                                                     "join_write"]
+    node = [1, 1, 2, 1, 1, 2, 2, 2, 3, 3, 3]
+    got = bench.step_bytes(node, kinds, [40] * len(node), nodes, sizes, 100, 1, k)
+    assert got == [10 * s1 + 40 * 5 + 1000 * s2, 0, 1000 * s2, 0, 0, 0, 70 * s1, 0,
+                   0, 0, (70 + 70 + 30) * s1]
