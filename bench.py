@@ -962,7 +962,7 @@ def hash_leg(cc, torch):
     """The hashed node rules, event-timed: `ba20k_grid2x4` (64 trials) with every introduce
     adding its projected entries into its forget's open-addressing hash table (fuse 1: one
     compare-and-swap to claim a key, one atomic add of the count, per entry), and pattern A of
-    Fig. 1 (three joins: hash join on the shared bag map) on the same graph with 16 trials, k =
+    Fig. 1 (three joins, these by groups of sorted children) on the same graph with 16 trials, k =
     n_F.  Reports each group's time and entries per second: for the hashed forget, entries
     inserted (= atomic updates) per second."""
     w = synth.WORKLOADS["ba20k_grid2x4"]
@@ -1003,8 +1003,9 @@ def hash_leg(cc, torch):
                           "entries_per_step": int(sizes.sum())}
     out["note"] = ("event-timed planned runs; intro_fused = introduce whose entries are inserted "
                    "into the forget's hash table (entries_per_s = hash inserts per second, one "
-                   "claim and one atomic count update each); join_* = hash join build and "
-                   "probe/write (entries_per_s = join output entries per second)")
+                   "claim and one atomic count update each); join_* = the three joins, group by "
+                   "group from 2^21 entries on, else through hash tables (entries_per_s = join "
+                   "output entries per second)")
     return out
 
 
@@ -1078,6 +1079,32 @@ def er_phase_leg(cc, torch, step=None, arena_gb=8):
         "note": "per point: load the pattern (minimum-width decomposition), colour ten times, one "
                 "DP over the ten colourings, decide; ms = host wall time of those calls",
     }
+
+
+# per leg: the arrays that go into the details file instead of the bench line
+DETAILS = {"er_phase": ("probs", "ms", "found_grid", "status_grid"),
+           "pl1m_ktree3_bound": ("per_pattern",)}
+
+
+def six_digits(x):
+    """x with every float in it at six significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: six_digits(v) for k, v in x.items()}
+    return [six_digits(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def brief(line):
+    """The bench line without its legs' arrays (one value per point of a study or pattern of a batch:
+    tens of kilobytes, more than a log's tail holds of one line), and those arrays.  The study's
+    times are summed over each row; extra keys keep six digits."""
+    legs = {k: dict(v) for k, v in line.items() if k in DETAILS and isinstance(v, dict)}
+    details = {k: {f: v.pop(f) for f in DETAILS[k] if f in v} for k, v in legs.items()}
+    if "ms" in details.get("er_phase", {}):
+        legs["er_phase"]["row_seconds"] = [sum(r) / 1e3 for r in details["er_phase"]["ms"]]
+    extra = [k for k, v in line.items() if isinstance(v, dict) and k not in ("e2e", "clocks")]
+    return {k: six_digits(legs.get(k, v)) if k in extra else v for k, v in line.items()}, details
 
 
 def serve_leg(cc, torch, count, arena_gb, budget_gb, slots, window_s):
@@ -1217,6 +1244,9 @@ def main():
     ap.add_argument("--legs", default="ba20k,latency,batching,hash,serve,er_phase,pl_bound",
                     help="extra keys to measure (comma list of ba20k, latency, batching, hash, "
                          "serve, er_phase, pl_bound; 'none' for none)")
+    ap.add_argument("--details", default="", metavar="JSON",
+                    help="also write the legs' arrays (per point of the Erdos-Renyi study, per "
+                         "pattern of the power-law batch) to this file")
     ap.add_argument("--er-phase-step", type=float, default=0.0,
                     help="grid step of the Erdos-Renyi study (default: the paper's 0.03)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
@@ -1350,6 +1380,10 @@ def main():
                                         args.serve_window)
     log("done")
     if rank == 0:
+        line, details = brief(line)
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(details, f)
         print(json.dumps(line), flush=True)
     if dist:
         dist.barrier()

@@ -171,3 +171,23 @@ def test_step_bytes_counts_a_rule_once():
     got = bench.step_bytes(node, kinds, [40] * len(node), nodes, sizes, 100, 1, k)
     assert got == [10 * s1 + 40 * 5 + 1000 * s2, 0, 1000 * s2, 0, 0, 0, 70 * s1, 0,
                    0, 0, (70 + 70 + 30) * s1]
+
+
+def test_bench_line_is_short():
+    """The study's points and the batch's patterns leave the bench line, whose numbers stay."""
+    import json
+
+    P = 34
+    line = {"metric": bench.METRIC, "value": 1 / 3, "e2e": {"value": 2 / 3}, "clocks": {"sm_mhz": 1},
+            "er_phase": {"probs": [0.03 * i for i in range(P)], "ms": [[1000 / 3] * P] * P,
+                         "found_grid": [[1] * P] * P, "status_grid": [[-2] * P] * P,
+                         "width_vs_q": [i / 7 for i in range(P)], "completed": 576},
+            "pl1m_ktree3_bound": {"patterns": 64, "per_pattern": [{"bytes": 2 / 3}] * 64}}
+    out, details = bench.brief(line)
+    assert len(json.dumps(out)) < 1500
+    assert out["value"] == 1 / 3 and out["e2e"] == {"value": 2 / 3}
+    assert out["er_phase"]["completed"] == 576 and out["pl1m_ktree3_bound"] == {"patterns": 64}
+    assert out["er_phase"]["row_seconds"] == [11.3333] * P
+    assert details["er_phase"]["ms"] == line["er_phase"]["ms"]
+    assert len(details["pl1m_ktree3_bound"]["per_pattern"]) == 64
+    assert "ms" in line["er_phase"]  # the caller's line is left alone
