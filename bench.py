@@ -199,15 +199,27 @@ def algorithmic_bytes(kind, node, nodes, sizes, cand, n, T, k):
 
 def step_bytes(node, kind, cand, nodes, sizes, n, T, k):
     """algorithmic_bytes of every launch of one step.  A node rule that runs as several timed launches
-    (an introduce run by run, a forget that sorts pairs and then the entries that share a mapping, a
-    join that matches, counts and writes) moves its bytes once: the first launch of a kind at a node
-    has them, and of a join's the one that writes."""
-    out, seen = [], set()
-    for x, kn, c in zip(node, kind, cand):
-        first = (int(x), kn) not in seen
-        seen.add((int(x), kn))
-        out.append(algorithmic_bytes(kn, int(x), nodes, sizes, c, n, T, k)
-                   if first and kn not in ("join_build", "join_count") else 0)
+    moves its bytes once: the first launch of a kind at a node has them, and of a join's the one that
+    writes.  An introduce run by run (several intro_write launches) below a forget writes the
+    forget's table: it has those bytes, and the sorts and reduces of the forget's pairs none."""
+    first, writes = {}, {}
+    for i, (x, kn) in enumerate(zip(node, kind)):
+        first.setdefault((int(x), kn), i)
+        writes[int(x)] = writes.get(int(x), 0) + (kn == "intro_write")
+    by_runs = {f: nodes[f][1] for f, nd in enumerate(nodes)
+               if nd[0] == 2 and writes.get(nd[1], 0) > 1}
+    out = []
+    for i, (x, kn, c) in enumerate(zip(node, kind, cand)):
+        x = int(x)
+        if first[x, kn] != i or kn in ("join_build", "join_count") or x in by_runs:
+            out.append(0)
+            continue
+        moved = algorithmic_bytes(kn, x, nodes, sizes, c, n, T, k)
+        for f, below in by_runs.items():
+            if below == x and kn == "intro_write":
+                moved += int(sizes[f]) * slot_bytes(len(nodes[f][4]), k)
+                moved -= int(sizes[x]) * slot_bytes(len(nodes[x][4]), k)
+        out.append(moved)
     return out
 
 

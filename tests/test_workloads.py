@@ -169,8 +169,12 @@ def test_step_bytes_counts_a_rule_once():
                                                                      "join_write"]
     node = [1, 1, 2, 1, 1, 2, 2, 2, 3, 3, 3]
     got = bench.step_bytes(node, kinds, [40] * len(node), nodes, sizes, 100, 1, k)
-    assert got == [10 * s1 + 40 * 5 + 1000 * s2, 0, 1000 * s2, 0, 0, 0, 70 * s1, 0,
-                   0, 0, (70 + 70 + 30) * s1]
+    # the introduce reads its child and writes the forget's table
+    assert got == [10 * s1 + 40 * 5 + 70 * s1] + [0] * 9 + [(70 + 70 + 30) * s1]
+    # entry by entry: the introduce writes its own, which the forget reads
+    got = bench.step_bytes([1, 2, 2], ["intro_write", "sort", "reduce"], [40] * 3, nodes, sizes,
+                           100, 1, k)
+    assert got == [10 * s1 + 40 * 5 + 1000 * s2, 1000 * s2, 70 * s1]
 
 
 def test_bench_line_is_short():
