@@ -1093,9 +1093,22 @@ def er_phase_leg(cc, torch, step=None, arena_gb=8):
     }
 
 
-# per leg: the arrays that go into the details file instead of the bench line
-DETAILS = {"er_phase": ("probs", "ms", "found_grid", "status_grid"),
-           "pl1m_ktree3_bound": ("per_pattern",)}
+# what the bench line keeps of each extra leg (a dotted name reaches into a dict)
+HEADLINE = {
+    "ba20k_grid2x4": ("value", "ms_per_step", "entries_per_step", "gpu_launches", "run_modes",
+                      "roofline.kernel", "roofline.frac"),
+    "er200_c5_latency": ("p50_ms", "p99_ms", "count"),
+    "batched_vs_plain": ("plain.entries_per_s", "batched.entries_per_s",
+                         "graph_batched.entries_per_s", "graph_replay.idle_fraction",
+                         "identical"),
+    "hashed_rules": ("forget_hashed.kinds.intro_fused.entries_per_s",
+                     "join.kinds.join_write.entries_per_s"),
+    "pl1m_ktree3_bound": ("patterns", "with_forest_bound", "proven_too_large"),
+    "er_phase": ("points", "seconds", "completed", "enomem", "width_limit", "found", "entries"),
+    "serving": ("keys", "light_keys", "classify_s", "served.completed", "served.qps",
+                "served.p50_ms", "served.p99_ms", "plain.completed", "plain.qps", "plain.p50_ms",
+                "plain.p99_ms", "identical"),
+}
 
 
 def six_digits(x):
@@ -1108,15 +1121,25 @@ def six_digits(x):
 
 
 def brief(line):
-    """The bench line without its legs' arrays (one value per point of a study or pattern of a batch:
-    tens of kilobytes, more than a log's tail holds of one line), and those arrays.  The study's
-    times are summed over each row; extra keys keep six digits."""
-    legs = {k: dict(v) for k, v in line.items() if k in DETAILS and isinstance(v, dict)}
-    details = {k: {f: v.pop(f) for f in DETAILS[k] if f in v} for k, v in legs.items()}
-    if "ms" in details.get("er_phase", {}):
-        legs["er_phase"]["row_seconds"] = [sum(r) / 1e3 for r in details["er_phase"]["ms"]]
-    extra = [k for k, v in line.items() if isinstance(v, dict) and k not in ("e2e", "clocks")]
-    return {k: six_digits(legs.get(k, v)) if k in extra else v for k, v in line.items()}, details
+    """The bench line as printed: the metric's own keys whole, of the roofline the groups without its
+    list of kernels, of the extra legs their headline figures at six digits.  (With every point of
+    the Erdos-Renyi study and every pattern of the power-law batch the line was tens of kilobytes,
+    more than a log's tail keeps.)"""
+    out = {}
+    for k, v in line.items():
+        if k == "roofline" and isinstance(v, dict):
+            v = six_digits({f: x for f, x in v.items() if f != "kernels"})
+        elif k in HEADLINE and isinstance(v, dict) and "error" not in v:
+            kept = {}
+            for name in HEADLINE[k]:
+                x = v
+                for part in name.split("."):
+                    x = x.get(part) if isinstance(x, dict) else None
+                if x is not None:
+                    kept[name] = six_digits(x)
+            v = kept
+        out[k] = v
+    return out
 
 
 def serve_leg(cc, torch, count, arena_gb, budget_gb, slots, window_s):
@@ -1257,8 +1280,8 @@ def main():
                     help="extra keys to measure (comma list of ba20k, latency, batching, hash, "
                          "serve, er_phase, pl_bound; 'none' for none)")
     ap.add_argument("--details", default="", metavar="JSON",
-                    help="also write the legs' arrays (per point of the Erdos-Renyi study, per "
-                         "pattern of the power-law batch) to this file")
+                    help="also write the line with every leg whole (per kernel kind, per point of "
+                         "the Erdos-Renyi study, per pattern of the power-law batch) to this file")
     ap.add_argument("--er-phase-step", type=float, default=0.0,
                     help="grid step of the Erdos-Renyi study (default: the paper's 0.03)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
@@ -1392,11 +1415,10 @@ def main():
                                         args.serve_window)
     log("done")
     if rank == 0:
-        line, details = brief(line)
         if args.details:
             with open(args.details, "w") as f:
-                json.dump(details, f)
-        print(json.dumps(line), flush=True)
+                json.dump(line, f)
+        print(json.dumps(brief(line)), flush=True)
     if dist:
         dist.barrier()
         dist.destroy_process_group()

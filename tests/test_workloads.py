@@ -178,20 +178,22 @@ def test_step_bytes_counts_a_rule_once():
 
 
 def test_bench_line_is_short():
-    """The study's points and the batch's patterns leave the bench line, whose numbers stay."""
+    """The line as printed keeps the metric's keys whole and the legs' headline figures."""
     import json
 
     P = 34
     line = {"metric": bench.METRIC, "value": 1 / 3, "e2e": {"value": 2 / 3}, "clocks": {"sm_mhz": 1},
-            "er_phase": {"probs": [0.03 * i for i in range(P)], "ms": [[1000 / 3] * P] * P,
-                         "found_grid": [[1] * P] * P, "status_grid": [[-2] * P] * P,
-                         "width_vs_q": [i / 7 for i in range(P)], "completed": 576},
+            "roofline": {"kernel": "introduce", "frac": 1 / 3, "kernels": {"sort": {"ms": 1.0}}},
+            "er_phase": {"ms": [[1000 / 3] * P] * P, "status_grid": [[-2] * P] * P,
+                         "completed": 576, "seconds": 2 / 3},
+            "hashed_rules": {"error": "x"},
+            "serving": {"served": {"qps": 2 / 3, "span_s": 1.0}, "identical": True},
             "pl1m_ktree3_bound": {"patterns": 64, "per_pattern": [{"bytes": 2 / 3}] * 64}}
-    out, details = bench.brief(line)
-    assert len(json.dumps(out)) < 1500
+    out = bench.brief(line)
+    assert len(json.dumps(out)) < 600
     assert out["value"] == 1 / 3 and out["e2e"] == {"value": 2 / 3}
-    assert out["er_phase"]["completed"] == 576 and out["pl1m_ktree3_bound"] == {"patterns": 64}
-    assert out["er_phase"]["row_seconds"] == [11.3333] * P
-    assert details["er_phase"]["ms"] == line["er_phase"]["ms"]
-    assert len(details["pl1m_ktree3_bound"]["per_pattern"]) == 64
-    assert "ms" in line["er_phase"]  # the caller's line is left alone
+    assert out["roofline"] == {"kernel": "introduce", "frac": 0.333333}
+    assert out["er_phase"] == {"completed": 576, "seconds": 0.666667}
+    assert out["hashed_rules"] == {"error": "x"}
+    assert out["serving"] == {"served.qps": 0.666667, "identical": True}
+    assert out["pl1m_ktree3_bound"] == {"patterns": 64}
