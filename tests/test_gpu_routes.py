@@ -112,9 +112,9 @@ def check_tables(ctx, g, pat, z, k, reps=2, **opt):
     cc.cc_release_colors(ctx.h, cid)
 
 
-# a bag of one vertex: k - 1 private colours.  One word of sums, the edge of a word, several
-# words, the most a warp keeps (11 private colours), one more (hash tables); few entries (hash
-# tables) and more than the 2^21 at which children are sorted and joined group by group
+# the join's bag is {0, 1}: k - 2 private colours.  One word of sums, several words, the most a warp
+# keeps (11 private colours, k = 13; one more is below, with the routes); few entries (hash tables)
+# and more than the 2^21 at which children are sorted and joined group by group
 @pytest.mark.parametrize("k", [4, 6, 7, 12, 13])
 @pytest.mark.parametrize("many", [0, 1])
 def test_join_routes(ctx, k, many):
@@ -308,3 +308,79 @@ def test_dropped_entries(ctx, name, n, hubs, trials, spare, opt):
         assert np.array_equal(cc.cc_table_stats(ctx.h, run, N)[0], ref.node_sizes.sum(axis=0)), rep
         cc.cc_release(ctx.h, run)
     cc.cc_release_colors(ctx.h, cid)
+
+
+def launched(ctx, g, pat, z, k, **opt):
+    """Per run (exact, planned): the (node, kernel kind) pairs it launched, with repeats, and the
+    number of its kernel launches.  Counts and sizes are checked."""
+    T = z.shape[0]
+    ref = oracle.run_dp(g, pat, z, k)
+    cc.cc_load_graph(ctx.h, *g)
+    pid = cc.cc_load_pattern(ctx.h, *pat)
+    N, _ = cc.cc_pattern_info(ctx.h, pid)
+    cid = cc.cc_set_colors(ctx.h, z, k)
+    out = []
+    for mode in ("exact", "planned"):
+        before = cc.cc_context_stats(ctx.h)[0]
+        run = cc.cc_run_dp(ctx.h, pid, cid, cc.cc_default_opts(profile=1, **opt))
+        launches = cc.cc_context_stats(ctx.h)[0] - before
+        assert cc.cc_run_mode(ctx.h, run) == mode
+        assert np.array_equal(cc.cc_count(ctx.h, run, T), ref.count)
+        assert np.array_equal(cc.cc_table_stats(ctx.h, run, N)[0], ref.node_sizes.sum(axis=0))
+        node, kind, _, _ = cc.cc_run_timings(ctx.h, run)
+        out.append(([(x, cc.KERNEL_KINDS[k2]) for x, k2 in zip(node.tolist(), kind.tolist())],
+                    launches))
+        cc.cc_release(ctx.h, run)
+    cc.cc_release_colors(ctx.h, cid)
+    return out, ref.node_sizes.sum(axis=0), cc.cc_pattern_nodes(ctx.h, pid, pat[0])
+
+
+@pytest.mark.parametrize("k,groups", [(13, True), (14, False)])
+def test_join_route_at_its_limit(ctx, k, groups):
+    """Eleven private colours are joined group by group, twelve through hash tables."""
+    n, trials = 8000, 6
+    made, sizes, nodes = launched(ctx, synth.erdos_renyi(n, 8 / n, 6), star_of_joins(4),
+                                  oracle.colors(n, trials, k, seed=k), k)
+    x, = [i for i, nd in enumerate(nodes) if nd[0] == cc.JOIN]
+    assert sizes[nodes[x][1]] + sizes[nodes[x][2]] >= 1 << 21 and len(nodes[x][4]) == 2
+    planned = made[1][0]  # only joins by groups count in planned runs
+    assert ((x, "join_count") in planned) == groups
+    assert (x, "join_write") in planned
+
+
+@pytest.mark.parametrize("over", [0, 1])
+def test_forget_route_at_its_limit(ctx, over):
+    """2^18 entries are added into the forget's hash table, two more are sorted: a properly coloured
+    ring, both ends of every edge."""
+    n = (1 << 17) + over
+    z = (np.arange(n) % 2).astype(np.uint8)[None]
+    if over:
+        z[0, -1] = 2
+    made, sizes, nodes = launched(ctx, synth.cycle_graph(n), synth.path_pattern(3), z, 3)
+    assert sizes[1] == 2 * n and nodes[2][0] == cc.FORGET
+    for kinds, _ in made:
+        assert ((1, "intro_fused") in kinds) == (not over)
+        assert ((2, "sort") in kinds) == bool(over)
+
+
+@pytest.mark.parametrize("trials", [7, 8])
+def test_run_wise_route_at_its_limit(ctx, trials):
+    """Eight colourings are taken run by run below a forget (four timed launches an introduce)."""
+    made, sizes, nodes = launched(ctx, hub_graph(1500, 3), synth.grid_pattern(2, 4),
+                                  oracle.colors(1500, trials, 8, seed=5), 8)
+    planned = made[1][0]
+    large = [x for x, nd in enumerate(nodes) if nd[0] == cc.INTRODUCE and sizes[x] > 1 << 20]
+    assert large and any((planned.count((x, "intro_write")) == 4) == (trials == 8) for x in large)
+    assert trials == 8 or all(planned.count((x, "intro_write")) <= 1 for x in large)
+
+
+def test_hub_route_at_its_limit(ctx):
+    """A largest degree of 65 takes each expanding introduce's second kernel, 64 does not."""
+    launches = []
+    for d in (64, 65):
+        g = synth.csr_from_edges(4 * (d + 1), np.array(
+            [(c * (d + 1), c * (d + 1) + 1 + i) for c in range(4) for i in range(d)]))
+        made, _, nodes = launched(ctx, g, synth.path_pattern(3),
+                                  oracle.colors(4 * (d + 1), 1, 3, seed=1), 3)
+        launches.append(made[1][1])
+    assert launches[1] - launches[0] == sum(nd[0] == cc.INTRODUCE for nd in nodes)
