@@ -197,3 +197,18 @@ def test_bench_line_is_short():
     assert out["hashed_rules"] == {"error": "x"}
     assert out["serving"] == {"served.qps": 0.666667, "identical": True}
     assert out["pl1m_ktree3_bound"] == {"patterns": 64}
+
+
+def test_kernel_table_tells_fused_introduces():
+    """In a run with both, only the introduces that add into a forget's hash table count with it."""
+    ns = "void cc::(anonymous namespace)::"
+    launches = [{"name": ns + n, "read": 1.0, "write": 0.0, "ms": 1.0} for n in (
+        "intro_warp_kernel<unsigned long long, (int)2>(IntroArgs)",
+        "intro_group_warp_kernel<unsigned long long, 2, 0>(IntroArgs)",
+        "intro_group_warp_kernel<unsigned __int128, 1, 1>(IntroArgs)",
+        "intro_heavy_kernel<unsigned long long, 1>(IntroArgs)",
+        "runs_write_kernel<unsigned long long>(RunsArgs)",
+        "sweep_pass_wide_kernel<unsigned long long, unsigned long long, 8, 1, 1>(SortSpec)")]
+    _, groups = bench.kernel_table(launches, True)
+    assert {g: v["launches"] for g, v in groups.items()} == {
+        "introduce+forget": 2, "introduce": 3, "forget": 1}
