@@ -373,11 +373,12 @@ __global__ void __launch_bounds__(BLOCK, 4) sweep_pass_kernel(SortSpec sp, const
 // (claim, barriers, look-back over 256 digit words, publication) are spread over twice the
 // records; the staging buffer lives in dynamic shared memory.
 //
-// What bounds it is latency inside the tile (two blocks an SM; 12 of 33 stall cycles an
-// instruction at barriers, 12 on shared memory, DRAM at 29 %), so a record's path is kept short:
-// peers of equal digit come from eight ballots, the leader's read of the warp's count gives the
-// rank at once (no shared-memory histogram beside it and no second walk over the items), and the
-// look-back reads four words of the tiles before at a time, while the upper warps stage.
+// What bounds it is latency inside the tile (two blocks an SM, half of its warps; 7 million
+// records: of 17 cycles between a warp's instructions 4 to 5 at barriers, 3 to 5 on loads, DRAM at
+// 22 to 29 %), so a record's path is kept short: peers of equal digit come from eight ballots, the
+// leader's read of the warp's count gives the rank at once (no shared-memory histogram beside it
+// and no second walk over the items), and the look-back reads four words of the tiles before at a
+// time, while the upper warps stage.
 // A sort of 27 million 16-byte records by a 40-bit full order (five passes and the histograms):
 // 2.05 to 1.69 ms; of 16 million by a 32-bit partial order 0.91 to 0.83.
 // KI: record type read; K: record type written (narrower when the records leave carrying a
