@@ -434,8 +434,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   R->pairs.assign(N, 0);
   R->runwise.assign(N, {});
   R->starved = false;
-  R->beside = 0;
   if (planned) R->learn_pairs = false;
+  R->beside = 0;
   R->checks.clear();
   std::vector<bool> made(N, false);
   const int grid = cc::intro_grid(c->dev, block);
@@ -1045,11 +1045,12 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     u64 *scan = (u64 *)hold(cc::scan_scratch_words(c->dev) * sizeof(u64));
     if (short_of) return CC_OK;
     a.off = off;
+    a.pairs = pairs_dev + x;
     r = timed(x, CC_K_JOIN_BUILD, 4,
               [&] { return cc::launch_join_match(c->stream, c->dev, R->kw, a, blk); });
     if (r) return r;
     r = timed(x, CC_K_JOIN_COUNT, 4, [&] {
-      const int e = cc::launch_join_groups(c->stream, c->dev, R->kw, 0, a);
+      const int e = cc::launch_join_groups(c->stream, c->dev, R->kw, R->learn_pairs ? 2 : 0, a);
       return e ? e : cc::launch_scan_u32(c->stream, c->dev, a.cnt, a.a.cap, off, scan, a.groups,
                                          R->d_counters + x);
     });
@@ -1059,8 +1060,9 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (r) return r;
     const u64 cap = std::max<u64>(1, total);
     void *p = A.alloc(cap * rb);
-    if (!p) {  // (the hash table's counter starts at 0)
+    if (!p) {  // (the hash table's counters start at 0)
       CUDA_OK(cudaMemsetAsync(R->d_counters + x, 0, sizeof(u64), c->stream));
+      CUDA_OK(cudaMemsetAsync(pairs_dev + x, 0, sizeof(u64), c->stream));
       return CC_OK;
     }
     R->tables[x] = {p, cap, 0, true};
@@ -1522,7 +1524,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       release_child(y);
     } else {  // join: group by group, or through hash tables
       int joined = 0;
-      if (!R->frugal && !R->learn_pairs && R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
+      if (!R->frugal && R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
           entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries) {
         rc = join_groups(x, &joined);
         if (rc) return rc;

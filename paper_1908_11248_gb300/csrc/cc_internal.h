@@ -246,6 +246,7 @@ struct JoinGroupArgs {
   unsigned long long *groups, *first, *blo;
   unsigned *blen, *cnt;
   const unsigned long long *off;
+  unsigned long long *pairs;  // mode 2: matching pairs, which a join through hash tables plans by
   TableDesc out;     // mode 1
   int *err;
 };
@@ -367,7 +368,7 @@ int prepare_join_kernels();  // once per device, as prepare_sort_kernels
 // lists a's groups and finds their ranges in b (blk: 2 * sort_grid(d) words)
 int launch_join_match(cudaStream_t s, const DevInfo &d, int kw, const JoinGroupArgs &a,
                       unsigned long long *blk);
-// mode 0 counts each group's results, mode 1 writes them
+// mode 0 counts each group's results, mode 1 writes them, mode 2 is 0 and counts matching pairs
 int launch_join_groups(cudaStream_t s, const DevInfo &d, int kw, int mode, const JoinGroupArgs &a);
 int launch_root(cudaStream_t s, const DevInfo &d, int kw, const RootArgs &a);
 int launch_unpack(cudaStream_t s, const DevInfo &d, int kw, const KeyLayout &L,

@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(256) join_match_kernel(JoinGroupArgs a) {
 }
 
 // MODE 0: the number of results of every group to cnt; MODE 1: the results themselves at the
-// offsets made from those counts.
+// offsets made from those counts; MODE 2: as 0, and the matching pairs (their count costs the
+// first pass a twentieth, so they are counted once, when a plan wants them).
 template <typename K, int MODE>
 __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupArgs a) {
   extern __shared__ u64 s_dyn[];
@@ -171,8 +172,9 @@ __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupAr
   const unsigned lt = (1u << lane) - 1u;
   const int k = a.L.k;
   const unsigned m = 1u << (k - a.bag), words = m > 32 ? m / 32 : 1;
-  u64 *acc = s_dyn + (size_t)w * m;  // MODE 1
-  unsigned *bits = reinterpret_cast<unsigned *>(s_dyn + (MODE ? (size_t)kJoinWarps * m : 0)) +
+  constexpr bool WRITE = MODE == 1;
+  u64 *acc = s_dyn + (size_t)w * m;  // WRITE
+  unsigned *bits = reinterpret_cast<unsigned *>(s_dyn + (WRITE ? (size_t)kJoinWarps * m : 0)) +
                    (size_t)w * words;
   const Slot<K> *ta = reinterpret_cast<const Slot<K> *>(a.a.slots);
   const Slot<K> *tb = reinterpret_cast<const Slot<K> *>(a.b.slots);
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupAr
   const u64 warps = (u64)gridDim.x * kJoinWarps;
   const uint32_t cmask = (uint32_t)((1ull << k) - 1ull);
   bool full = false;
+  unsigned hits = 0;  // MODE 2: pairs of this lane
   for (u64 base = ((u64)blockIdx.x * kJoinWarps + w) * 32; base < groups; base += warps * 32) {
     const u64 g = base + lane;
     u64 af = 0, ae = 0, bf = 0;
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupAr
       ae = g + 1 < groups ? a.first[g + 1] : na;
       bf = a.blo[g];
       bl = a.blen[g];
-      if (MODE == 0 && bl == 0) a.cnt[g] = 0;
+      if (!WRITE && bl == 0) a.cnt[g] = 0;
     }
     for (unsigned todo = __ballot_sync(0xffffffffu, bl != 0); todo; todo &= todo - 1) {
       const int l = __ffs(todo) - 1;
@@ -208,7 +211,7 @@ __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupAr
                                 (u64)key_slot(gkey, a.L, lane)];
       bagc = __reduce_or_sync(0xffffffffu, bagc);
       for (unsigned j = lane; j < words; j += 32) bits[j] = 0;
-      if (MODE)
+      if (WRITE)
         for (unsigned j = lane; j < m; j += 32) acc[j] = 0;
       __syncwarp();
       for (u64 x0 = a0; x0 < a1; x0 += 32) {
@@ -232,17 +235,18 @@ __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupAr
           const int ny = b1 - y0 < 32 ? (int)(b1 - y0) : 32;
           for (int j = 0; j < ny; ++j) {
             const uint32_t cj = __shfl_sync(0xffffffffu, cb, j);
-            const u64 dj = MODE ? __shfl_sync(0xffffffffu, c2, j) : 0;
+            const u64 dj = WRITE ? __shfl_sync(0xffffffffu, c2, j) : 0;
             if (ca != ~0u && (ca & cj) == 0) {
               const uint32_t s = ca | cj;
               atomicOr(&bits[s >> 5], 1u << (s & 31));
-              if (MODE) atomicAdd(&acc[s], c1 * dj);
+              if (WRITE) atomicAdd(&acc[s], c1 * dj);
+              if (MODE == 2) ++hits;
             }
           }
         }
       }
       __syncwarp();
-      if (MODE == 0) {
+      if (!WRITE) {
         unsigned n = 0;
         for (unsigned j = lane; j < words; j += 32) n += __popc(bits[j]);
         n = __reduce_add_sync(0xffffffffu, n);
@@ -266,12 +270,17 @@ __global__ void __launch_bounds__(32 * kJoinWarps) join_group_kernel(JoinGroupAr
       __syncwarp();  // the sums are cleared for the next group
     }
   }
+  if (MODE == 2) {
+    u64 all = hits;
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_down_sync(0xffffffffu, all, o);
+    if (lane == 0 && all) atomicAdd(a.pairs, all);
+  }
   if (full) atomicOr(a.err, kErrOverflow);
 }
 
 size_t join_smem(int mode, int private_colours) {
   const size_t m = size_t(1) << private_colours, words = m > 32 ? m / 32 : 1;
-  return kJoinWarps * ((mode ? m * sizeof(u64) : 0) + words * sizeof(unsigned));
+  return kJoinWarps * ((mode == 1 ? m * sizeof(u64) : 0) + words * sizeof(unsigned));
 }
 
 }  // namespace
@@ -311,10 +320,12 @@ int launch_join_groups(cudaStream_t s, const DevInfo &d, int kw, int mode,
 #define CC_JG(K, M) join_group_kernel<K, M><<<grid, 32 * kJoinWarps, smem, s>>>(a)
   if (kw == 1) {
     if (mode == 0) CC_JG(u64, 0);
-    else CC_JG(u64, 1);
+    else if (mode == 1) CC_JG(u64, 1);
+    else CC_JG(u64, 2);
   } else {
     if (mode == 0) CC_JG(u128, 0);
-    else CC_JG(u128, 1);
+    else if (mode == 1) CC_JG(u128, 1);
+    else CC_JG(u128, 2);
   }
 #undef CC_JG
   return (int)cudaGetLastError();

@@ -230,8 +230,9 @@ struct Run {
   size_t beside = 0;      // bytes of transposed colours
   size_t room = 0;        // free arena bytes when it started
   bool starved = false;   // an introduce run by run was left for want of memory (exact runs)
-  bool learn_pairs = false;  // a planned attempt had to join through hash tables without knowing how
-                             // many pairs match: joins that way, exactly
+  // a planned attempt lacked the matching pairs of a join that had to go through hash tables: the
+  // exact one counts them while it joins by groups
+  bool learn_pairs = false;
   int sliced = 0;         // most slices one of its trials was split into (0: none)
   u64 *d_blk = nullptr;  // per-run scratch: block counts and bases, pair counters
   int *d_err = nullptr;  // per-run device error word

@@ -259,6 +259,36 @@ def test_join_without_room_to_sort():
         assert hashed
 
 
+def test_what_fits_exactly_goes_on_fitting():
+    """In every room in which a key's first run fits, its later ones do, though the planned
+    capacities may not (kept tables of three joins: by groups they fit, as hash tables they would
+    not)."""
+    p, n, trials = synth.make_pattern(("A",)), 4000, 3
+    g = synth.barabasi_albert(n, 4, 3)
+    z = oracle.colors(n, trials, 9, seed=5)
+    want = oracle.run_dp(g, p, z, 9)
+    fitted = 0
+    with cc.Context(arena_bytes=1024 << 20) as c:
+        cc.cc_load_graph(c.h, *g)
+        cid = cc.cc_set_colors(c.h, z, 9)
+        size, left = cc.cc_context_stats(c.h)[2], 560 << 20
+        while left > 320 << 20:
+            left = int(left / 1.03)
+            held = cc.cc_color(c.h, 1, (size - cc.cc_context_stats(c.h)[1] - left) // n, 9)
+            pid = cc.cc_load_pattern(c.h, *p)
+            for rep in range(3):
+                try:
+                    run = cc.cc_run_dp(c.h, pid, cid, cc.cc_default_opts(retain=1))
+                except cc.CCError as ex:
+                    assert ex.code == cc.CC_ENOMEM and rep == 0, (left >> 10, rep)
+                    break
+                fitted += 1
+                assert np.array_equal(cc.cc_count(c.h, run, trials), want.count)
+                cc.cc_release(c.h, run)
+            cc.cc_release_colors(c.h, held)
+    assert fitted
+
+
 @pytest.mark.parametrize("retain", [0, 1])
 @pytest.mark.parametrize("pat", [("A",), ("cycle", 5)])
 def test_run_that_does_not_fit_is_tried_once(pat, retain):
