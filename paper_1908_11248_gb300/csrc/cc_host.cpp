@@ -1296,12 +1296,15 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         while (grouped && R->trials == 1 && a.win > 8 && warps * a.win * 16 > scan) a.win >>= 1;
         while (a.stretch > 1 && warps * a.win * 16 * a.stretch > scan) a.stretch >>= 1;
         // hubs: room for the parts of their lists (8 MB at most; what does not fit is walked in
-        // place), and for the second kernel's last chunks
+        // place), and for the second kernel's last chunks, which the node's three record buffers
+        // have to hold: where those would not fit with it, the lists stay where they are
         if (a.nnb == 1 && !R->frugal && a.G.row_ptr == c->d_row_ptr &&
             c->max_deg > cc::kHeavyList) {
           const u64 parts = (u64)(c->max_deg + cc::kHeavyPart - 1) / cc::kHeavyPart;
           const u64 places = std::min<u64>(1 << 20, room(plan->entries[y]) * parts);
-          heavy_mem = A.alloc((places + 1) * sizeof(u64));
+          const u64 records = 3 * (room(plan->entries[x]) + 2 * slack);
+          if (records * rb + places * sizeof(u64) < A.largest_free())
+            heavy_mem = A.alloc((places + 1) * sizeof(u64));
           if (heavy_mem) {
             a.heavy_cap = places;
             a.heavy_n = (u64 *)heavy_mem;
