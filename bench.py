@@ -253,7 +253,8 @@ KERNEL_GROUPS = {
     "part_local_kernel": "forget",
     "join_build_kernel": "join", "join_probe_kernel": "join",
     "join_heads_count_kernel": "join", "join_heads_scan_kernel": "join",
-    "join_heads_list_kernel": "join", "join_match_kernel": "join", "join_group_kernel": "join",
+    "join_heads_list_kernel": "join", "join_match_kernel": "join", "join_tested_kernel": "join",
+    "join_group_kernel": "join",
     "root_kernel": "root",
 }
 

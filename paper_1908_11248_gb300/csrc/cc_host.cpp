@@ -432,6 +432,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   R->tables.assign(N, {});
   R->sizes.assign(N, 0);
   R->pairs.assign(N, 0);
+  R->tested.assign(N, 0);
+  R->groups.assign(N, 0);
   R->runwise.assign(N, {});
   R->starved = false;
   if (planned) R->learn_pairs = false;
@@ -448,6 +450,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
   u64 *blk = R->d_blk;
   u64 *cursor = R->d_counters + N;      // per node: chunked-append cursor (scan bound)
   u64 *pairs_dev = R->d_counters + 2 * N;  // per join: matching colour-set pairs
+  u64 *tested_dev = R->d_counters + 3 * N;  // per join: those tested
+  u64 *groups_dev = R->d_counters + 7 * N;  // per join: groups of its smaller child
   CUDA_OK(cudaMemsetAsync(R->d_err, 0, sizeof(int), c->stream));
   const size_t rb = cc::slot_bytes(R->kw);
   // planned room for a quantity last seen at v (plus slack for chunked appends)
@@ -553,6 +557,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       if (z.child1 >= 0) todo.push_back(z.child1);
     }
     return below;
+  };
+  // how many vertices x's subtree has (an entry of x has a colour for each)
+  auto subtree_vertices = [&](int x) {
+    return P.nodes[x].bag.size() + __builtin_popcount(forgotten_below(x));
   };
   // true if a vertex forgotten below y has all its F-neighbours among those of u in y's bag
   // (IntroArgs::twin; with allowed mappings or the distance bound a candidate of u need not be
@@ -696,6 +704,34 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     *out = (uint8_t *)transposed.p[0];
     return CC_OK;
   };
+  // pairs of entries to test for a group from which join x is made group by group (kJoinTested: fewer
+  // if a join above takes the sorted result)
+  auto tests_for_groups = [&](int x) {
+    const int up = P.nodes[x].parent;
+    return up >= 0 && P.nodes[up].type == 3 ? cc::kJoinTestedBelowJoin : cc::kJoinTested;
+  };
+  // true if join x's groups are long enough to be joined one by one: by what the plan knows of them,
+  // else by the most colour sets that a group of either child can hold
+  auto long_groups = [&](int x) {
+    const NiceNode &nd = P.nodes[x];
+    const int b = (int)nd.bag.size(), priv = R->L.k - b;
+    if (priv > cc::kJoinBits) return false;
+    if (planned) {
+      const u64 tested = plan->tested[x];
+      if (plan->entries[x] && !plan->pairs[x]) return true;  // (hash tables are planned by the pairs)
+      return tested > 0 && tested >= tests_for_groups(x) * plan->groups[x];
+    }
+    u64 sets = 1;  // choose(priv, v - b) for a child of v vertices
+    for (int y : {nd.child0, nd.child1})
+      for (int j = 0; j < (int)subtree_vertices(y) - b; ++j)
+        sets = sets * (u64)(priv - j) / (u64)(j + 1);
+    return sets > cc::kJoinSets;
+  };
+  // true if join x is made group by group
+  auto by_groups = [&](int x) {
+    const NiceNode &nd = P.nodes[x];
+    return entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries && long_groups(x);
+  };
   // Introduce x (arguments a, child y) run by run, with its parent forget f when f >= 0
   // (cc_runs.cu).  *taken: 1 if it made the table of x (or of f), 0 if the entry kernels have to;
   // *total: the entries of x when an exact run has counted them here (else left alone).  Taken
@@ -819,7 +855,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       // an entry in (k - s) of k cases.  Too few a pair: nothing is listed that the entry kernels
       // would do again.  (First run of the six-cycle, Erdos-Renyi, n = 6000, 8 colourings: 8.65 ms
       // with the pairs of such nodes counted and given up, 7.57 so; 7.55 by the entry kernels alone.)
-      const u64 s = ny.bag.size() + __builtin_popcount(forgotten_below(y)), k = R->L.k;
+      const u64 s = subtree_vertices(y), k = R->L.k;
       if (most * (k - s) < cc::kRunYield * slots * k) return CC_OK;
     } else {
       slots = room(plan->runwise[x].slots);
@@ -1046,11 +1082,24 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (short_of) return CC_OK;
     a.off = off;
     a.pairs = pairs_dev + x;
-    r = timed(x, CC_K_JOIN_BUILD, 4,
-              [&] { return cc::launch_join_match(c->stream, c->dev, R->kw, a, blk); });
+    a.tested = tested_dev + x;
+    a.n_groups = groups_dev + x;
+    r = timed(x, CC_K_JOIN_BUILD, planned ? 4 : 5, [&] {
+      const int e = cc::launch_join_match(c->stream, c->dev, R->kw, a, blk);
+      return e || planned ? e : cc::launch_join_tested(c->stream, c->dev, R->kw, a);
+    });
     if (r) return r;
+    // planned runs join through hash tables after all when the groups turn out short: for those the
+    // matching pairs are counted too
+    bool want_pairs = R->learn_pairs;
+    if (!planned) {
+      u64 n_groups = 0;
+      r = read_two(c, tested_dev + x, &R->tested[x], groups_dev + x, &n_groups);
+      if (r) return r;
+      want_pairs = want_pairs || R->tested[x] < tests_for_groups(x) * n_groups;
+    }
     r = timed(x, CC_K_JOIN_COUNT, 4, [&] {
-      const int e = cc::launch_join_groups(c->stream, c->dev, R->kw, R->learn_pairs ? 2 : 0, a);
+      const int e = cc::launch_join_groups(c->stream, c->dev, R->kw, want_pairs ? 2 : 0, a);
       return e ? e : cc::launch_scan_u32(c->stream, c->dev, a.cnt, a.a.cap, off, scan, a.groups,
                                          R->d_counters + x);
     });
@@ -1063,6 +1112,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (!p) {  // (the hash table's counters start at 0)
       CUDA_OK(cudaMemsetAsync(R->d_counters + x, 0, sizeof(u64), c->stream));
       CUDA_OK(cudaMemsetAsync(pairs_dev + x, 0, sizeof(u64), c->stream));
+      CUDA_OK(cudaMemsetAsync(tested_dev + x, 0, sizeof(u64), c->stream));
+      CUDA_OK(cudaMemsetAsync(groups_dev + x, 0, sizeof(u64), c->stream));
       return CC_OK;
     }
     R->tables[x] = {p, cap, 0, true};
@@ -1104,6 +1155,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     a.index_cap = icap;
     a.next = next;
     a.pairs = pairs;
+    a.tested = tested_dev + x;
+    a.groups = groups_dev + x;
     a.err = R->d_err;
     rc = timed(x, CC_K_JOIN_BUILD, 1,
                [&] { return cc::launch_join(c->stream, c->dev, R->kw, 0, block, a); });
@@ -1526,9 +1579,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       if (rc) return rc;
       release_child(y);
     } else {  // join: group by group, or through hash tables
+      const bool able = R->L.k - (int)nd.bag.size() <= cc::kJoinBits;
+      const bool groups = able && !R->frugal && by_groups(x);
       int joined = 0;
-      if (!R->frugal && R->L.k - (int)nd.bag.size() <= cc::kJoinBits &&
-          entries(nd.child0) + entries(nd.child1) >= cc::kJoinEntries) {
+      if (groups) {
         rc = join_groups(x, &joined);
         if (rc) return rc;
       }
@@ -1540,6 +1594,12 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
           return CC_ENOMEM;
         }
         rc = join_hashed(x);
+        if (rc == CC_ENOMEM && able && !groups) {  // groups need less room than hash tables
+          for (u64 *w : {pairs_dev, tested_dev, groups_dev})
+            CUDA_OK(cudaMemsetAsync(w + x, 0, sizeof(u64), c->stream));
+          rc = join_groups(x, &joined);
+          if (!rc && !joined) rc = CC_ENOMEM;
+        }
         if (rc) return rc;
       }
       release_child(nd.child0);
@@ -1568,6 +1628,8 @@ int finish_run(Ctx *c, Run *R) {
   for (int x = 0; x < N; ++x) {
     R->sizes[x] = words[x];
     if (words[2 * N + x]) R->pairs[x] = words[2 * N + x];
+    if (words[3 * N + x]) R->tested[x] = words[3 * N + x];
+    if (words[7 * N + x]) R->groups[x] = words[7 * N + x];
     if (words[4 * N + x])
       R->runwise[x] = {words[4 * N + x], words[5 * N + x], words[6 * N + x], words[7 * N + x],
                        R->runwise[x].state};
@@ -2105,11 +2167,17 @@ void update_plan(Ctx *c, const std::vector<long long> &key, const Run *R, size_t
   const size_t N = R->sizes.size();
   plan.entries.resize(N, 0);
   plan.pairs.resize(N, 0);
+  plan.tested.resize(N, 0);
+  plan.groups.resize(N, 0);
   plan.runwise.resize(N);
   for (size_t x = 0; x < N; ++x) {
     plan.entries[x] = std::max(plan.entries[x], R->sizes[x]);
     plan.pairs[x] = std::max(plan.pairs[x], R->pairs[x]);
     if (x >= R->runwise.size()) continue;  // a run put together from parts
+    if (R->tested[x]) {  // (both of one run: their quotient counts)
+      plan.tested[x] = R->tested[x];
+      plan.groups[x] = R->groups[x];
+    }
     cc::RunSizes &p = plan.runwise[x];
     const cc::RunSizes &r = R->runwise[x];
     p = {std::max(p.slots, r.slots), std::max(p.pairs, r.pairs), std::max(p.more, r.more),
@@ -2349,6 +2417,8 @@ int replay_graph(Ctx *c, cc::GraphSet &gs, const std::vector<Run *> &Rs) {
                             cudaMemcpyDeviceToDevice, c->stream));
     R->sizes = S->sizes;
     R->pairs = S->pairs;
+    R->tested = S->tested;
+    R->groups = S->groups;
     R->runwise = S->runwise;
     R->planned = true;
     R->graphed = true;

@@ -134,7 +134,9 @@ struct JoinArgs {
   unsigned long long index_cap;
   unsigned long long *next;  // per build slot: next chained slot + 1 (0 ends a chain)
   TableDesc out;        // hashed output (mode 1)
-  unsigned long long *pairs;  // mode 0: number of matching (C', C'') pairs
+  unsigned long long *pairs;   // mode 0: number of matching (C', C'') pairs
+  unsigned long long *tested;  // mode 0: pairs looked at (the lengths of the chains walked)
+  unsigned long long *groups;  // build: mappings with their trial
   int *err;
 };
 
@@ -246,16 +248,27 @@ struct JoinGroupArgs {
   unsigned long long *groups, *first, *blo;
   unsigned *blen, *cnt;
   const unsigned long long *off;
-  unsigned long long *pairs;  // mode 2: matching pairs, which a join through hash tables plans by
+  // pairs of entries that share their group, and a's groups again (launch_join_tested)
+  unsigned long long *tested, *n_groups;
+  unsigned long long *pairs;   // mode 2: those of them that match (a join through hash tables plans by it)
   TableDesc out;     // mode 1
   int *err;
 };
 // most private colours (k - bag size) whose sums a warp keeps in shared memory
 constexpr int kJoinBits = 11;
-// fewest entries of both children together that are joined group by group.  Partial 2-trees on a
-// 2000-vertex power-law graph: 0.19 ms through hash tables against 0.7 with two sorts at 1.9
-// million entries, 1.04 against 0.6 at 4.1 million; joins of 10 000 entries 0.04 against 0.3.
+// Fewest entries of both children together that are joined group by group, and fewest pairs of entries
+// to test for a group (of the smaller child): a short group costs its warp what a long one does, and
+// short chains cost the hash tables little.  Through hash tables against by groups, in ms (pairs
+// tested a group): 0.47 and 3.3 (1; 4-cycle of two paths, 9.8 million entries), 0.27 and 0.84 (2;
+// second join of a partial 2-tree, 4.4 million), 0.97 and 1.9 (6; star of joins, 10 million), 0.95
+// and 1.6 (10; the same, one colour more), 0.39 and 0.61 (13; first join of a larger star, 3.9
+// million, whose second takes the sorted result: 6.4 and 2.5), 6.0 and 2.5 (32; first join of the
+// partial 2-tree, 22 million), 0.93 and 0.64 (72; first of the 9-vertex tree, 6.4 million), 20.7 and
+// 1.4 (720; its third, 18 million).  Few entries: 0.05 and 0.4 (0.13 million), 0.26 and 0.43 (2.1
+// million).  An exact run does not know its groups and goes by the most colour sets that a group of
+// either child can hold.
 constexpr unsigned long long kJoinEntries = 1ull << 21;
+constexpr unsigned long long kJoinTested = 16, kJoinTestedBelowJoin = 12, kJoinSets = 20;
 
 // Stable LSD radix sort of the nonempty records of `src` (n_src slots, n of them nonempty) into
 // buf_a / buf_b (n records each); *which (0 or 1) names the buffer holding the result.  hist
@@ -368,6 +381,8 @@ int prepare_join_kernels();  // once per device, as prepare_sort_kernels
 // lists a's groups and finds their ranges in b (blk: 2 * sort_grid(d) words)
 int launch_join_match(cudaStream_t s, const DevInfo &d, int kw, const JoinGroupArgs &a,
                       unsigned long long *blk);
+// adds the pairs of entries that share a group to *a.tested; *a.n_groups = *a.groups
+int launch_join_tested(cudaStream_t s, const DevInfo &d, int kw, const JoinGroupArgs &a);
 // mode 0 counts each group's results, mode 1 writes them, mode 2 is 0 and counts matching pairs
 int launch_join_groups(cudaStream_t s, const DevInfo &d, int kw, int mode, const JoinGroupArgs &a);
 int launch_root(cudaStream_t s, const DevInfo &d, int kw, const RootArgs &a);

@@ -162,6 +162,20 @@ __global__ void __launch_bounds__(256) join_match_kernel(JoinGroupArgs a) {
   }
 }
 
+// the pairs of entries that share a group (the exact run's, for the plan; in the kernel above the sum
+// would cost half of the searches in flight)
+template <typename K>
+__global__ void __launch_bounds__(256) join_tested_kernel(JoinGroupArgs a) {
+  __shared__ u64 s_red[8];
+  const u64 groups = block_run_failed(a.err) ? 0 : *a.groups, na = table_bound<K>(a.a);
+  u64 tested = 0;
+  for (u64 g = blockIdx.x * 256ull + threadIdx.x; g < groups; g += gridDim.x * 256ull)
+    tested += ((g + 1 < groups ? a.first[g + 1] : na) - a.first[g]) * a.blen[g];
+  tested = block_sum<256>(tested, s_red);
+  if (threadIdx.x == 0 && tested) atomicAdd(a.tested, tested);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.n_groups = groups;
+}
+
 // MODE 0: the number of results of every group to cnt; MODE 1: the results themselves at the
 // offsets made from those counts; MODE 2: as 0, and the matching pairs (their count costs the
 // first pass a twentieth, so they are counted once, when a plan wants them).
@@ -307,6 +321,12 @@ int launch_join_match(cudaStream_t s, const DevInfo &d, int kw, const JoinGroupA
     CC_JM(u128);
   }
 #undef CC_JM
+  return (int)cudaGetLastError();
+}
+
+int launch_join_tested(cudaStream_t s, const DevInfo &d, int kw, const JoinGroupArgs &a) {
+  if (kw == 1) join_tested_kernel<u64><<<sort_grid(d), 256, 0, s>>>(a);
+  else join_tested_kernel<u128><<<sort_grid(d), 256, 0, s>>>(a);
   return (int)cudaGetLastError();
 }
 

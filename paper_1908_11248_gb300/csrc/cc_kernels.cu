@@ -1233,11 +1233,13 @@ __device__ __forceinline__ K phi_key(K key, const KeyLayout &L) {
 
 template <typename K, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) join_build_kernel(JoinArgs a) {
+  __shared__ u64 s_red[BLOCK / 32];
   const Slot<K> *bt = reinterpret_cast<const Slot<K> *>(a.build.slots);
   Slot<K> *idx = reinterpret_cast<Slot<K> *>(a.index);
   const u64 bound = block_run_failed(a.err) ? 0 : table_bound<K>(a.build);
   const u64 icap = a.index_cap;
   bool full = false;
+  u64 groups = 0;
   for (u64 i = blockIdx.x * (u64)BLOCK + threadIdx.x; i < bound; i += (u64)gridDim.x * BLOCK) {
     K key;
     u64 c;
@@ -1248,8 +1250,12 @@ __global__ void __launch_bounds__(BLOCK) join_build_kernel(JoinArgs a) {
       full = true;
       continue;
     }
-    a.next[i] = atomicExch(&idx[h].cnt, (u64)(i + 1));
+    const u64 before = atomicExch(&idx[h].cnt, (u64)(i + 1));
+    a.next[i] = before;
+    groups += before == 0;
   }
+  groups = block_sum<BLOCK>(groups, s_red);
+  if (threadIdx.x == 0 && groups) atomicAdd(a.groups, groups);
   if (full) atomicOr(a.err, kErrOverflow);
 }
 
@@ -1263,7 +1269,7 @@ __global__ void __launch_bounds__(BLOCK) join_probe_kernel(JoinArgs a) {
   const u64 bound = block_run_failed(a.err) ? 0 : table_bound<K>(a.probe);
   const u64 icap = a.index_cap, ocap = a.out.cap;
   const K cmask = (K)((1ull << a.L.k) - 1ull);
-  u64 pairs = 0, fresh = 0;
+  u64 pairs = 0, fresh = 0, tested = 0;
   bool full = false;
   for (u64 i = blockIdx.x * (u64)BLOCK + threadIdx.x; i < bound; i += (u64)gridDim.x * BLOCK) {
     K key;
@@ -1285,6 +1291,7 @@ __global__ void __launch_bounds__(BLOCK) join_probe_kernel(JoinArgs a) {
       u64 c1;
       load_slot(bt, e - 1, k1, c1);
       const uint32_t C1 = key_mask(k1, a.L);
+      ++tested;
       if ((C1 & C2) == bagc) {
         ++pairs;
         if (MODE == 1 && !full) {
@@ -1300,6 +1307,8 @@ __global__ void __launch_bounds__(BLOCK) join_probe_kernel(JoinArgs a) {
   if (MODE == 0) {
     u64 s = block_sum<BLOCK>(pairs, s_red);
     if (threadIdx.x == 0 && s) atomicAdd(a.pairs, s);
+    s = block_sum<BLOCK>(tested, s_red);
+    if (threadIdx.x == 0 && s) atomicAdd(a.tested, s);
   } else {
     u64 f = block_sum<BLOCK>(fresh, s_red);
     if (threadIdx.x == 0 && f) atomicAdd(a.out.count, f);

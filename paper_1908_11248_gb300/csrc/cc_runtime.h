@@ -184,7 +184,8 @@ struct RunSizes {
 // Capacities learned from exact runs of one (pattern, graph, trials, colours, options): the
 // largest table sizes and join pair counts seen, per node.
 struct Plan {
-  std::vector<u64> entries, pairs;
+  // (of joins: matching pairs, pairs tested and groups of the last exact run)
+  std::vector<u64> entries, pairs, tested, groups;
   std::vector<RunSizes> runwise;  // of introduces taken run by run
   size_t peak_bytes = 0;  // largest arena use of a run beyond what it started with
   int runs = 0;
@@ -215,11 +216,12 @@ struct Run {
   int kw = 1;
   int32_t trials = 0;
   std::vector<NodeTable> tables;
-  // per node, kWords words: entries, chunk cursor, join pairs, candidates examined, RunSizes
+  // per node, kWords words: entries, chunk cursor, join pairs, candidates examined (of a join: pairs
+  // tested), RunSizes (of a join the last: groups)
   u64 *d_counters = nullptr;
   unsigned *d_exists = nullptr;
   u64 *d_count = nullptr;
-  std::vector<u64> sizes, pairs;
+  std::vector<u64> sizes, pairs, tested, groups;
   std::vector<RunSizes> runwise;
   std::vector<std::pair<const u64 *, u64>> checks;  // planned runs: device word <= capacity
   bool retained = false;

@@ -384,3 +384,18 @@ def test_hub_route_at_its_limit(ctx):
                                   oracle.colors(4 * (d + 1), 1, 3, seed=1), 3)
         launches.append(made[1][1])
     assert launches[1] - launches[0] == sum(nd[0] == cc.INTRODUCE for nd in nodes)
+
+
+@pytest.mark.parametrize("pat,n,trials,k,long", [("star", 12_000, 7, 5, False), ("A", 4000, 3, 9, True)])
+def test_join_route_by_group_length(ctx, pat, n, trials, k, long):
+    """More than 2^21 entries are joined group by group where a group has many pairs to test, and
+    through hash tables where it has few."""
+    p = star_of_joins(4) if pat == "star" else synth.pattern_A()
+    g = synth.erdos_renyi(n, 8 / n, 6) if pat == "star" else synth.barabasi_albert(n, 4, 3)
+    made, sizes, nodes = launched(ctx, g, p, oracle.colors(n, trials, k, seed=k), k)
+    joins = [x for x, nd in enumerate(nodes) if nd[0] == cc.JOIN
+             and sizes[nd[1]] + sizes[nd[2]] > 1 << 21]
+    assert joins
+    planned = made[1][0]  # only joins by groups count in planned runs
+    for x in joins:
+        assert ((x, "join_count") in planned) == long
