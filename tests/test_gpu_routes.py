@@ -389,7 +389,8 @@ def test_hub_route_at_its_limit(ctx):
 @pytest.mark.parametrize("pat,n,trials,k,long", [("star", 12_000, 7, 5, False), ("A", 4000, 3, 9, True)])
 def test_join_route_by_group_length(ctx, pat, n, trials, k, long):
     """More than 2^21 entries are joined group by group where a group has many pairs to test, and
-    through hash tables where it has few."""
+    through hash tables where it has few, exactly and planned; introduces that the join stores go run
+    by run where its groups are long."""
     p = star_of_joins(4) if pat == "star" else synth.pattern_A()
     g = synth.erdos_renyi(n, 8 / n, 6) if pat == "star" else synth.barabasi_albert(n, 4, 3)
     made, sizes, nodes = launched(ctx, g, p, oracle.colors(n, trials, k, seed=k), k)
@@ -399,3 +400,8 @@ def test_join_route_by_group_length(ctx, pat, n, trials, k, long):
     planned = made[1][0]  # only joins by groups count in planned runs
     for x in joins:
         assert ((x, "join_count") in planned) == long
+    stored = [y for x in joins for y in nodes[x][1:3] if nodes[y][0] == cc.INTRODUCE
+              and sizes[y] > 1 << 20]
+    assert stored
+    for y in stored:
+        assert planned.count((y, "intro_write")) == (4 if long else 1)
