@@ -405,3 +405,15 @@ def test_join_route_by_group_length(ctx, pat, n, trials, k, long):
     assert stored
     for y in stored:
         assert planned.count((y, "intro_write")) == (4 if long else 1)
+
+
+def test_no_chain_over_an_introduce(ctx):
+    """Two introduces over one whose table run by run comes sorted are not chained."""
+    n, trials, k = 4000, 16, 6
+    p = synth.random_partial_ktree(5, 3, 207)
+    made, sizes, nodes = launched(ctx, synth.power_law_config(n, 7.0, 2.5, 3), p,
+                                  oracle.colors(n, trials, k, seed=5), k)
+    assert [nd[0] for nd in nodes[:4]] == [cc.LEAF] + [cc.INTRODUCE] * 3 and sizes[1] > 1 << 18
+    planned = made[1][0]
+    assert planned.count((1, "intro_write")) == 4
+    assert not any(kind == "intro_chain" for _, kind in planned)
