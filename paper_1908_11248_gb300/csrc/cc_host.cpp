@@ -765,7 +765,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     if (planned) {
       const cc::RunSizes &r = plan->runwise[x];
       if (r.state != cc::Runwise::kDone || plan->entries[x] <= kHashEntries || r.slots == 0 ||
-          plan->entries[x] < cc::kRunYield * r.slots || 2 * r.more > plan->entries[x])
+          plan->entries[x] < cc::kRunYield * r.slots || 2 * r.more > plan->entries[x] ||
+          (f < 0 && r.slots < cc::kRunSlots))
         return CC_OK;
     }
     // On every way out: how far the attempt came; of one that was left nothing stays, neither a
@@ -865,7 +866,8 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       // would do again.  (First run of the six-cycle, Erdos-Renyi, n = 6000, 8 colourings: 8.65 ms
       // with the pairs of such nodes counted and given up, 7.57 so; 7.55 by the entry kernels alone.)
       const u64 s = subtree_vertices(y), k = R->L.k;
-      if (most * (k - s) < cc::kRunYield * slots * k) return CC_OK;
+      if (most * (k - s) < cc::kRunYield * slots * k || (f < 0 && slots < cc::kRunSlots))
+        return CC_OK;
     } else {
       slots = room(plan->runwise[x].slots);
     }

@@ -191,6 +191,11 @@ struct RunsArgs {
 // fewest trials for it below a forget or above a leaf, and fewest entries a pair must yield
 constexpr int kRunTrials = 8;
 constexpr unsigned long long kRunYield = 2;
+// Fewest pairs for a stored introduce: a thread a pair counts its run's entries, so few pairs of long
+// runs leave the GPU idle, and there are no entries to sort to make up for it.  Entry by entry against
+// run by run: 0.08 and 0.56 ms (6000 pairs of runs of 800 entries), 0.11 and 0.37 (9000 of 440), 0.05
+// and 0.12 (32 000 of 30; its sorted result is worth 0.5 to the join above).
+constexpr unsigned long long kRunSlots = 1ull << 14;
 
 struct RootArgs {
   KeyLayout L;

@@ -417,3 +417,15 @@ def test_no_chain_over_an_introduce(ctx):
     planned = made[1][0]
     assert planned.count((1, "intro_write")) == 4
     assert not any(kind == "intro_chain" for _, kind in planned)
+
+
+def test_few_pairs_stored_entry_by_entry(ctx):
+    """Stored introduces of few (run, candidate) pairs are not taken run by run, however many entries
+    a pair stands for."""
+    made, sizes, nodes = launched(ctx, hub_graph(500, 3), synth.pattern_B(),
+                                  oracle.colors(500, 64, 7, seed=5), 7)
+    planned = made[1][0]
+    stored = [x for x, nd in enumerate(nodes) if nd[0] == cc.INTRODUCE and sizes[x] > 1 << 18
+              and (x, "intro_write") in planned]
+    assert stored
+    assert all(planned.count((x, "intro_write")) == 1 for x in stored)
