@@ -429,3 +429,14 @@ def test_few_pairs_stored_entry_by_entry(ctx):
               and (x, "intro_write") in planned]
     assert stored
     assert all(planned.count((x, "intro_write")) == 1 for x in stored)
+
+
+def test_small_first_runs_try_nothing(ctx):
+    """An exact run that expects few entries counts them once: no runs or pairs are listed first."""
+    pat = (4, np.array([(0, 1), (1, 2), (2, 3), (0, 3)], np.int32),
+           ([[0, 2], [0, 1, 2], [0, 2, 3]], [-1, 0, 0]))
+    made, sizes, nodes = launched(ctx, hub_graph(171, 3), pat, oracle.colors(171, 9, 4, seed=5), 4)
+    exact = made[0][0]
+    for x, nd in enumerate(nodes):
+        if nd[0] == cc.INTRODUCE:
+            assert sizes[x] < 1 << 17 and exact.count((x, "intro_count")) == 1
