@@ -705,10 +705,12 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     return CC_OK;
   };
   // pairs of entries to test for a group from which join x is made group by group (kJoinTested: fewer
-  // if a join above takes the sorted result)
+  // among joins, of which one hands the next its result in order)
   auto tests_for_groups = [&](int x) {
-    const int up = P.nodes[x].parent;
-    return up >= 0 && P.nodes[up].type == 3 ? cc::kJoinTestedBelowJoin : cc::kJoinTested;
+    const NiceNode &nd = P.nodes[x];
+    bool among = false;
+    for (int y : {nd.parent, nd.child0, nd.child1}) among = among || (y >= 0 && P.nodes[y].type == 3);
+    return among ? cc::kJoinTestedAmong : cc::kJoinTested;
   };
   // true if join x's groups are long enough to be joined one by one: by what the plan knows of them,
   // else by the most colour sets that a group of either child can hold

@@ -273,7 +273,7 @@ constexpr int kJoinBits = 11;
 // million).  An exact run does not know its groups and goes by the most colour sets that a group of
 // either child can hold.
 constexpr unsigned long long kJoinEntries = 1ull << 21;
-constexpr unsigned long long kJoinTested = 16, kJoinTestedBelowJoin = 12, kJoinSets = 20;
+constexpr unsigned long long kJoinTested = 16, kJoinTestedAmong = 8, kJoinSets = 20;
 
 // Stable LSD radix sort of the nonempty records of `src` (n_src slots, n of them nonempty) into
 // buf_a / buf_b (n records each); *which (0 or 1) names the buffer holding the result.  hist
