@@ -843,7 +843,7 @@ __global__ void __launch_bounds__(256, CHAIN ? 3 : 4) intro_group_warp_kernel(In
   // the next window's records are loaded while the current one is processed
   K nkey = 0;
   u64 nc_ = 0;
-  const u64 stretch = CHAIN ? 8 : a.stretch, w0 = wid * stretch;
+  const u64 stretch = a.stretch, w0 = wid * stretch;
   if (w0 < nwin && w0 * width + mylane < bound) load_slot(in, w0 * width + mylane, nkey, nc_);
   for (u64 win = w0, follow; win < nwin; win = follow) {
     const K key = nkey;
