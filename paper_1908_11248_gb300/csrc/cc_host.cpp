@@ -765,8 +765,10 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
         !long_groups(nd.parent))
       return CC_OK;
     if (planned) {
+      const bool hubs = c->max_deg > cc::kHeavyList;
       const cc::RunSizes &r = plan->runwise[x];
-      if (r.state != cc::Runwise::kDone || plan->entries[x] <= kHashEntries || r.slots == 0 ||
+      if (r.state != cc::Runwise::kDone || r.slots == 0 ||
+          plan->entries[x] <= (hubs ? kHashEntries : f < 0 ? cc::kRunStored : cc::kRunEntries) ||
           plan->entries[x] < cc::kRunYield * r.slots || 2 * r.more > plan->entries[x] ||
           (f < 0 && r.slots < cc::kRunSlots))
         return CC_OK;

@@ -191,6 +191,12 @@ struct RunsArgs {
 // fewest trials for it below a forget or above a leaf, and fewest entries a pair must yield
 constexpr int kRunTrials = 8;
 constexpr unsigned long long kRunYield = 2;
+// Fewest entries of planned ones, below a forget and stored, on a graph without hubs (kHeavyList): three
+// dozen launches against one (4-cycle of two paths, Erdos-Renyi, 16 colourings, 0.7 and 1.06 million
+// entries: 0.53 and 0.57 ms with every introduce entry by entry, 0.84 and 0.86 run by run); a stored
+// one is mostly worth what it gives the next.  With hubs those of more than 2^18 entries, as a pair of a
+// hub's run stands for many (2x4 grid, n = 4999, 13 colourings: 3.88 ms, 4.33 with these lines).
+constexpr unsigned long long kRunEntries = 1ull << 21, kRunStored = 1ull << 19;
 // Fewest pairs for a stored introduce: a thread a pair counts its run's entries, so few pairs of long
 // runs leave the GPU idle, and there are no entries to sort to make up for it.  Entry by entry against
 // run by run: 0.08 and 0.56 ms (6000 pairs of runs of 800 entries), 0.11 and 0.37 (9000 of 440), 0.05

@@ -409,7 +409,7 @@ def test_join_route_by_group_length(ctx, pat, n, trials, k, long):
 
 def test_no_chain_over_an_introduce(ctx):
     """Two introduces over one whose table run by run comes sorted are not chained."""
-    n, trials, k = 4000, 16, 6
+    n, trials, k = 4000, 28, 6
     p = synth.random_partial_ktree(5, 3, 207)
     made, sizes, nodes = launched(ctx, synth.power_law_config(n, 7.0, 2.5, 3), p,
                                   oracle.colors(n, trials, k, seed=5), k)
