@@ -251,7 +251,7 @@ KERNEL_GROUPS = {
     "reduce_write_kernel": "forget", "forget_kernel": "forget", "part_hist_kernel": "forget",
     "part_cursor_kernel": "forget", "part_split_kernel": "forget",
     "part_local_kernel": "forget",
-    "join_build_kernel": "join", "join_probe_kernel": "join",
+    "join_build_kernel": "join", "join_sample_kernel": "join", "join_probe_kernel": "join",
     "join_heads_count_kernel": "join", "join_heads_scan_kernel": "join",
     "join_heads_list_kernel": "join", "join_match_kernel": "join", "join_tested_kernel": "join",
     "join_group_kernel": "join",

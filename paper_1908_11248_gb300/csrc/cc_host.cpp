@@ -1030,6 +1030,35 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     return CC_OK;
   };
 
+  // true if the groups of the smaller child of join x hold less than kJoinMean entries on average, by a
+  // sample (exact runs; false if there is no room for it)
+  auto short_groups = [&](int x, bool *is) -> int {
+    *is = false;
+    int y = P.nodes[x].child0, z = P.nodes[x].child1;
+    if (entries(y) > entries(z)) std::swap(y, z);
+    cc::JoinArgs a{};
+    a.G = G;
+    a.L = R->L;
+    a.build = desc(y);
+    a.index_cap = hash_cap(std::max<u64>(1024, entries(y) / 8), lf);
+    const size_t bytes = a.index_cap * cc::index_slot_bytes(R->kw);
+    Held held{A, {A.alloc(bytes)}};
+    a.index = held.p[0];
+    if (!a.index) return CC_OK;
+    a.tested = tested_dev + x;
+    a.groups = groups_dev + x;
+    a.err = R->d_err;
+    CUDA_OK(cudaMemsetAsync(a.index, 0, bytes, c->stream));
+    int r = timed(x, CC_K_JOIN_BUILD, 1,
+                  [&] { return cc::launch_join(c->stream, c->dev, R->kw, -1, block, a); });
+    u64 members = 0, groups = 0;
+    if (!r) r = read_two(c, a.tested, &members, a.groups, &groups);
+    if (r) return r;
+    *is = members < cc::kJoinMean * groups;
+    CUDA_OK(cudaMemsetAsync(a.tested, 0, sizeof(u64), c->stream));
+    CUDA_OK(cudaMemsetAsync(a.groups, 0, sizeof(u64), c->stream));
+    return CC_OK;
+  };
   // Join x of two children sorted by (mapping, trial), group by group (cc_join.cu).  *taken: 0 if
   // its scratch or its result does not fit, after which the children are what they were or sorted.
   auto join_groups = [&](int x, int *taken) -> int {
@@ -1606,7 +1635,13 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
       release_child(y);
     } else {  // join: group by group, or through hash tables
       const bool able = R->L.k - (int)nd.bag.size() <= cc::kJoinBits;
-      const bool groups = able && !R->frugal && by_groups(x);
+      bool groups = able && !R->frugal && by_groups(x);
+      if (groups && !planned) {
+        bool brief = false;
+        rc = short_groups(x, &brief);
+        if (rc) return rc;
+        groups = !brief;
+      }
       int joined = 0;
       if (groups) {
         rc = join_groups(x, &joined);

@@ -277,9 +277,11 @@ constexpr int kJoinBits = 11;
 // partial 2-tree, 22 million), 0.93 and 0.64 (72; first of the 9-vertex tree, 6.4 million), 20.7 and
 // 1.4 (720; its third, 18 million).  Few entries: 0.05 and 0.4 (0.13 million), 0.26 and 0.43 (2.1
 // million).  An exact run does not know its groups and goes by the most colour sets that a group of
-// either child can hold.
+// either child can hold, and by the mean of a sample of the smaller child's (first run of a 9-vertex
+// tree of six branches, 146 million entries a child, 1.02 a group: 90 ms, 173 by groups).
 constexpr unsigned long long kJoinEntries = 1ull << 21;
-constexpr unsigned long long kJoinTested = 16, kJoinTestedAmong = 8, kJoinSets = 20;
+constexpr unsigned long long kJoinTested = 16, kJoinTestedAmong = 8, kJoinSets = 20,
+                             kJoinMean = 2;
 
 // Stable LSD radix sort of the nonempty records of `src` (n_src slots, n of them nonempty) into
 // buf_a / buf_b (n records each); *which (0 or 1) names the buffer holding the result.  hist
@@ -376,7 +378,7 @@ int launch_intro_group_warp(cudaStream_t s, const DevInfo &d, int kw, int mode,
                             const IntroArgs &a);
 int launch_forget(cudaStream_t s, const DevInfo &d, int kw, int block, const ForgetArgs &a);
 int launch_join(cudaStream_t s, const DevInfo &d, int kw, int phase, int block,
-                const JoinArgs &a);  // phase 0 build, 1 count pairs, 2 write
+                const JoinArgs &a);  // phase 0 build, 1 count pairs, 2 write; -1 sample
 int launch_runs_colours(cudaStream_t s, const DevInfo &d, const uint8_t *colors, int n, int T,
                         uint8_t *colT);
 // runs of the child (blk: 2 * sort_grid(d) words) and their candidate counts

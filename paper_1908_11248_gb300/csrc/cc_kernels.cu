@@ -1259,6 +1259,33 @@ __global__ void __launch_bounds__(BLOCK) join_build_kernel(JoinArgs a) {
   if (full) atomicOr(a.err, kErrOverflow);
 }
 
+// A sixteenth of the build table's groups (by a hash of mapping and trial, all entries of each): how many
+// to *a.groups and their entries to *a.tested.
+template <typename K, int BLOCK>
+__global__ void __launch_bounds__(BLOCK) join_sample_kernel(JoinArgs a) {
+  __shared__ u64 s_red[BLOCK / 32];
+  const Slot<K> *bt = reinterpret_cast<const Slot<K> *>(a.build.slots);
+  Slot<K> *idx = reinterpret_cast<Slot<K> *>(a.index);
+  const u64 bound = block_run_failed(a.err) ? 0 : table_bound<K>(a.build);
+  u64 groups = 0, members = 0;
+  for (u64 i = blockIdx.x * (u64)BLOCK + threadIdx.x; i < bound; i += (u64)gridDim.x * BLOCK) {
+    K key;
+    u64 c;
+    load_slot(bt, i, key, c);
+    if (key == 0) continue;
+    const K g = phi_key(key, a.L);
+    if (key_hash(g) & 15u) continue;
+    const long long h = hash_claim(idx, a.index_cap, g);
+    if (h < 0) continue;  // (a full sample says less, no more)
+    groups += atomicExch(&idx[h].cnt, 1ull) == 0;
+    ++members;
+  }
+  groups = block_sum<BLOCK>(groups, s_red);
+  if (threadIdx.x == 0 && groups) atomicAdd(a.groups, groups);
+  members = block_sum<BLOCK>(members, s_red);
+  if (threadIdx.x == 0 && members) atomicAdd(a.tested, members);
+}
+
 template <typename K, int MODE, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) join_probe_kernel(JoinArgs a) {
   __shared__ u64 s_red[BLOCK / 32];
@@ -1535,7 +1562,10 @@ int launch_join(cudaStream_t s, const DevInfo &d, int kw, int phase, int block,
                 const JoinArgs &a) {
   (void)block;
   int grid = grid_for(d, 256);
-  if (phase == 0) {
+  if (phase < 0) {
+    if (kw == 1) join_sample_kernel<u64, 256><<<grid, 256, 0, s>>>(a);
+    else join_sample_kernel<u128, 256><<<grid, 256, 0, s>>>(a);
+  } else if (phase == 0) {
     if (kw == 1) join_build_kernel<u64, 256><<<grid, 256, 0, s>>>(a);
     else join_build_kernel<u128, 256><<<grid, 256, 0, s>>>(a);
   } else if (phase == 1) {

@@ -440,3 +440,12 @@ def test_small_first_runs_try_nothing(ctx):
     for x, nd in enumerate(nodes):
         if nd[0] == cc.INTRODUCE:
             assert sizes[x] < 1 << 17 and exact.count((x, "intro_count")) == 1
+
+
+@pytest.mark.parametrize("n,deg", [(1100, 37.0), (60_000, 5.0)])
+def test_join_by_sampled_groups(ctx, n, deg):
+    """Eight colours for the 4-cycle of two paths: a group could hold many colour sets; an exact run
+    samples whether it does (dense graph) or not (sparse)."""
+    pat = (4, np.array([(0, 1), (1, 2), (2, 3), (0, 3)], np.int32),
+           ([[0, 2], [0, 1, 2], [0, 2, 3]], [-1, 0, 0]))
+    check_tables(ctx, synth.erdos_renyi(n, deg / n, 8), pat, oracle.colors(n, 2, 8, seed=8), 8)
