@@ -1208,7 +1208,7 @@ int run_nodes(Ctx *c, Run *R, const Pattern &P, const cc::Coloring &col, const c
     a.next = next;
     a.pairs = pairs;
     a.tested = tested_dev + x;
-    a.groups = groups_dev + x;
+    a.groups = planned ? nullptr : groups_dev + x;
     a.err = R->d_err;
     rc = timed(x, CC_K_JOIN_BUILD, 1,
                [&] { return cc::launch_join(c->stream, c->dev, R->kw, 0, block, a); });

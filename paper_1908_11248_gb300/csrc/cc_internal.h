@@ -136,7 +136,7 @@ struct JoinArgs {
   TableDesc out;        // hashed output (mode 1)
   unsigned long long *pairs;   // mode 0: number of matching (C', C'') pairs
   unsigned long long *tested;  // mode 0: pairs looked at (the lengths of the chains walked)
-  unsigned long long *groups;  // build: mappings with their trial
+  unsigned long long *groups;  // build: mappings with their trial (null: not counted)
   int *err;
 };
 

@@ -1254,8 +1254,10 @@ __global__ void __launch_bounds__(BLOCK) join_build_kernel(JoinArgs a) {
     a.next[i] = before;
     groups += before == 0;
   }
-  groups = block_sum<BLOCK>(groups, s_red);
-  if (threadIdx.x == 0 && groups) atomicAdd(a.groups, groups);
+  if (a.groups) {
+    groups = block_sum<BLOCK>(groups, s_red);
+    if (threadIdx.x == 0 && groups) atomicAdd(a.groups, groups);
+  }
   if (full) atomicOr(a.err, kErrOverflow);
 }
 
